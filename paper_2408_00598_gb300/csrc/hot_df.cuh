@@ -7,7 +7,9 @@
 // rounding error of hi * hi from a fused multiply-add in place of Dekker's
 // splitting.  FP64 arithmetic runs at a small fraction of the FP32
 // rate on GB300, so sums and comparisons that must be accurate to FP64 level
-// use these pairs on the FP32 pipe.
+// use these pairs on the FP32 pipe.  Every operation names its rounding
+// (__fadd_rn, __fmul_rn): none can be contracted into a fused multiply-add, so
+// two kernels that form the same sum in the same order get the same bits.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -18,11 +20,11 @@ struct DF {
     float hi, lo;
 };
 __device__ __forceinline__ DF df_add(DF a, float b) {
-    const float s = a.hi + b;
-    const float bb = s - a.hi;
-    const float e = ((a.hi - (s - bb)) + (b - bb)) + a.lo;
-    const float h = s + e;
-    return DF{h, e - (h - s)};
+    const float s = __fadd_rn(a.hi, b);
+    const float bb = __fsub_rn(s, a.hi);
+    const float e = __fadd_rn(__fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, bb)), __fsub_rn(b, bb)), a.lo);
+    const float h = __fadd_rn(s, e);
+    return DF{h, __fsub_rn(e, __fsub_rn(h, s))};
 }
 __device__ __forceinline__ DF df_add(DF a, DF b) {
     DF r = df_add(a, b.hi);
@@ -40,19 +42,19 @@ __device__ __forceinline__ DF df_sub(DF a, DF b) { return df_add(a, df_neg(b)); 
 __device__ __forceinline__ float df_f(DF a) { return a.hi + a.lo; }
 // products: the error of hi*hi is exact by fma; the cross terms are FP32
 __device__ __forceinline__ DF df_mul(DF a, DF b) {
-    const float p = a.hi * b.hi;
+    const float p = __fmul_rn(a.hi, b.hi);
     float e = fmaf(a.hi, b.hi, -p);
     e = fmaf(a.hi, b.lo, e);
     e = fmaf(a.lo, b.hi, e);
-    const float h = p + e;
-    return DF{h, e - (h - p)};
+    const float h = __fadd_rn(p, e);
+    return DF{h, __fsub_rn(e, __fsub_rn(h, p))};
 }
 __device__ __forceinline__ DF df_mul(DF a, float b) {
-    const float p = a.hi * b;
+    const float p = __fmul_rn(a.hi, b);
     float e = fmaf(a.hi, b, -p);
     e = fmaf(a.lo, b, e);
-    const float h = p + e;
-    return DF{h, e - (h - p)};
+    const float h = __fadd_rn(p, e);
+    return DF{h, __fsub_rn(e, __fsub_rn(h, p))};
 }
 __device__ __forceinline__ DF df_shfl_down(DF a, int o) {
     return DF{__shfl_down_sync(0xffffffffu, a.hi, o), __shfl_down_sync(0xffffffffu, a.lo, o)};

@@ -117,6 +117,65 @@ int validate_pair(const double* mu, const double* nu, int m, int n, int space, i
     return HOT_OK;
 }
 
+constexpr size_t kGroupStateBytes = (size_t)120 << 20;   // u and one delta
+// k_group32 or the chain of kernels: the group kernel holds one column per
+// thread and one round of slab sums (sides up to 256).
+static int group_rule(const Inst& I) {
+    return !I.fp64 && std::max(I.m, I.n) <= kMaxGroupSide && I.big_bytes / 5 * 2 <= kGroupStateBytes ? 1 : 0;
+}
+
+// Groups of CTAs for one launch of k_group32.  An iteration of an instance
+// costs its CTAs two waits plus their tiles one after the other; the plan
+// takes the smallest time in which every instance fits into the grid: large
+// ones get as many CTAs as they need, small ones share a CTA (group size 1).
+GroupPlan plan_groups(const std::vector<int>& inst, const std::vector<int>& tiles, const std::vector<int>& elems,
+                      int grid) {
+    GroupPlan P;
+    const int n = (int)inst.size();
+    const double wait = 4.0, self = 1.5;                      // microseconds: two waits and the stage; the stage alone
+    auto tile_us = [&](int q) { return 0.9 + elems[q] * 0.00015; };
+    std::vector<int> order(n);
+    for (int q = 0; q < n; ++q) order[q] = q;
+    std::stable_sort(order.begin(), order.end(),
+                     [&](int a, int b) { return tiles[a] * tile_us(a) > tiles[b] * tile_us(b); });
+    std::vector<std::vector<int4>> cta;
+    auto build = [&](double tau, bool write) {
+        int used = 0;
+        double room = -1.0;                                   // of the shared CTA being filled
+        for (int q : order) {
+            const double alone = self + tiles[q] * tile_us(q);
+            if (alone > tau) {
+                const int per = std::max(1, (int)((tau - wait) / tile_us(q)));
+                int G = (tiles[q] + per - 1) / per;
+                G = std::min(G, std::min(kMaxGroup, grid));
+                if (write)
+                    for (int r = 0; r < G; ++r) cta.push_back({make_int4(inst[q], r, G, 0)});
+                used += G;
+            } else {
+                if (room < alone) {
+                    ++used;
+                    room = tau;
+                    if (write) cta.emplace_back();
+                }
+                room -= alone;
+                if (write) cta.back().push_back(make_int4(inst[q], 0, 1, 0));
+            }
+            if (used > grid) return false;
+        }
+        return true;
+    };
+    // shared CTAs come after the large ones in `order`, so the last one is open
+    double tau = wait + 1.0;
+    while (!build(tau, false)) tau *= 1.08;
+    build(tau, true);
+    P.start.assign(grid + 1, 0);
+    for (int c = 0; c < grid; ++c) {
+        if (c < (int)cta.size()) P.entries.insert(P.entries.end(), cta[c].begin(), cta[c].end());
+        P.start[c + 1] = (int)P.entries.size();
+    }
+    return P;
+}
+
 // --------------------------------------------------------------- instances --
 
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -147,6 +206,7 @@ int inst_create(const PairHost& p, int fp64, const hot_config& cfg, double tol, 
     const size_t V = MN * (size_t)(mp + np);
     const size_t es = fp64 ? 8 : 4;
     I->big_bytes = 5 * align256(V * es);
+    I->group_ok = group_rule(*I);
 
     // small-buffer layout; per-slab arrays hold 2mn entries (one per slab row:
     // n slabs of m rows, m slabs of n rows), column partials one per band
@@ -186,6 +246,10 @@ int inst_create(const PairHost& p, int fp64, const hot_config& cfg, double tol, 
     const size_t o_vec2 = take(vec2_entries(m, n) * F2);
     const size_t o_dab2 = take(4 * MN * F2);
     const size_t o_stg2 = take(4 * (size_t)L * F2);
+    const size_t o_rs2b = take(2 * MN * F2);
+    const size_t o_cs32b = fp64 ? 0 : take(CP * 4);
+    const size_t o_tp = fp64 ? 0 : take((size_t)NS * sizeof(float4));
+    const size_t o_gcount = fp64 ? 0 : take(sizeof(unsigned int));
     const size_t o_vcnt = take(sizeof(unsigned int));
     const size_t o_zero_end = off;                 // everything above starts at 0
     const size_t o_mu1f = take(MN * F2);
@@ -332,6 +396,10 @@ int inst_create(const PairHost& p, int fp64, const hot_config& cfg, double tol, 
     d.dab2 = fp64 ? nullptr : (float2*)(sm + o_dab2);
     d.stg2 = fp64 ? nullptr : (float2*)(sm + o_stg2);
     d.vcount = (unsigned int*)(sm + o_vcnt);
+    d.rs2b = fp64 ? nullptr : (float2*)(sm + o_rs2b);
+    d.cs32b = fp64 ? nullptr : (float*)(sm + o_cs32b);
+    d.tp = fp64 ? nullptr : (float4*)(sm + o_tp);
+    d.gcount = fp64 ? nullptr : (unsigned int*)(sm + o_gcount);
     d.mu1f = fp64 ? nullptr : (float2*)(sm + o_mu1f);
     d.mu2f = fp64 ? nullptr : (float2*)(sm + o_mu2f);
     d.cm2 = fp64 ? nullptr : (float2*)(sm + o_cm2);
@@ -434,6 +502,10 @@ Batch::~Batch() {
     cudaFree(d_pre);
     cudaFree(d_running);
     cudaFree(d_st);
+    cudaFree(d_gstart);
+    cudaFree(d_gent);
+    cudaFreeHost(h_gstart);
+    cudaFreeHost(h_gent);
     cudaFreeHost(h_work);
     cudaFreeHost(h_inst);
     cudaFreeHost(h_pre);
@@ -452,8 +524,7 @@ void Batch::drop_graphs() {
             cudaGraphExecDestroy(tgraph[p]);
             tgraph[p] = nullptr;
         }
-    single = -1;
-    pad_captured = -1;
+    captured = -1;
 }
 
 int Batch::reserve(int n) {
@@ -465,6 +536,10 @@ int Batch::reserve(int n) {
     cudaFree(d_pre);
     cudaFree(d_running);
     cudaFree(d_st);
+    cudaFree(d_gstart);
+    cudaFree(d_gent);
+    cudaFreeHost(h_gstart);
+    cudaFreeHost(h_gent);
     cudaFreeHost(h_work);
     cudaFreeHost(h_inst);
     cudaFreeHost(h_pre);
@@ -473,31 +548,33 @@ int Batch::reserve(int n) {
     cudaFreeHost(h_stb);
     h_stb = nullptr;
     d_work = nullptr;
+    d_gstart = nullptr;
+    d_gent = nullptr;
+    h_gstart = nullptr;
+    h_gent = nullptr;
+    ggrid = fp64 ? 0 : group_grid();
+    HOT_CK(cudaMalloc(&d_gstart, sizeof(int) * (ggrid + 1)));
+    HOT_CK(cudaMalloc(&d_gent, sizeof(int4) * (ggrid + ncap)));
+    HOT_CK(cudaMallocHost(&h_gstart, sizeof(int) * (ggrid + 1)));
+    HOT_CK(cudaMallocHost(&h_gent, sizeof(int4) * (ggrid + ncap)));
     HOT_CK(cudaMalloc(&d_work, sizeof(WorkDev)));
     HOT_CK(cudaMalloc(&d_inst, sizeof(HotInst) * ncap));
     HOT_CK(cudaMalloc(&d_pre, sizeof(int) * kPreTables * (ncap + 1)));
-    HOT_CK(cudaMalloc(&d_running, sizeof(int)));
+    HOT_CK(cudaMalloc(&d_running, sizeof(int) * 2));
     HOT_CK(cudaMalloc(&d_st, sizeof(int) * ncap));
     HOT_CK(cudaMallocHost(&h_st, sizeof(int) * ncap));
     HOT_CK(cudaMallocHost(&h_stb, sizeof(int) * 2 * ncap));
     HOT_CK(cudaMallocHost(&h_work, sizeof(WorkDev)));
     HOT_CK(cudaMallocHost(&h_inst, sizeof(HotInst) * ncap));
     HOT_CK(cudaMallocHost(&h_pre, sizeof(int) * kPreTables * (ncap + 1)));
-    HOT_CK(cudaMallocHost(&h_running, sizeof(int) * 4));
+    HOT_CK(cudaMallocHost(&h_running, sizeof(int) * 6));
     cap = ncap;
     return HOT_OK;
 }
 
-int Batch::set_instances(const std::vector<Inst*>& v, cudaStream_t st) {
+int Batch::set_instances(const std::vector<Inst*>& v, cudaStream_t st, bool group) {
     int rc = reserve((int)v.size());
     if (rc != HOT_OK) return rc;
-    // a single instance and a batch of several run different Prop. 3 kernels
-    // (launch_solve_kernels), and padded slab rows a sweep variant of their
-    // own: a change of either needs new graphs
-    pad = 0;
-    for (const Inst* I : v) pad |= (I->m % 4 != 0) || (I->n % 4 != 0) || I->desc.coord_real;
-    if ((single >= 0 && single != (v.size() == 1 ? 1 : 0)) || (pad_captured >= 0 && pad_captured != pad))
-        drop_graphs();
     // the pinned staging is rewritten here: wait for earlier copies out of it
     HOT_CK(cudaStreamSynchronize(st));
     const int n = (int)v.size();
@@ -506,20 +583,49 @@ int Batch::set_instances(const std::vector<Inst*>& v, cudaStream_t st) {
     int* pv = h_pre + 2 * (cap + 1);
     int* pk = h_pre + 3 * (cap + 1);
     int* pa = h_pre + 4 * (cap + 1);
-    pt[0] = ps[0] = pv[0] = pk[0] = pa[0] = 0;
+    int* pw = h_pre + 5 * (cap + 1);
+    pt[0] = ps[0] = pv[0] = pk[0] = pa[0] = pw[0] = 0;
     int running = 0;
-    size_t swept = 0;                 // bytes one sweep streams: u, d read, d written
+    size_t swept = 0;                 // bytes one sweep of the chain streams: u, d read, d written
+    n_group = n_chain = 0;
+    pad = gpad = 0;
+    // many tiles per CTA hide the chain's launches, and its sweep has more
+    // CTAs per SM: beyond a few tiles per CTA the chain is the faster one
+    long long gtiles = 0;
+    for (const Inst* I : v)
+        if (I->group_ok && I->ctl_host.status == ST_RUNNING) gtiles += (long long)I->n * I->nb1 + (long long)I->m * I->nb2;
+    if (gtiles > group_tiles()) group = false;
+    std::vector<int> gi, gt, ge;      // grouped instances: index, tiles, elements of a tile
     for (int i = 0; i < n; ++i) {
         h_inst[i] = v[i]->desc;
-        swept += 3 * (v[i]->big_bytes / 5);
+        const int g = group && ggrid > 0 && v[i]->group_ok ? 1 : 0;
+        h_inst[i].grp = g;
         const int m = v[i]->m, nn = v[i]->n;
-        pt[i + 1] = pt[i] + nn * v[i]->nb1 + m * v[i]->nb2;
+        const int tiles = nn * v[i]->nb1 + m * v[i]->nb2;
+        const int odd = (m % 4 != 0) || (nn % 4 != 0) || v[i]->desc.coord_real;
+        if (g) {
+            ++n_group;
+            gpad |= odd;
+            if (v[i]->ctl_host.status == ST_RUNNING) {
+                gi.push_back(i);
+                gt.push_back(tiles);
+                ge.push_back((int)(v[i]->big_bytes / 20 / tiles));
+            }
+        } else {
+            ++n_chain;
+            pad |= odd;
+            swept += 3 * (v[i]->big_bytes / 5);
+        }
+        pt[i + 1] = pt[i] + tiles;
+        pw[i + 1] = pw[i] + (g ? 0 : tiles);
         ps[i + 1] = ps[i] + m + nn;
-        pv[i + 1] = pv[i] + (v[i]->fp64 ? 2 * (m + nn) : vec32_items(m, nn));
-        pk[i + 1] = pk[i] + v[i]->n_k1;
-        pa[i + 1] = pa[i] + v[i]->desc.n_achunk;
+        pv[i + 1] = pv[i] + (g ? 0 : v[i]->fp64 ? 2 * (m + nn) : vec32_items(m, nn));
+        pk[i + 1] = pk[i] + v[i]->n_k1 + (g ? v[i]->desc.n_achunk : 0);
+        pa[i + 1] = pa[i] + (g ? 0 : v[i]->desc.n_achunk);
         if (v[i]->ctl_host.status == ST_RUNNING) ++running;
     }
+    // the kernels of a block, and their variants, depend on the mix: a change needs new graphs
+    if (captured >= 0 && captured != shape()) drop_graphs();
     // a state larger than L2: alternate the sweep's tile order, so that each
     // sweep starts on the tiles the previous one touched last (still in L2);
     // a state that fits gains nothing from it
@@ -533,30 +639,56 @@ int Batch::set_instances(const std::vector<Inst*>& v, cudaStream_t st) {
     h_work->pre_vec = d_pre + 2 * (cap + 1);
     h_work->pre_k1 = d_pre + 3 * (cap + 1);
     h_work->pre_achunk = d_pre + 4 * (cap + 1);
+    h_work->pre_swp = d_pre + 5 * (cap + 1);
+    h_work->gstart = d_gstart;
+    h_work->gent = d_gent;
     h_work->n_running = d_running;
+    h_work->err = d_running + 1;
     h_work->st_out = d_st;
     for (int i = 0; i < n; ++i) h_st[i] = v[i]->ctl_host.status;
     h_running[0] = running;
+    h_running[1] = 0;
+    if (n_group > 0) {
+        const GroupPlan gp = plan_groups(gi, gt, ge, ggrid);
+        std::copy(gp.start.begin(), gp.start.end(), h_gstart);
+        std::copy(gp.entries.begin(), gp.entries.end(), h_gent);
+        HOT_CK(cudaMemcpyAsync(d_gstart, h_gstart, sizeof(int) * gp.start.size(), cudaMemcpyHostToDevice, st));
+        if (!gp.entries.empty())
+            HOT_CK(cudaMemcpyAsync(d_gent, h_gent, sizeof(int4) * gp.entries.size(), cudaMemcpyHostToDevice, st));
+    }
     if (n > 0) HOT_CK(cudaMemcpyAsync(d_inst, h_inst, sizeof(HotInst) * n, cudaMemcpyHostToDevice, st));
     HOT_CK(cudaMemcpyAsync(d_pre, h_pre, sizeof(int) * kPreTables * (cap + 1), cudaMemcpyHostToDevice, st));
     HOT_CK(cudaMemcpyAsync(d_work, h_work, sizeof(WorkDev), cudaMemcpyHostToDevice, st));
-    HOT_CK(cudaMemcpyAsync(d_running, h_running, sizeof(int), cudaMemcpyHostToDevice, st));
+    HOT_CK(cudaMemcpyAsync(d_running, h_running, sizeof(int) * 2, cudaMemcpyHostToDevice, st));
     if (n > 0) HOT_CK(cudaMemcpyAsync(d_st, h_st, sizeof(int) * n, cudaMemcpyHostToDevice, st));
     ninst = n;
     return HOT_OK;
+}
+
+int Batch::launches() const {
+    return (n_group > 0 ? 1 : 0) + (n_chain > 0 ? launches_per_block(fp64, K, n_chain == 1) : 0) + kLaunchesBlockEnd;
+}
+
+// The K iterations of a block: k_group32 for the grouped instances, the chain
+// of kernels for the others; with ev, an event pair around the sweep of
+// iteration timed_iter().
+void Batch::launch_iterations(cudaStream_t st, cudaEvent_t* ev) const {
+    if (n_group > 0) launch_group(d_work, ggrid, K, gpad != 0, st);
+    if (n_chain == 0) return;
+    for (int j = 0; j < K; ++j) {
+        launch_solve_kernels(d_work, ld, fp64, j, j == K - 1, n_chain == 1, st);
+        const bool t = ev && j == timed_iter() && j < K - 1;
+        if (t) cudaEventRecordWithFlags(ev[0], st, cudaEventRecordExternal);
+        launch_sweep(d_work, ld, fp64, j, j == K - 1, pad != 0, st);
+        if (t) cudaEventRecordWithFlags(ev[1], st, cudaEventRecordExternal);
+    }
 }
 
 // One check block (K iterations plus the block end) captured into *out; with
 // ev, an event pair recorded around the sweep of iteration timed_iter().
 int Batch::capture(cudaGraphExec_t* out, cudaEvent_t* ev) {
     HOT_CK(cudaStreamBeginCapture(cap_stream, cudaStreamCaptureModeThreadLocal));
-    for (int j = 0; j < K; ++j) {
-        launch_solve_kernels(d_work, ld, fp64, j, j == K - 1, ninst == 1, cap_stream);
-        const bool t = ev && j == timed_iter() && j < K - 1;
-        if (t) cudaEventRecordWithFlags(ev[0], cap_stream, cudaEventRecordExternal);
-        launch_sweep(d_work, ld, fp64, j, j == K - 1, pad != 0, cap_stream);
-        if (t) cudaEventRecordWithFlags(ev[1], cap_stream, cudaEventRecordExternal);
-    }
+    launch_iterations(cap_stream, ev);
     launch_block_end(d_work, ld, fp64, K, a1, a2, a3, cap_stream);
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamEndCapture(cap_stream, &g);
@@ -579,8 +711,7 @@ int Batch::ensure_graph(int want_timing) {
     if (timing ? (tgraph[0] && tgraph[1]) : graph != nullptr) return HOT_OK;
     if (!cap_stream) HOT_CK(cudaStreamCreateWithFlags(&cap_stream, cudaStreamNonBlocking));
     ld = make_launch_dims(device, fp64);
-    single = ninst == 1 ? 1 : 0;
-    pad_captured = pad;
+    captured = shape();
     if (!timing) return capture(&graph, nullptr);
     for (int p = 0; p < 2; ++p) {
         for (int q = 0; q < 2; ++q)
@@ -659,10 +790,11 @@ int run_solve(Ctx* ctx, const std::vector<PairHost>& pairs, double tol, long lon
         }
         insts.push_back(I);
     }
-    int rc = B.set_instances(insts, st);
     // live sweep timing: single-instance graph solves only (the bytes of a
-    // timed launch are then those of the one instance)
+    // timed launch are then those of the one instance).  It and the profiled
+    // solve time the chain's kernels, so they run the chain at every size.
     const int timing = ctx->sweep_timing && insts.size() == 1 && !kt ? 1 : 0;
+    int rc = B.set_instances(insts, st, !timing && !kt);
     if (rc == HOT_OK) rc = B.ensure_graph(timing);   // also fixes the launch dimensions
     if (rc != HOT_OK) {
         cleanup();
@@ -706,8 +838,8 @@ int run_solve(Ctx* ctx, const std::vector<PairHost>& pairs, double tol, long lon
                 err = HOT_ECUDA;
                 break;
             }
-            launches += launches_per_block(fp64, (int)K, B.ninst == 1) + kLaunchesBlockEnd;
-            cudaMemcpyAsync(&B.h_running[1 + (nb & 1)], B.d_running, sizeof(int), cudaMemcpyDeviceToHost, st);
+            launches += B.launches();
+            cudaMemcpyAsync((void*)B.running(nb), B.d_running, 2 * sizeof(int), cudaMemcpyDeviceToHost, st);
             if (track)
                 cudaMemcpyAsync(B.h_stb + (size_t)(nb & 1) * B.cap, B.d_st, sizeof(int) * live.size(),
                                 cudaMemcpyDeviceToHost, st);
@@ -720,8 +852,27 @@ int run_solve(Ctx* ctx, const std::vector<PairHost>& pairs, double tol, long lon
                 // the kernels stop walking the finished pairs' items (and a last
                 // pair runs the single-instance kernels).  Every pair keeps its
                 // own state, so its iterates do not change.
-                const int run_prev = B.h_running[1 + ((nb - 1) & 1)];
-                if (track && live.size() > 1 && run_prev > 0 && (size_t)run_prev * 4 <= live.size()) {
+                const int run_prev = B.running(nb - 1)[0];
+                if (B.running(nb - 1)[1]) {                      // a bounded wait ran out on the device
+                    err = HOT_ECUDA;
+                    ++nb;
+                    break;
+                }
+                bool rebuild = track && live.size() > 1 && run_prev > 0 && (size_t)run_prev * 4 <= live.size();
+                if (track && !rebuild && run_prev > 0 && run_prev < (int)live.size() && B.n_group == 0) {
+                    // or once few enough tiles run for k_group32
+                    const int* sts = B.h_stb + (size_t)((nb - 1) & 1) * B.cap;
+                    long long tiles = 0;
+                    bool any = false;
+                    for (size_t q = 0; q < live.size(); ++q) {
+                        const Inst* I = insts[live[q]];
+                        if (sts[q] != ST_RUNNING || !I->group_ok) continue;
+                        any = true;
+                        tiles += (long long)I->n * I->nb1 + (long long)I->m * I->nb2;
+                    }
+                    rebuild = any && tiles <= B.group_tiles();
+                }
+                if (rebuild) {
                     cudaEventSynchronize(ev[nb & 1]);            // block nb and its status copy
                     const int* sts = B.h_stb + (size_t)(nb & 1) * B.cap;
                     note_finished(sts);
@@ -761,7 +912,7 @@ int run_solve(Ctx* ctx, const std::vector<PairHost>& pairs, double tol, long lon
                         cudaGetLastError();
                     }
                 }
-                if (B.h_running[1 + ((nb - 1) & 1)] <= 0) {
+                if (run_prev <= 0) {
                     ++nb;
                     break;
                 }
@@ -776,7 +927,7 @@ int run_solve(Ctx* ctx, const std::vector<PairHost>& pairs, double tol, long lon
             }
             launch_block_end(B.d_work, B.ld, fp64, (int)K, B.a1, B.a2, B.a3, st);
             cudaEventRecord(pev[3 * K], st);
-            cudaMemcpyAsync(&B.h_running[1], B.d_running, sizeof(int), cudaMemcpyDeviceToHost, st);
+            cudaMemcpyAsync((void*)B.running(0), B.d_running, 2 * sizeof(int), cudaMemcpyDeviceToHost, st);
             if (cudaStreamSynchronize(st) != cudaSuccess) {
                 err = HOT_ECUDA;
                 break;
@@ -799,7 +950,7 @@ int run_solve(Ctx* ctx, const std::vector<PairHost>& pairs, double tol, long lon
             cudaEventElapsedTime(&c, pev[3 * K - 1], pev[3 * K]);
             kt->block_end_ms += c;
             kt->block_end_launches += kLaunchesBlockEnd;
-            if (B.h_running[1] <= 0) {
+            if (B.running(0)[0] <= 0) {
                 ++nb;
                 break;
             }
@@ -826,7 +977,7 @@ int run_solve(Ctx* ctx, const std::vector<PairHost>& pairs, double tol, long lon
         cleanup();
         return HOT_ECUDA;
     }
-    if (kt) launches = nb * (launches_per_block(fp64, (int)K, insts.size() == 1) + kLaunchesBlockEnd);
+    if (kt) launches = nb * B.launches();
     for (size_t q = 0; q < insts.size(); ++q) {
         Inst* I = insts[q];
         cudaMemcpy(&I->ctl_host, I->desc.ctl, sizeof(HotCtl), cudaMemcpyDeviceToHost);

@@ -37,6 +37,7 @@ struct Inst {
     int m = 0, n = 0;        // grid: the histograms are m x n
     int fp64 = 0;
     int TR = 0, nb1 = 0, nb2 = 0, n_k1 = 0;
+    int group_ok = 0;        // k_group32 may run its iterations (group_rule)
     size_t big_bytes = 0, small_bytes = 0;
     char* big = nullptr;     // v0, d0, d1, xr, zr
     char* small = nullptr;   // sums, vectors, mu, ctl
@@ -70,8 +71,15 @@ int inst_create(const PairHost& p, int fp64, const hot_config& cfg, double tol, 
 void inst_destroy(Inst* I, cudaStream_t st);
 
 // Device work tables plus the instantiated block graph that reads them.
-// Prefix tables (cap + 1 ints each): tiles, slabs, k_vec items, k_kkt1 chunks, k_alpha32 chunks.
-constexpr int kPreTables = 5;
+// Prefix tables (cap + 1 ints each): tiles, slabs, k_vec items, k_kkt1 chunks, k_alpha32 chunks, sweep tiles.
+constexpr int kPreTables = 6;
+// CTAs of k_group32 for the grouped instances of a batch, by a cost model of
+// one iteration: entries (instance, rank, group size) per CTA.
+struct GroupPlan {
+    std::vector<int> start;      // [grid + 1]
+    std::vector<int4> entries;
+};
+GroupPlan plan_groups(const std::vector<int>& inst, const std::vector<int>& tiles, const std::vector<int>& elems, int grid);
 struct Batch {
     int device = 0;
     int cap = 0;
@@ -81,14 +89,21 @@ struct Batch {
     WorkDev* d_work = nullptr;
     HotInst* d_inst = nullptr;
     int* d_pre = nullptr;
-    int* d_running = nullptr;
+    int* d_running = nullptr;       // [2]: instances still running, error flag of the bounded waits
+    int* d_gstart = nullptr;        // [ggrid + 1]
+    int4* d_gent = nullptr;         // [ggrid + cap]
+    int* h_gstart = nullptr;        // pinned
+    int4* h_gent = nullptr;         // pinned
+    int ggrid = 0;                  // grid of k_group32 on this device
+    // k_group32 takes part while the instances it may run have at most this many tiles
+    long long group_tiles() const { return 4LL * ggrid; }
     int* d_st = nullptr;            // [cap] per-instance status after each check
     int* h_st = nullptr;            // pinned mirror
     int* h_stb = nullptr;           // pinned, [2][cap]: statuses after the last two blocks (finish times)
     WorkDev* h_work = nullptr;      // pinned
     HotInst* h_inst = nullptr;      // pinned
     int* h_pre = nullptr;           // pinned
-    int* h_running = nullptr;       // pinned, [4]
+    int* h_running = nullptr;       // pinned, [6]: staging, then the pairs copied after even and odd blocks
     cudaGraphExec_t graph = nullptr;
     // sweep-timing mode: two instances of the block graph, launched
     // alternately, each with a CUDA event pair around the sweep of iteration
@@ -100,14 +115,23 @@ struct Batch {
     cudaStream_t cap_stream = nullptr;
     LaunchDims ld{};
     int ninst = 0;
-    int single = -1;                // the instance count the graphs were captured for is 1 (1), more (0), none (-1)
-    int pad = 0;                    // some instance needs the general sweep: a side that is not a
-                                    // multiple of 4, or (FP32) real-valued bin coordinates
-    int pad_captured = -1;          // pad of the captured graphs
+    // instances that k_group32 runs, and those of the chain of kernels; pad:
+    // some instance of that kind needs the general sweep: a side that is not
+    // a multiple of 4, or (FP32) real-valued bin coordinates
+    int n_group = 0, n_chain = 0;
+    int pad = 0, gpad = 0;
+    int shape() const {             // what a captured graph depends on
+        return (n_group > 0) | (n_chain > 0) << 1 | (n_chain == 1) << 2 | (pad != 0) << 3 | (gpad != 0) << 4;
+    }
+    int captured = -1;              // shape() of the captured graphs (-1: none)
+    int launches() const;           // kernels of one block
+    const int* running(long long block) const { return h_running + 2 + 2 * (block & 1); }
     void drop_graphs();
     ~Batch();
     int reserve(int n);
-    int set_instances(const std::vector<Inst*>& v, cudaStream_t st);   // async H2D
+    // async H2D; group: k_group32 takes the instances it may take
+    int set_instances(const std::vector<Inst*>& v, cudaStream_t st, bool group = true);
+    void launch_iterations(cudaStream_t st, cudaEvent_t* ev) const;
     int ensure_graph(int timing = 0);
     int launch_block(cudaStream_t st, long long block = 0) const;
     int timed_iter() const { return (K - 1) / 2; }   // a non-check iteration when K >= 2

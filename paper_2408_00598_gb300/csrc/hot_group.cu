@@ -1,0 +1,699 @@
+// One check block (K iterations of Algorithm 2, arXiv 2408.00598) of an FP32
+// bulk instance in one kernel: k_group32.
+//
+// The chain k_vec32 -> k_alpha32 -> k_sweep32 costs three launch boundaries
+// per iteration, about 20 us on small grids whose sweep itself takes one or
+// two.  Here a group of CTAs takes an instance through the K iterations of a
+// block with two waits per iteration:
+//   A  slab sums: T and P of each slab (a warp per slab) from the row sums;
+//      wait 1
+//   B  every CTA forms the O(m + n) stage of Prop. 3 for itself (a few
+//      thousand cycles, the same bits in every CTA), then for each of its
+//      tiles the pieces of A^T y-bar (in shared memory), Steps 2-4, and the
+//      tile's row and column sums;
+//      wait 2
+// A CTA owns the same tiles in every iteration, so the flow state needs no
+// exchange: only the row sums (2mn pairs), column partials and slab sums go
+// through L2.  The first pass of the next iteration's state is loaded before
+// the waits.  Every sum that feeds the iterates is formed in the order of the
+// chain of kernels (hot_dev.cuh, k_vec32, k_sweep32), so an instance's iterates
+// do not depend on which of the two ran, nor on the size of its group.
+//
+// The groups of one launch are independent.  The grid is launched
+// cooperatively, so that the CTAs of a group are resident together; every
+// wait is bounded and sets W->err when it runs out.
+#include "hot_dev.cuh"
+
+namespace hot {
+
+namespace {
+
+constexpr int kW = kThreads / 32;
+constexpr int kRowN = kRowSmemBytes / sizeof(float) + 256;
+constexpr int kTileTable = 32;            // tiles of a CTA whose geometry is kept
+constexpr int kRing = 4;                  // passes of state in flight (one float4 of u and of d per thread each)
+constexpr int kPollLimit = 1 << 22;       // polls of a wait before it gives up (a few seconds)
+
+// Geometry of a tile; offsets fit 32 bits (sides up to kMaxGroupSide).
+struct GTile {
+    int slab, band, r0, nr;
+    int row, colp, elem;          // g_row, g_colp, first element of row r0
+    int tile;
+};
+__device__ __forceinline__ GTile gtile(const HotInst& I, int t) {
+    GTile g;
+    g_tile_slab(I, t, g.slab, g.band);
+    const int S = g_side(I, g.slab);
+    g.r0 = g.band * I.TR;
+    g.nr = min(S, g.r0 + I.TR) - g.r0;
+    g.row = (int)g_row(I, g.slab);
+    g.colp = (int)g_colp(I, g.slab, g.band);
+    g.elem = (int)g_elem(I, g.slab) + g.r0 * g_pitch(I, g.slab);
+    g.tile = t;
+    return g;
+}
+struct GroupSmem {
+    float row[kRowN];
+    float xrow[kRowN];
+    float col[kThreads * 4];
+    float xcol[kThreads * 4];
+    float2 rdf[kW][kMaxTR];
+    float4 st[kRing][2][kThreads];        // the state's passes in flight: u, delta
+    float4 alpha[kMaxTR];
+    float4 beta[kMaxGroupSide];
+    // T and P of every slab, replaced in place by the stage's vectors:
+    // (mvA, sy) of column j at j, (mvS, sp) of row k at n + k
+    float4 vec[2 * kMaxGroupSide];
+    float2 mar[2 * kMaxGroupSide];        // column totals of mu (cm2), row totals of nu (rm2)
+    float2 red[(kNK - 1) * 32];
+    HotInst I;
+    CycleK C;
+    GTile tile[kTileTable];
+    StageK K;
+    DF sm1, sm2;                          // the marginals' sums
+    P32 p[64];                            // of every iteration of the block (check_every <= 64)
+    int dead;
+};
+
+// All CTAs of the group have arrived for the `epoch`-th time in this launch
+// (k_block_end clears the counter).  One thread per CTA arrives with a release
+// and polls with an acquire: 2,300 cycles with 32 CTAs, 2,800 with 304 (a flag
+// per CTA polled by whole warps took 2,000 and 8,200: the polls hold up the
+// arrivals).  The barrier at the top orders the CTA's writes before thread 0's
+// arrival, the one at the end the other CTAs' writes before this CTA's reads
+// (through L2, __ldcg).  Without the __syncwarp the first warp stayed split
+// after the poll, and what it runs alone next (group_stage) took three times
+// as long.
+__device__ __forceinline__ bool group_wait(GroupSmem& s, int G, unsigned epoch, int* err) {
+    __syncthreads();
+    if (G == 1) return true;
+    if (threadIdx.x == 0) {
+        unsigned* count = s.I.gcount;
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;\n" ::"l"(count) : "memory");
+        unsigned v;
+        int left = kPollLimit;
+        do {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(v) : "l"(count) : "memory");
+        } while (v < epoch * (unsigned)G && --left > 0);
+        if (left <= 0) {
+            s.dead = 1;
+            atomicExch(err, 1);
+        }
+    }
+    __syncwarp();                                // the polling thread rejoins its warp
+    __syncthreads();
+    return s.dead == 0;
+}
+
+// What a thread needs of a half (f1 or f2): side, row pitch, column groups,
+// rows per pass, and the thread's row and column group of a pass.
+struct Half {
+    int S, Sp, NC, P, ro, cg;
+};
+__device__ __forceinline__ Half half_of(int side) {
+    Half h;
+    h.S = side;
+    h.Sp = (side + 3) & ~3;
+    h.NC = h.Sp / 4;
+    h.P = kThreads / h.NC;
+    h.ro = (int)threadIdx.x / h.NC;
+    h.cg = (int)threadIdx.x - h.ro * h.NC;
+    return h;
+}
+
+// T or P of slab q (k_vec32's sums, in its order), one warp: T, the total of
+// the slab's row sums (lane-strided, then the shuffle tree), or P, the column
+// sum across the other half's slabs: P2[j] for f1 slab j, P1[k] for f2 slab k,
+// in blocks of kVecRows rows, each block in eight runs of eight rows.  Valid
+// in lane 0.
+__device__ __forceinline__ DF slab_sum(const HotInst& I, const float2* __restrict__ rs, int q, bool cross, int lane) {
+    const int m = I.m, n = I.n, h2 = n * m;               // h2: first row of the f2 half
+    const bool f1 = q < n;
+    const int len = f1 ? m : n;
+    int at, step, left;                                   // this lane's terms: at, at + step, ... (left of them)
+    if (cross) {
+        const int c0 = (lane >> 3) * kVecRows + (lane & 7) * 8;
+        step = f1 ? n : m;
+        at = (f1 ? h2 + q : q - n) + c0 * step;
+        left = len - c0;                                  // f1 slab j: m rows k; f2 slab k: n rows j
+    } else {
+        step = 32;
+        at = (f1 ? q * m : h2 + (q - n) * n) + lane;
+        left = (len - lane + 31) >> 5;
+    }
+    float2 v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = u < left ? __ldcg(rs + at + u * step) : make_float2(0.f, 0.f);
+    DF c{0.f, 0.f}, b{0.f, 0.f};
+#pragma unroll
+    for (int u = 0; u < 8; ++u) c = df_add(c, df_ld(v[u]));
+    if (!cross) {
+#pragma unroll 1
+        for (int o = 16; o > 0; o >>= 1) c = df_add(c, df_shfl_down(c, o));
+        return c;
+    }
+#pragma unroll 1
+    for (int u = 0; u < 8; ++u)                           // the block's eight runs, in order
+        b = df_add(b, DF{__shfl_sync(0xffffffffu, c.hi, (lane & ~7) + u), __shfl_sync(0xffffffffu, c.lo, (lane & ~7) + u)});
+    c = DF{0.f, 0.f};
+#pragma unroll 1
+    for (int u = 0; u * kVecRows < len; ++u)
+        c = df_add(c, DF{__shfl_sync(0xffffffffu, b.hi, 8 * u), __shfl_sync(0xffffffffu, b.lo, 8 * u)});
+    return c;
+}
+
+// Half totals F1, F2 (the order of k_vec32's item totals and alpha32_stage's
+// block sum: the items of 8 slabs left to right, the shuffle tree over 32
+// items, then the warps' totals) and the stage's scalars, by one warp.
+__device__ __forceinline__ void group_stage(GroupSmem& s, float kdl, int lane) {
+    const int m = s.I.m, n = s.I.n;
+    const int t1 = (n + 7) / 8, t2 = (m + 7) / 8;                 // t1 + t2 <= 64
+    DF F1{0.f, 0.f}, F2{0.f, 0.f};
+#pragma unroll 1
+    for (int q = lane; q - lane < t1 + t2; q += 32) {
+        DF a{0.f, 0.f}, b{0.f, 0.f};
+        const bool first = q < t1;
+        const int s0 = (first ? q : q - t1) * 8, cnt = first ? n : m;
+        const float4* tp = s.vec + (first ? 0 : n);
+        DF tot{0.f, 0.f};
+#pragma unroll 1
+        for (int w = 0; w < 8; ++w)
+            if (s0 + w < cnt) tot = df_add(tot, DF{tp[s0 + w].x, tp[s0 + w].y});
+        if (first) a = tot;
+        else b = tot;
+#pragma unroll 1
+        for (int o = 16; o > 0; o >>= 1) {
+            a = df_add(a, df_shfl_down(a, o));
+            b = df_add(b, df_shfl_down(b, o));
+        }
+        F1 = df_add(F1, a);
+        F2 = df_add(F2, b);
+    }
+    F1 = DF{__shfl_sync(0xffffffffu, F1.hi, 0), __shfl_sync(0xffffffffu, F1.lo, 0)};
+    F2 = DF{__shfl_sync(0xffffffffu, F2.hi, 0), __shfl_sync(0xffffffffu, F2.lo, 0)};
+    const float4 last = s.vec[n + m - 1];
+    const StageK K = stage_scalars(m, n, s.C, s.sm1, s.sm2, F1, F2, DF{last.x, last.y}, DF{last.z, last.w},
+                                   df_ld(s.mar[n + m - 1]), kdl);
+    if (lane == 0) s.K = K;
+}
+
+// The stage's vectors, one entry per thread.
+__device__ __forceinline__ void group_vectors(GroupSmem& s) {
+    const int m = s.I.m, n = s.I.n;
+    const StageK& K = s.K;
+#pragma unroll 1
+    for (int q = threadIdx.x; q < m + n; q += kThreads) {
+        const float4 t = s.vec[q];
+        const DF T{t.x, t.y}, P{t.z, t.w};
+        const bool col = q < n, last = q == n + m - 1;
+                const DF c = df_ld(s.mar[q]);
+        // column: a_j, bb_j; row: (T2 - P1)/sigma, r3_k
+        const DF A = df_mul(col ? df_sub(P, T) : df_sub(T, P), K.is);
+        DF B = df_mul(df_sub(c, T), K.is);
+        if (last) B = df_sub(B, K.drop);
+        const DF Bi = df_mul(B, col ? K.imin : K.in);       // bb_j (1/m + 1/n); r3_k / n
+        const DF e = df_add(A, col ? df_neg(B) : B);    // a_j - bb_j; e_k
+        const DF f = df_mul(df_add(e, col ? K.T3in : K.cst), col ? K.in : K.imn);   // sy_j + yasum; s_k
+        DF x, y;
+        if (col) {
+            x = df_sub(df_mul(A, K.in), Bi);                   // mvA_j
+            y = df_sub(f, K.yasum);                            // sy_j
+        } else {
+            const DF ya = df_add(df_neg(df_mul(df_add(f, K.dsiw), last ? K.dl : K.im)), K.tin);
+            x = df_sub(df_add(Bi, K.T3in2), df_mul(ya, (float)(m + n)));   // mvS_k
+            y = df_sub(f, df_mul(ya, (float)n));                  // sp_k
+        }
+        s.vec[q] = make_float4(x.hi, x.lo, y.hi, y.lo);
+    }
+}
+
+// The inputs of one piece of a tile that do not wait for the stage: item < nr
+// is the alpha piece of row r0 + item, item >= nr the beta piece of column
+// item - nr.
+struct PieceLd {
+    float2 a0, x, y;              // y: a column's first two bands until piece_finish sums them
+    float2 z;                     // and the next two
+    float xc;
+};
+__device__ __forceinline__ PieceLd piece_load(const HotInst& I, const GTile& g, int S, int item,
+                                              const float2* __restrict__ rs, const float* __restrict__ cs) {
+    PieceLd p;
+    const int m = I.m, n = I.n;
+    const bool f1 = g.slab < n, row = item < g.nr;
+    const int e = row ? g.r0 + item : item - g.nr;
+    p.a0 = I.ab0_32[2 * g.row + (row ? 0 : S) + e];
+    p.xc = I.X32[(f1 ? 0 : m) + e];
+    if (row) {
+        const int j = f1 ? g.slab : e, k = f1 ? e : g.slab - n;
+        p.x = __ldcg(rs + n * m + k * n + j);
+        p.y = __ldcg(rs + j * m + k);
+    } else {
+        const int nb = f1 ? I.nb1 : I.nb2;
+        const float* c = cs + (g.colp - g.band * S) + e;
+        p.y.x = __ldcg(c);
+        p.y.y = nb > 1 ? __ldcg(c + S) : 0.f;
+        p.z.x = nb > 2 ? __ldcg(c + 2 * S) : 0.f;
+        p.z.y = nb > 3 ? __ldcg(c + 3 * S) : 0.f;
+        p.x = I.K2[g.row + e];
+    }
+    return p;
+}
+// The piece itself (piece_dv and piece_pack), into shared memory; the pair and
+// the float4 also go to global memory on check iterations (the restart and the
+// objective read them there).
+__device__ __forceinline__ void piece_finish(GroupSmem& s, const GTile& g, int S, int item, const PieceLd& p,
+                                             const float* __restrict__ cs, bool out) {
+    const HotInst& I = s.I;
+    const PieceK K = piece_consts(I, s.C);
+    const int n = I.n;
+    const bool f1 = g.slab < n, row = item < g.nr;
+    const int e = row ? g.r0 + item : item - g.nr;
+    const float4 own = s.vec[g.slab];                            // of the slab itself
+    const float4 oth = s.vec[row ? (f1 ? n + e : e) : g.slab];
+    const float4 vj = f1 ? own : oth, vk = f1 ? oth : own;
+    float kd = 0.f;                                              // the column's total over its bands, left to right
+    if (!row) {
+        const int nb = f1 ? I.nb1 : I.nb2;
+        kd = __fadd_rn(kd, p.y.x);
+        if (nb > 1) kd = __fadd_rn(kd, p.y.y);
+        if (nb > 2) kd = __fadd_rn(kd, p.z.x);
+        if (nb > 3) kd = __fadd_rn(kd, p.z.y);
+#pragma unroll 1
+        for (int b = 4; b < nb; ++b) kd = __fadd_rn(kd, __ldcg(cs + (g.colp + (b - g.band) * S) + e));
+    }
+    // row: R1 / sigma, then + mvA_j + mvS_k, over m + n; column: K2 - kd / (sigma side) + colc
+    DF q = df_mul(row ? df_sub(df_ld(p.x), df_ld(p.y)) : DF{kd, 0.f}, row ? K.is : f1 ? K.isim : K.isin);
+    DF dv{0.f, 0.f};                                             // the dropped row's piece stays 0
+    if (row) {
+        q = df_add(df_add(q, DF{vj.x, vj.y}), DF{vk.x, vk.y});
+        dv = df_mul(q, K.imn);
+        if (!f1) dv = df_neg(dv);
+    } else if (g.slab != n + I.m - 1 || e != n - 1) {
+        const DF colc = df_mul(DF{own.z, own.w}, f1 ? df_neg(K.im) : K.in);
+        dv = df_add(df_sub(df_ld(p.x), q), colc);
+    }
+    PieceIn a;
+    a.a0 = p.a0;
+    a.xc = p.xc;
+    const float4 w = piece_pack(a, dv, K, I.coord_real);
+    if (row) s.alpha[item] = w;
+    else s.beta[e] = w;
+    if (out && (row || g.band == 0)) {
+        const int o = 2 * g.row + (row ? 0 : S) + e;
+        I.dab2[o] = df_st(dv);
+        I.ab32[o] = w;
+    }
+}
+
+// Asynchronous copies of the state into the ring: pass slot c of a tile into
+// st[c % kRing], a commit group per pass.  A thread reads back only what it
+// copied, so its own wait_group is enough; no registers are held meanwhile
+// (spilled registers are costly here: an acquire drops the L1 lines they
+// sit in).
+__device__ __forceinline__ void copy16(void* smem, const void* gmem) {
+    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void copy_pass(GroupSmem& s, int c, bool v, int o, const float* __restrict__ u,
+                                          const float* din) {
+    if (v) {
+        copy16(&s.st[c][0][threadIdx.x], u + o);
+        if (din) copy16(&s.st[c][1][threadIdx.x], din + o);
+        else s.st[c][1][threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+}
+__device__ __forceinline__ int tile_off(const GTile& g, const Half& hf) { return g.elem + hf.ro * hf.Sp + hf.cg * 4; }
+// the first kRing passes of a tile
+__device__ __forceinline__ void copy_tile(GroupSmem& s, const GTile& g, const Half& hf, const float* __restrict__ u,
+                                          const float* din) {
+    int rr = hf.ro < hf.P ? hf.ro : g.nr, o = tile_off(g, hf);
+#pragma unroll 1
+    for (int c = 0; c < kRing; ++c) {
+        copy_pass(s, c, rr < g.nr, o, u, din);
+        rr += hf.P;
+        o += hf.P * hf.Sp;
+    }
+}
+
+// block_sum_df in rolled loops (the same order): the code of this kernel has
+// to stay in the instruction caches.
+__device__ __forceinline__ void group_block_sum(DF (&v)[kNK - 1], float2* sh) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll 1
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int q = 0; q < kNK - 1; ++q) v[q] = df_add(v[q], df_shfl_down(v[q], o));
+    __syncthreads();
+    if (lane == 0)
+#pragma unroll
+        for (int q = 0; q < kNK - 1; ++q) sh[q * 32 + warp] = df_st(v[q]);
+    __syncthreads();
+    if (warp < kNK - 1) {                            // a warp per sum
+        DF x = lane < kW ? df_ld(sh[warp * 32 + lane]) : DF{0.f, 0.f};
+#pragma unroll 1
+        for (int o = 16; o > 0; o >>= 1) x = df_add(x, df_shfl_down(x, o));
+        __syncwarp();
+        if (lane == 0) sh[warp * 32] = df_st(x);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kNK - 1; ++q) v[q] = df_ld(sh[q * 32]);
+    __syncthreads();
+}
+
+// Steps 2-4 on one tile (k_sweep32's arithmetic and sums).  The tile's first
+// passes are in the ring; din = nullptr: the delta is zero.  `between`
+// runs after the state's last use and before the sums: it loads what the next
+// tile needs, under the sums' latency.
+template <bool CHECK, bool PAD, typename F>
+__device__ __forceinline__ void group_sweep(GroupSmem& s, const GTile& g, const Half& hf, const P32& p,
+                                            const float* __restrict__ u, const float* din, float* dout,
+                                            float2* __restrict__ rs_out, float* __restrict__ cs_out, F between) {
+    const HotInst& I = s.I;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int S = hf.S, Sp = hf.Sp, NC = hf.NC, P = hf.P, nr = g.nr;
+    const int ro = hf.ro;
+    const bool active = ro < P;
+    const int c0 = hf.cg * 4;
+    const int nval = PAD ? S - c0 : 4;
+    const int cr = PAD ? I.coord_real : 0;
+    const float h = p.h;
+    float4 bq[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        bq[e] = active && (!PAD || c0 + e < S) ? s.beta[c0 + e] : make_float4(0.f, 0.f, 0.f, 0.f);
+        if (!cr) {
+            const float cf = bq[e].w;
+            bq[e] = make_float4(fmaf(cf * cf, h, -bq[e].x), bq[e].y, bq[e].z, cf);
+        }
+    }
+    float cacc[4], xacc[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) cacc[e] = xacc[e] = 0.f;
+    float k32[kNK - 1] = {0.f, 0.f, 0.f, 0.f};
+    const int step = P * Sp, rstep = P * (NC + 1);
+    int at = tile_off(g, hf);                         // this thread's element of the pass
+    int sr = ro * (NC + 1) + hf.cg;                   // and its row partial
+    int rr = active ? ro : nr;
+    const int npass = (nr + P - 1) / P;
+    // this thread's row of the tile (rows below) and its row sum of u
+    const int r = tid;
+    const float2 r0 = r < nr ? I.rs02[g.row + g.r0 + r] : make_float2(0.f, 0.f);
+#pragma unroll 1
+    for (int q = 0; q < npass; ++q) {
+            asm volatile("cp.async.wait_group %0;\n" ::"n"(kRing - 1) : "memory");
+            const int c = q % kRing;
+            if (rr < nr) {
+                const float4 Uq = s.st[c][0][tid], Dq = s.st[c][1][tid];
+                const float uu[4] = {Uq.x, Uq.y, Uq.z, Uq.w};
+                const float dd[4] = {Dq.x, Dq.y, Dq.z, Dq.w};
+                const float4 a = s.alpha[rr];
+                const float rf = a.w;
+                const float Ar = fmaf(rf * rf, h, -a.x);
+                const float m2hr = -2.f * h * rf;
+                float out[4], xo[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float4 b = bq[e];
+                    float Gh, Gl;
+                    if (PAD && cr) {
+                        reduced_cost(a, b, h, 1, Gh, Gl);
+                    } else {
+                        Gh = fmaf(m2hr, b.w, Ar + b.x);
+                        Gl = -(a.y + b.y);
+                    }
+                    const float Dv = a.z + b.z;
+                    const float sv = uu[e] + dd[e];
+                    const float w = fmaf(-sv, p.sih, -Dv);
+                    const float mg = -(Gh + Gl);
+                    const float r = fmaxf(w, mg);
+                    out[e] = !PAD || e < nval ? fmaf(p.trs, r, p.rho * dd[e]) : 0.f;
+                    if constexpr (CHECK) {
+                        xo[e] = 0.f;
+                        if (!PAD || e < nval) {
+                            const float zb = (w > mg) ? ((Gh + Gl) + w) : 0.f;
+                            const float xb = fmaf(p.sf, Dv, sv);
+                            xo[e] = xb;
+                            const float mn = fminf(xb, zb);
+                            k32[0] = fmaf(r, r, k32[0]);
+                            k32[1] = fmaf(mn, mn, k32[1]);
+                            k32[2] = fmaf(xb, xb, k32[2]);
+                            k32[3] = fmaf(zb, zb, k32[3]);
+                            xacc[e] += xb;
+                        }
+                    }
+                    cacc[e] += out[e];
+                }
+                *reinterpret_cast<float4*>(dout + at) = make_float4(out[0], out[1], out[2], out[3]);
+                s.row[sr] = (out[0] + out[1]) + (out[2] + out[3]);
+                if constexpr (CHECK) s.xrow[sr] = (xo[0] + xo[1]) + (xo[2] + xo[3]);
+            }
+            copy_pass(s, c, rr + kRing * P < nr, at + kRing * step, u, din);   // into the slot just read
+            rr += P;
+            at += step;
+            sr += rstep;
+    }
+    if (active) {
+        *reinterpret_cast<float4*>(&s.col[ro * Sp + c0]) = make_float4(cacc[0], cacc[1], cacc[2], cacc[3]);
+        if constexpr (CHECK)
+            *reinterpret_cast<float4*>(&s.xcol[ro * Sp + c0]) = make_float4(xacc[0], xacc[1], xacc[2], xacc[3]);
+    }
+    between();
+    __syncthreads();
+    {
+        const int w0 = (warp * NC) / kW, w1 = ((warp + 1) * NC) / kW;
+#pragma unroll 1
+        for (int t = lane; t < nr; t += 32) {
+            DF a{0.f, 0.f};
+#pragma unroll 1
+            for (int cc = w0; cc < w1; ++cc) a = df_add(a, s.row[t * (NC + 1) + cc]);
+            s.rdf[warp][t] = df_st(a);
+        }
+    }
+    if constexpr (CHECK) {
+        DF kd[kNK - 1];
+#pragma unroll
+        for (int qq = 0; qq < kNK - 1; ++qq) kd[qq] = DF{k32[qq], 0.f};
+        group_block_sum(kd, s.red);                  // its barriers also publish rdf
+        if (tid == 0) {
+            float2* o = reinterpret_cast<float2*>(I.tile_kkt) + g.tile * kNK;
+#pragma unroll
+            for (int qq = 0; qq < kNK - 1; ++qq) o[qq] = df_st(kd[qq]);
+        }
+    } else {
+        __syncthreads();
+    }
+    // rows on the first warps, columns on the last: side by side up to sides of 128
+    if (r < nr) {
+        float2 v[kW];
+#pragma unroll
+        for (int w = 0; w < kW; ++w) v[w] = s.rdf[w][r];
+        DF a = df_ld(v[0]);
+#pragma unroll
+        for (int w = 1; w < kW; ++w) a = df_add(a, df_ld(v[w]));
+        a = df_add(a, df_ld(r0));
+        __stcg(rs_out + g.row + g.r0 + r, df_st(a));
+    }
+    if (const int cc = kThreads - 1 - tid; cc < S) {
+        DF a{0.f, 0.f}, x{0.f, 0.f};
+#pragma unroll 4
+        for (int qq = 0; qq < P; ++qq) {
+            a = df_add(a, s.col[qq * Sp + cc]);
+            if constexpr (CHECK) x = df_add(x, s.xcol[qq * Sp + cc]);
+        }
+        __stcg(cs_out + g.colp + cc, df_f(a));
+        if constexpr (CHECK) I.xcs_part[g.colp + cc] = df_val(x);
+    }
+    if constexpr (CHECK) {
+        // the row sums of x-bar, in the same order, through the same buffer
+        __syncthreads();
+        const int w0 = (warp * NC) / kW, w1 = ((warp + 1) * NC) / kW;
+#pragma unroll 1
+        for (int t = lane; t < nr; t += 32) {
+            DF x{0.f, 0.f};
+#pragma unroll 1
+            for (int cc = w0; cc < w1; ++cc) x = df_add(x, s.xrow[t * (NC + 1) + cc]);
+            s.rdf[warp][t] = df_st(x);
+        }
+        __syncthreads();
+        if (r < nr) {
+            DF x = df_ld(s.rdf[0][r]);
+#pragma unroll 1
+            for (int w = 1; w < kW; ++w) x = df_add(x, df_ld(s.rdf[w][r]));
+            I.xrs[g.row + g.r0 + r] = df_val(x);
+        }
+    }
+}
+
+template <bool PAD>
+__device__ __forceinline__ void group_instance(GroupSmem& s, int rank, int G, int K, int* err) {
+    const HotInst& I = s.I;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int ns = I.m + I.n, nt = g_ntiles(I);
+    const int nq = (nt - rank + G - 1) / G;            // tiles of this CTA: rank, rank + G, ...
+    const bool dz = I.ctl->dzero != 0;
+    const float* u = (const float*)I.u;
+    float* d0 = (float*)I.d0;
+    float* d1 = (float*)I.d1;
+    const Half h1 = half_of(I.m), h2 = half_of(I.n);
+    if (tid < K) s.p[tid] = make_p32(I.ctl->sigma, I.ctl->k + tid, I.h, I.gadmm, I.relax);
+    if (tid == 64) {
+        s.sm1 = df_from(I.sum_mu1);
+        s.sm2 = df_from(I.sum_mu2);
+    }
+#pragma unroll 1
+    for (int q = tid; q < ns; q += kThreads) s.mar[q] = q < I.n ? I.cm2[q] : I.rm2[q - I.n];
+    if (tid >= 128 && tid - 128 < min(nq, kTileTable)) s.tile[tid - 128] = gtile(I, rank + (tid - 128) * G);
+    __syncthreads();
+    unsigned epoch = 0;
+#pragma unroll 1
+    for (int it = 0; it < K; ++it) {
+        // iteration it reads the delta of it - 1: d0 at the block's start, then
+        // d1 in place; the check iteration leaves d1 for the restart and writes d0
+        const bool check = it == K - 1;
+        const float* din = it == 0 ? (dz ? nullptr : d0) : d1;
+        float* dout = check ? d0 : d1;
+        const float2* rs = it & 1 ? I.rs2b : I.rs2;
+        float2* rs_out = it & 1 ? I.rs2 : I.rs2b;
+        const float* cs = it & 1 ? I.cs32b : I.cs32;
+        float* cs_out = it & 1 ? I.cs32 : I.cs32b;
+        PieceLd pl = {};
+        if (it > 0 && !group_wait(s, G, ++epoch, err)) return;
+#pragma unroll 1
+        for (int q = 0; q < nq; ++q) {
+            const GTile& g = s.tile[q & (kTileTable - 1)];
+            const Half& hf = g.slab < I.n ? h1 : h2;
+            if (q == 0) {
+                copy_tile(s, g, hf, u, din);                  // arrives under the sums and the second wait
+                // A: slab sums (T and P of slab w as two jobs, on the last warps first)
+#pragma unroll 1
+                for (int w = rank + G * (kW - 1 - warp); w < 2 * ns; w += G * kW) {
+                    const bool cross = w >= ns;
+                    const int slab = cross ? w - ns : w;
+                    const DF v = slab_sum(I, rs, slab, cross, lane);
+                    if (lane == 0) __stcg(reinterpret_cast<float2*>(I.tp + slab) + (cross ? 1 : 0), df_st(v));
+                }
+                if (tid < g.nr + hf.S) pl = piece_load(I, g, hf.S, tid, rs, cs);   // arrives under the wait
+                float kdl = 0.f;
+                if (warp == 0) {
+                    const float* c = cs + g_colp(I, ns - 1, 0) + (I.n - 1);
+#pragma unroll 1
+                    for (int b = 0; b < I.nb2; ++b) kdl = __fadd_rn(kdl, __ldcg(c + b * I.n));
+                }
+                if (!group_wait(s, G, ++epoch, err)) return;
+                // B: the stage
+#pragma unroll 1
+                for (int w = tid; w < ns; w += kThreads) s.vec[w] = __ldcg(I.tp + w);
+                __syncthreads();
+                if (warp == 0) group_stage(s, kdl, lane);
+                __syncthreads();
+                group_vectors(s);
+                __syncthreads();
+            }
+#pragma unroll 1
+            for (int item = tid; item < g.nr + hf.S; item += kThreads) {
+                if (item != tid) pl = piece_load(I, g, hf.S, item, rs, cs);
+                piece_finish(s, g, hf.S, item, pl, cs, check);
+            }
+            __syncthreads();
+            auto between = [&]() {
+                const int qn = q + 1;
+                if (qn == nq || (qn & (kTileTable - 1)) == 0) return;     // the table's end: below
+                const GTile& gn = s.tile[qn & (kTileTable - 1)];
+                const Half& hn = gn.slab < I.n ? h1 : h2;
+                copy_tile(s, gn, hn, u, din);
+                if (tid < gn.nr + hn.S) pl = piece_load(I, gn, hn.S, tid, rs, cs);
+            };
+            if (check)
+                group_sweep<true, PAD>(s, g, hf, s.p[it], u, din, dout, rs_out, cs_out, between);
+            else
+                group_sweep<false, PAD>(s, g, hf, s.p[it], u, din, dout, rs_out, cs_out, between);
+            if (nq > kTileTable && (((q + 1) & (kTileTable - 1)) == 0 || q + 1 == nq)) {
+                // the next tiles' geometry (the first ones' after the last)
+                const int qn = q + 1 == nq ? 0 : q + 1;
+                __syncthreads();
+                if (tid < min(nq - qn, kTileTable)) s.tile[tid] = gtile(I, rank + (qn + tid) * G);
+                __syncthreads();
+                if (qn > 0) {
+                    const GTile& gn = s.tile[0];
+                    const Half& hn = gn.slab < I.n ? h1 : h2;
+                    copy_tile(s, gn, hn, u, din);
+                    if (tid < gn.nr + hn.S) pl = piece_load(I, gn, hn.S, tid, rs, cs);
+                }
+            }
+        }
+    }
+}
+
+template <bool PAD>
+__global__ void __launch_bounds__(kThreads, 2) k_group32(const WorkDev* __restrict__ W, int K) {
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    GroupSmem& s = *reinterpret_cast<GroupSmem*>(s_raw);
+    const int tid = threadIdx.x;
+    const int e0 = W->gstart[blockIdx.x], e1 = W->gstart[blockIdx.x + 1];
+    if (tid == 0) s.dead = 0;
+#pragma unroll 1
+    for (int e = e0; e < e1; ++e) {
+        const int4 ge = W->gent[e];                    // instance, rank, group size
+        __syncthreads();
+        const HotInst* src = W->inst + ge.x;
+#pragma unroll 1
+        for (int q = tid; q < (int)(sizeof(HotInst) / 8); q += kThreads)
+            reinterpret_cast<double*>(&s.I)[q] = reinterpret_cast<const double*>(src)[q];
+        const CycleK* cyc = src->cyc;
+#pragma unroll 1
+        for (int q = tid; q < (int)(sizeof(CycleK) / 8); q += kThreads)
+            reinterpret_cast<double*>(&s.C)[q] = reinterpret_cast<const double*>(cyc)[q];
+        __syncthreads();
+        if (s.I.ctl->status != ST_RUNNING) continue;   // the same for the whole group
+        group_instance<PAD>(s, ge.y, ge.z, K, W->err);
+        asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    }
+}
+
+}  // namespace
+
+static_assert(sizeof(HotInst) % 8 == 0 && sizeof(CycleK) % 8 == 0, "descriptors are copied in 8-byte words");
+
+size_t group_smem() { return sizeof(GroupSmem); }
+
+cudaError_t group_init() {
+    cudaError_t e =
+        cudaFuncSetAttribute(k_group32<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GroupSmem));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_group32<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GroupSmem));
+    return e;
+}
+
+int group_grid() {
+    static int cache[64];                    // per device ordinal; 0 = not yet queried
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    if (cache[dev] == 0) {
+        int sms = 0, a = 0, b = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (group_init() != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_group32<false>, kThreads, sizeof(GroupSmem)) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_group32<true>, kThreads, sizeof(GroupSmem)) != cudaSuccess)
+            return 0;
+        cache[dev] = sms * (a < b ? a : b);
+    }
+    return cache[dev];
+}
+
+void launch_group(const WorkDev* w, int grid, int K, bool pad, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = sizeof(GroupSmem);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;       // the CTAs of a group wait on one another
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, pad ? k_group32<true> : k_group32<false>, w, K);
+}
+
+}  // namespace hot

@@ -40,6 +40,8 @@ constexpr int kAPT = 4;                // k_alpha32: pieces per thread and chunk
 constexpr int kAlphaChunk = kThreads * kAPT;
 constexpr int kMaxTR = 128;            // FP32 tiles: TR * max(m, n) <= kRowSmemBytes / 4
 constexpr int kMaxTileElems = 16384;   // FP32 tiles: TR * (longer row pitch) <= this
+constexpr int kMaxGroupSide = 256;     // k_group32: longest side (one column per thread)
+constexpr int kMaxGroup = 512;         // k_group32: most CTAs of one instance
 
 enum : int {
     ST_RUNNING = 0,
@@ -107,6 +109,8 @@ struct HotInst {
     int stop_abs;          // 1: stop on the absolute KKT residual
     int coord_real;        // FP32 mode: some bin coordinate is not an integer in [-2048, 2048], so the
                            // pieces carry h x^2 - alpha as pairs and the sweep forms the cost term in pairs
+    int grp;               // 1: k_group32 runs this instance's iterations, not the chain of kernels
+    int pad0;
     double relax;          // rho of the generalized ADMM
     double h;              // 2^-E
     double norm_b;         // ||b||
@@ -156,6 +160,12 @@ struct HotInst {
     float2* vec2;          // rows of max(m, n): T1, T2, then ceil(n/64) partials of P1 and ceil(m/64) of P2, of u + d
     float2* dab2;          // [4mn] pieces of A^T(y-bar - y0)
     float2* stg2;          // [4][max(m, n)] Prop. 3 stage of the current iteration: mvA, mvS, sy, sp (k_stage32)
+    // k_group32 only: the other row-sum and column-partial buffers (odd
+    // iterations read them), T and P of every slab, the arrival counter
+    float2* rs2b;          // [2mn]
+    float* cs32b;          // [slab][band][column]
+    float4* tp;            // [m + n]
+    unsigned int* gcount;  // arrivals of the group's CTAs in the running launch (0 between launches)
     unsigned int* vcount;  // k_vec32 items of this instance finished in the running launch (0 between launches)
     float2* mu1f;          // [m][n] mu1 as pairs
     float2* mu2f;          // [m][n] mu2 as pairs
@@ -220,12 +230,16 @@ struct WorkDev {
     int ninst;
     int alternate;         // the sweeps' state exceeds L2: odd iterations take the tiles in reverse
     HotInst* inst;         // [ninst]
-    int* pre_tile;         // sweep / restart tiles: n nb1 + m nb2 per instance
+    int* pre_tile;         // restart tiles: n nb1 + m nb2 per instance
+    int* pre_swp;          // sweep tiles: the same, 0 for instances that k_group32 runs
     int* pre_slab;         // k_alpha: m + n slabs per instance
-    int* pre_vec;          // k_vec: 2(m + n) per instance (one warp each); k_vec32: vec32_items(m, n) CTA items
-    int* pre_k1;           // k_kkt1: n_k1 per instance
-    int* pre_achunk;       // k_alpha32: n_achunk per instance
+    int* pre_vec;          // k_vec: 2(m + n) per instance (one warp each); k_vec32: vec32_items(m, n) CTA items (0 for k_group32's)
+    int* pre_k1;           // k_kkt1: n_k1 per instance, and n_achunk more for k_group32's
+    int* pre_achunk;       // k_alpha32: n_achunk per instance (0 for k_group32's)
+    int* gstart;           // k_group32: entries of CTA c are gent[gstart[c]] ... gent[gstart[c + 1] - 1]
+    int4* gent;            // instance, rank in its group, group size
     int* n_running;        // instances still running
+    int* err;              // set when a bounded wait ran out
     int* st_out;           // [ninst] status of each instance after its last check
 };
 
@@ -269,6 +283,10 @@ void launch_solve_kernels(const WorkDev* w, const LaunchDims& ld, int fp64, int 
 void launch_sweep(const WorkDev* w, const LaunchDims& ld, int fp64, int j, bool check, bool pad, cudaStream_t st);
 void launch_block_end(const WorkDev* w, const LaunchDims& ld, int fp64, int K, double a1, double a2, double a3,
                       cudaStream_t st);
+// k_group32 (hot_group.cu): K iterations of every grouped instance in one cooperative launch
+void launch_group(const WorkDev* w, int grid, int K, bool pad, cudaStream_t st);
+int group_grid();                          // CTAs resident at once on the current device (0: not available)
+cudaError_t group_init();
 LaunchDims make_launch_dims(int device, int fp64);
 // resident CTAs of the (non-check) sweep on the current device
 int sweep_grid(int fp64);

@@ -66,7 +66,7 @@ static size_t inst_bytes_estimate(Ctx* ctx, int m, int n, int fp64) {
     const size_t CP = (size_t)n * ((m + tr - 1) / tr) * m + (size_t)m * ((n + tr - 1) / tr) * n;
     // pieces 3 x 32 MN, slab-row sums 5 x 16 MN, marginals 16 MN, column partials 28 CP
     size_t small = MN * (96 + 80 + 16) + CP * 28 + 1024 * 64;
-    if (!fp64) small += MN * 192;       // double-float arrays of FP32 mode
+    if (!fp64) small += MN * 208 + CP * 4 + (size_t)(m + n) * 16;   // double-float arrays and group buffers of FP32 mode
     return big + small;
 }
 
@@ -184,7 +184,9 @@ static void serve_loop(Ctx* ctx) {
         s->batch->launch_block(s->st);
         const int n = (int)insts.size();
         cudaMemcpyAsync(s->batch->h_st, s->batch->d_st, sizeof(int) * n, cudaMemcpyDeviceToHost, s->st);
-        const cudaError_t e = cudaStreamSynchronize(s->st);
+        cudaMemcpyAsync((void*)s->batch->running(0), s->batch->d_running, 2 * sizeof(int), cudaMemcpyDeviceToHost, s->st);
+        cudaError_t e = cudaStreamSynchronize(s->st);
+        if (e == cudaSuccess && s->batch->running(0)[1]) e = cudaErrorUnknown;   // a bounded wait ran out on the device
         std::lock_guard<std::mutex> g(s->mu);
         s->blocks += 2;
         std::vector<Req*> still;

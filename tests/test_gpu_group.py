@@ -1,0 +1,73 @@
+"""k_group32 (one kernel per check block for small instances) against the chain of
+kernels: the same iterates and results, bit for bit.
+
+The live sweep timing mode times the chain's kernels and therefore runs the chain at
+every size; everything else runs k_group32 up to its size rule.  Sides of 2 and 3,
+sides around a tile and a warp, several bands per slab, more tiles than CTAs, and
+real-valued bin positions."""
+import numpy as np
+import pytest
+
+from paper_2408_00598_gb300 import synthetic as syn
+
+pytestmark = pytest.mark.gpu
+
+SIZES = [(2, 2, "white"), (3, 2, "white"), (5, 7, "gauss"), (16, 16, "shapes"), (17, 23, "white"), (33, 31, "white"),
+         (64, 64, "shapes"), (65, 63, "white"), (20, 90, "white"), (96, 96, "gauss"), (129, 127, "white"),
+         (200, 136, "white"), (255, 3, "white"), (3, 256, "white"), (257, 4, "white")]
+
+
+def _both(ctx, mu, nu, **kw):
+    got = []
+    for chain in (0, 1):
+        ctx.sweep_timing(chain)
+        r = ctx.solve(mu, nu, tol=1e-6, max_iter=250, **kw)
+        got.append((r, ctx.flows(r)))
+        ctx.release(r)
+    ctx.sweep_timing(0)
+    return got
+
+
+def _same(got):
+    (a, xa), (b, xb) = got
+    for key in ("ot_value", "dual_value", "rel_kkt", "abs_kkt", "sigma", "iters", "restarts", "status", "max_abs_dual"):
+        assert a[key] == b[key], (key, a[key], b[key])
+    np.testing.assert_array_equal(xa, xb)
+
+
+@pytest.mark.parametrize("m,n,kind", SIZES)
+def test_group_kernel_equals_the_chain(m, n, kind):
+    from paper_2408_00598_gb300 import hot
+    mu, nu = syn.make_pair(kind, m, 1, n)
+    with hot.Context(precision="fp32") as ctx:
+        _same(_both(ctx, mu, nu))
+
+
+@pytest.mark.parametrize("m,n", [(24, 24), (45, 77), (130, 9)])
+def test_group_kernel_equals_the_chain_at_real_positions(m, n):
+    from paper_2408_00598_gb300 import hot
+    rng = np.random.default_rng(m)
+    mu, nu = syn.make_pair("white", m, 2, n)
+    with hot.Context(precision="fp32") as ctx:
+        _same(_both(ctx, mu, nu, xs=np.sort(rng.random(m)), ys=np.sort(rng.random(n))))
+
+
+@pytest.mark.parametrize("check_every", [2, 4, 64])
+def test_group_kernel_equals_the_chain_for_other_block_lengths(check_every):
+    from paper_2408_00598_gb300 import hot
+    mu, nu = syn.make_pair("gauss", 40, 3)
+    with hot.Context(precision="fp32", check_every=check_every) as ctx:
+        _same(_both(ctx, mu, nu))
+
+
+@pytest.mark.parametrize("count", [3, 40])
+def test_groups_of_a_batch_equal_single_solves(count):
+    """Groups of several sizes in one launch, CTAs shared by several instances among them."""
+    from paper_2408_00598_gb300 import hot
+    pairs = [syn.make_pair("white", 4 + (7 * q) % 23, q) for q in range(count)]
+    with hot.Context(precision="fp32") as ctx:
+        out = ctx.solve_batch([p[0] for p in pairs], [p[1] for p in pairs], tol=1e-6, max_iter=300)
+        for (mu, nu), b in zip(pairs, out):
+            a = ctx.solve(mu, nu, tol=1e-6, max_iter=300)
+            ctx.release(a)
+            assert (a["ot_value"], a["dual_value"], a["iters"]) == (b["ot_value"], b["dual_value"], b["iters"])
