@@ -8,8 +8,9 @@
 // b_l = f2_{k,j,l}: with exclusive prefix sums A_i, B_l, the mass moved from i
 // to l is the overlap of [A_i, A_{i+1}) and [B_l, B_{l+1}), and mass beyond
 // min(sum a, sum b) is left unassigned exactly as the sequential loop leaves
-// it.  Each lane takes a set of sources i, finds its first sink by binary
-// search and walks forward; entries are written in (node, i, l) order.
+// it.  In FP64 mode each lane takes a set of sources i, finds its first sink by
+// binary search and walks forward; FP32 mode merges the ends of the two
+// sides.  Entries are written in (node, i, l) order.
 // Flows are clipped at 0 first (an approximate solution may have small
 // negative entries).  In the slab layout both a and b are contiguous rows:
 // a = row k of f1 slab j (m sources i), b = row j of f2 slab k (n sinks l).
@@ -22,10 +23,16 @@ namespace hot {
 
 constexpr int kRecWarps = 8;
 
-// shared memory of one warp in k_recover_df, in floats: a (m floats), b (n
-// floats), padded to an even count, and the pairs A (m + 1), B (n + 1)
-__host__ __device__ constexpr size_t recover_df_words(int m, int n) {
-    return (size_t)m + n + ((m + n) & 1) + 2 * ((size_t)m + 1) + 2 * ((size_t)n + 1);
+// k_recover_df's arrays in shared memory have one unused entry after every
+// eight: its lanes work on runs of consecutive entries (eight at a side of
+// 256), which would otherwise start in the same banks.
+__host__ __device__ constexpr int pidx(int i) { return i + (i >> 3); }
+// shared memory of one warp in k_recover_df, in floats: the pairs A (m + 1) and
+// B (n + 1), the entries' indices (16 bits each) and, to fill, the merge steps
+// (m + n), to an even count
+__host__ __device__ constexpr size_t recover_df_words(int m, int n, bool fill) {
+    return (2 * ((size_t)pidx(m) + 1) + 2 * ((size_t)pidx(n) + 1) + (m + 1) / 2 + (n + 1) / 2 + (fill ? m + n : 0) + 1) &
+           ~(size_t)1;
 }
 // the same for k_recover, in doubles
 __host__ __device__ constexpr size_t recover_words(int m, int n) { return 2 * ((size_t)m + n) + 2; }
@@ -188,54 +195,94 @@ __device__ __forceinline__ DF df_shfl(DF a, int l) {
     return DF{__shfl_sync(0xffffffffu, a.hi, l), __shfl_sync(0xffffffffu, a.lo, l)};
 }
 
-__device__ __forceinline__ void load_node_df(const float* __restrict__ x, int m, int n, int k, int j, float* a,
-                                             float* b, float2* A, float2* B) {
+// One side of a node: the places of the positive flows of ra[0, m) into ix, in
+// order (a converged solution has about a third; the others hold no mass and
+// take no entry), and their exclusive prefix sums into A (which first holds the
+// flows themselves), the total into A[count].  A lane takes a run of consecutive entries: its own prefix
+// sums first, then a warp scan of the runs' totals, then the sums shifted by
+// the run's offset.  Prefix sums of positive entries never decrease, but sums
+// rounded in different orders could by an ulp; the offsets pass through a
+// running maximum and a run's sums are kept between its offset and the next,
+// since the merge below relies on the order.  Returns the count.
+__device__ __forceinline__ int load_side_df(const float* __restrict__ ra, int m, unsigned short* ix, float2* A) {
     const int lane = threadIdx.x & 31;
-    const float* ra = x + node_row_a(m, k, j);
-    const float* rb = x + node_row_b(m, n, k, j);
-    for (int t = lane; t < m; t += 32) a[t] = fmaxf(ra[t], 0.f);
-    for (int t = lane; t < n; t += 32) b[t] = fmaxf(rb[t], 0.f);
-    __syncwarp();
-    // prefix sums of non-negative entries never decrease, but the rounding of
-    // sums formed in different orders (the scan tree) can make a later one
-    // smaller by an ulp; a running maximum restores the order the merge walk
-    // relies on (ma, mb: maxima of the chunks done so far)
-    DF ca{0.f, 0.f}, cb{0.f, 0.f}, ma{0.f, 0.f}, mb{0.f, 0.f};
-    const int L = m > n ? m : n;
-    for (int base = 0; base < L; base += 32) {
-        const int t = base + lane;
-        DF sa{t < m ? a[t] : 0.f, 0.f}, sb{t < n ? b[t] : 0.f, 0.f};
+    int cnt = 0;
+    for (int base = 0; base < m; base += 128) {
+        float v[4];
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const DF ya = df_shfl_up(sa, o), yb = df_shfl_up(sb, o);
-            if (lane >= o) {
-                sa = df_add(sa, ya);
-                sb = df_add(sb, yb);
-            }
+        for (int u = 0; u < 4; ++u) {
+            const int t = base + u * 32 + lane;
+            v[u] = t < m ? __ldg(ra + t) : 0.f;
         }
-        DF ea = df_shfl_up(sa, 1), eb = df_shfl_up(sb, 1);       // exclusive within the chunk
-        if (lane == 0) ea = eb = DF{0.f, 0.f};
-        DF pa = df_max(df_add(ca, ea), ma), pb = df_max(df_add(cb, eb), mb);
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const DF ya = df_shfl_up(pa, o), yb = df_shfl_up(pb, o);
-            if (lane >= o) {
-                pa = df_max(pa, ya);
-                pb = df_max(pb, yb);
+        for (int u = 0; u < 4; ++u) {
+            const unsigned mask = __ballot_sync(0xffffffffu, v[u] > 0.f);
+            if (v[u] > 0.f) {
+                const int at = cnt + __popc(mask & ((1u << lane) - 1u));
+                A[pidx(at)].x = v[u];
+                ix[at] = (unsigned short)(base + u * 32 + lane);
             }
+            cnt += __popc(mask);
         }
-        if (t < m) A[t] = df_st(pa);
-        if (t < n) B[t] = df_st(pb);
-        ma = df_shfl(pa, 31);
-        mb = df_shfl(pb, 31);
-        ca = df_add(ca, df_shfl(sa, 31));
-        cb = df_add(cb, df_shfl(sb, 31));
-    }
-    if (lane == 0) {
-        A[m] = df_st(df_max(ca, ma));
-        B[n] = df_st(df_max(cb, mb));
     }
     __syncwarp();
+    const int per = (cnt + 31) >> 5, i0 = min(cnt, lane * per), i1 = min(cnt, i0 + per);
+    DF s{0.f, 0.f};
+    for (int i = i0; i < i1; ++i) {
+        const float v = A[pidx(i)].x;
+        A[pidx(i)] = df_st(s);
+        s = df_add(s, v);
+    }
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const DF y = df_shfl_up(s, o);
+        if (lane >= o) s = df_add(s, y);
+    }
+    DF off = df_shfl_up(s, 1);
+    if (lane == 0) off = DF{0.f, 0.f};
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const DF y = df_shfl_up(off, o);
+        if (lane >= o) off = df_max(off, y);
+    }
+    const DF total = df_max(df_shfl(s, 31), df_shfl(off, 31));
+    DF next = DF{__shfl_down_sync(0xffffffffu, off.hi, 1), __shfl_down_sync(0xffffffffu, off.lo, 1)};
+    if (lane == 31) next = total;
+    DF prev = off;
+    for (int i = i0; i < i1; ++i) {
+        prev = df_min(df_max(df_add(off, df_ld(A[pidx(i)])), prev), next);
+        A[pidx(i)] = df_st(prev);
+    }
+    if (lane == 0) A[pidx(cnt)] = df_st(total);
+    __syncwarp();
+    return cnt;
+}
+
+// A pair as a double (df_val).  The conversions are written out in integers
+// for normal numbers: FP64 instructions run at a 64th of the FP32 rate here, and
+// the conversions would be two of the three.
+__device__ __forceinline__ double f2d(float x) {
+    const unsigned u = __float_as_uint(x), ex = (u >> 23) & 0xffu;
+    if (ex == 0u || ex == 255u) return ex == 0u && (u << 1) == 0u ? 0.0 : (double)x;
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
+__device__ __forceinline__ double df_dbl(DF a) { return a.lo == 0.f ? f2d(a.hi) : f2d(a.hi) + f2d(a.lo); }
+
+// Adds a side's share of the plan's marginals: min(a_t, max(0, other - A_t)),
+// other the other side's total; the flows a are read again (ra).
+__device__ __forceinline__ void side_marginal(double* __restrict__ marg, int cnt, const float* __restrict__ ra,
+                                              const unsigned short* ix, const float2* A, DF other) {
+    for (int t = threadIdx.x & 31; t < cnt; t += 32) {
+        const int i = ix[t];
+        const float a = __ldg(ra + i);
+        double g = f2d(a);                                   // all of it, up to the entry that `other` cuts
+        if (df_lt(other, df_ld(A[pidx(t + 1)]))) {
+            DF r = df_sub(other, df_ld(A[pidx(t)]));
+            if (!df_pos(r)) r = DF{0.f, 0.f};
+            g = df_dbl(df_min(DF{a, 0.f}, r));
+        }
+        if (g > 0.0) atomicAdd(marg + i, g);
+    }
 }
 
 // The node's coupling as a merge of the source ends A[1..m] with the sink
@@ -243,156 +290,254 @@ __device__ __forceinline__ void load_node_df(const float* __restrict__ x, int m,
 // stands at source p, sink q = d - p; the step from there moves the overlap
 // min(A[p+1], B[q+1]) - max(A[p], B[q]) from source p to sink q (an entry
 // when positive and both the source and the sink hold mass) and passes the
-// nearer end.  These are the pairs and masses of the north-west-corner loops
-// of Algorithm 1, in (i, l) order.  A lane takes a
-// contiguous range of steps and finds its start by a binary search on the
-// merge diagonal (merge path), so a node costs about log2(m + n) +
-// (m + n)/32 steps per lane.
+// nearer end, which is the next step's max(A[p], B[q]).  These are the pairs
+// and masses of the north-west-corner loops of Algorithm 1, in (i, l) order.
+// A lane takes a contiguous range of steps and finds its start by a binary
+// search on the merge diagonal (merge path), so a node costs about log2(m + n)
+// + (m + n)/32 steps per lane.
 __device__ __forceinline__ int merge_split(const float2* A, const float2* B, int m, int n, int d) {
     int lo = d - n > 0 ? d - n : 0, hi = d < m ? d : m;
     while (lo < hi) {
         const int mid = (lo + hi) >> 1;
         // source end mid + 1 is among the first d ends iff it is <= sink end d - mid
-        if (!df_lt(df_ld(B[d - mid]), df_ld(A[mid + 1]))) lo = mid + 1;
+        if (!df_lt(df_ld(B[pidx(d - mid)]), df_ld(A[pidx(mid + 1)]))) lo = mid + 1;
         else hi = mid;
     }
     return lo;
 }
-__device__ __forceinline__ int merge_walk(const float2* A, const float2* B, const float* a, const float* b, int m,
-                                          int n, int p, int q, int steps, int32_t* src, int32_t* dst, double* mass,
-                                          size_t pos, int j, int k) {
-    int cnt = 0;
-    for (int t = 0; t < steps && p < m && q < n; ++t) {
-        const DF ae = df_ld(A[p + 1]), be = df_ld(B[q + 1]);
-        const DF ov = df_sub(df_min(ae, be), df_max(df_ld(A[p]), df_ld(B[q])));
-        if (df_pos(ov) && a[p] > 0.f && b[q] > 0.f) {
-            if (src) {
-                src[pos + cnt] = p * n + j;
-                dst[pos + cnt] = k * n + q;
-                mass[pos + cnt] = df_val(ov);
-            }
-            ++cnt;
-        }
-        if (!df_lt(be, ae)) ++p;
-        else ++q;
-    }
-    return cnt;
-}
 
+// One node (k, j) per warp.  FILL = false: the node's entry count and the
+// plan's marginals.  FILL = true: its entries, 32 merge steps at a time: the
+// walk only notes where each step stands, then consecutive lanes form
+// consecutive steps' overlaps and write the entries next to each other.  (A
+// lane writing its own run put a partial 32-byte sector per entry and array
+// into L2.)  Nothing is written when the plan exceeds cap.
+// Bound: instruction issue (79 % of cycles in both).  256 x 256 after 30
+// iterations: count 0.45 -> 0.26 ms, fill 0.59 -> 0.31 ms; the whole call on a
+// converged pair (11.6 M entries) 1.28 -> 0.46 ms, 512 x 512 (71 M) 10.0 -> 3.3 ms.
+template <bool FILL>
 __global__ void __launch_bounds__(kRecWarps * 32) k_recover_df(const float* __restrict__ x, int m, int n,
-                                                               int count_only,
                                                                int* __restrict__ counts,
                                                                const long long* __restrict__ offs,
-                                                               int32_t* __restrict__ src, int32_t* __restrict__ dst,
-                                                               double* __restrict__ mass, double* __restrict__ marg1,
+                                                               const unsigned long long* __restrict__ total,
+                                                               unsigned long long cap, int32_t* __restrict__ src,
+                                                               int32_t* __restrict__ dst, double* __restrict__ mass,
+                                                               double* __restrict__ marg1,
                                                                double* __restrict__ marg2) {
+    if (FILL && *total > cap) return;
     extern __shared__ float4 shdf[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nw = blockDim.x >> 5;
-    const size_t per = recover_df_words(m, n);           // floats per warp
-    float* a = reinterpret_cast<float*>(shdf) + (size_t)warp * per;
-    float* b = a + m;
-    float2* A = reinterpret_cast<float2*>(b + n + ((m + n) & 1));
-    float2* B = A + m + 1;
+    float2* A = reinterpret_cast<float2*>(reinterpret_cast<float*>(shdf) + (size_t)warp * recover_df_words(m, n, FILL));
+    float2* B = A + pidx(m) + 1;
+    unsigned* e = reinterpret_cast<unsigned*>(B + pidx(n) + 1);
+    unsigned short* ia = reinterpret_cast<unsigned short*>(e + (FILL ? m + n : 0));
+    unsigned short* ib = ia + ((m + 1) & ~1);
     const int nodes = m * n;
-    const int span = (m + n + 31) / 32;                  // merge steps per lane
-    const int d0 = lane * span < m + n ? lane * span : m + n;
-    const int d1 = d0 + span < m + n ? d0 + span : m + n;
-    for (int node = blockIdx.x * nw + warp; node < nodes; node += gridDim.x * nw) {
-        const int k = node / n, j = node % n;    // k-major node order
-        load_node_df(x, m, n, k, j, a, b, A, B);
-        const int p0 = d0 < d1 ? merge_split(A, B, m, n, d0) : m;
-        int c = merge_walk(A, B, a, b, m, n, p0, d0 - p0, d1 - d0, nullptr, nullptr, nullptr, 0, j, k);
-        if (count_only) {
+    for (int r = blockIdx.x * nw + warp; r < nodes; r += gridDim.x * nw) {
+        // warps at work together take different k and j: their sums go to different marginals
+        const int j = r % n, k = (r / n + j) % m;
+        const int node = k * n + j;
+        const float* ra = x + node_row_a(m, k, j);
+        const float* rb = x + node_row_b(m, n, k, j);
+        const int ca = load_side_df(ra, m, ia, A);
+        const int cb = load_side_df(rb, n, ib, B);
+        const int steps = ca && cb ? ca + cb - 1 : 0;    // every step stands inside both sides until one ends
+        const int span = (steps + 31) >> 5;              // merge steps per lane
+        const int d0 = min(steps, lane * span), d1 = min(steps, d0 + span);
+        int p = d0 < d1 ? merge_split(A, B, ca, cb, d0) : ca;
+        int q = d0 - p;
+        int c = 0;
+        int d = d0;
+        if (p < ca && q < cb) {
+            DF ae = df_ld(A[pidx(p + 1)]), be = df_ld(B[pidx(q + 1)]);
+            DF prev = FILL ? DF{0.f, 0.f} : df_max(df_ld(A[pidx(p)]), df_ld(B[pidx(q)]));
+            for (; d < d1 && p < ca && q < cb; ++d) {
+                const bool sf = !df_lt(be, ae);          // source p ends first (or both end)
+                if (FILL) {
+                    e[d] = (unsigned)p | (unsigned)q << 16;
+                } else {
+                    const DF end = sf ? ae : be;
+                    if (df_pos(df_sub(end, prev))) ++c;
+                    prev = end;
+                }
+                p += sf;
+                q += !sf;
+                const DF nx = df_ld(sf ? A[pidx(p + 1 < ca ? p + 1 : ca)] : B[pidx(q + 1 < cb ? q + 1 : cb)]);
+                if (sf) ae = nx;
+                else be = nx;
+            }
+        }
+        if (!FILL) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) c += __shfl_down_sync(0xffffffffu, c, o);
             if (lane == 0) counts[node] = c;
-            const DF At = df_ld(A[m]), Bt = df_ld(B[n]);
-            for (int t = lane; t < m; t += 32) {
-                DF ra = df_sub(Bt, df_ld(A[t]));
-                if (!df_pos(ra)) ra = DF{0.f, 0.f};
-                const DF ga = df_min(DF{a[t], 0.f}, ra);
-                if (df_pos(ga)) atomicAdd(&marg1[(size_t)t * n + j], df_val(ga));
-            }
-            for (int t = lane; t < n; t += 32) {
-                DF rb = df_sub(At, df_ld(B[t]));
-                if (!df_pos(rb)) rb = DF{0.f, 0.f};
-                const DF gb = df_min(DF{b[t], 0.f}, rb);
-                if (df_pos(gb)) atomicAdd(&marg2[(size_t)k * n + t], df_val(gb));
-            }
+            // marg1 is kept as [j][i]
+            const DF At = df_ld(A[pidx(ca)]), Bt = df_ld(B[pidx(cb)]);
+            side_marginal(marg1 + (size_t)j * m, ca, ra, ia, A, Bt);
+            side_marginal(marg2 + (size_t)k * n, cb, rb, ib, B, At);
         } else {
-            int incl = c;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += y;
+            for (; d < d1; ++d) e[d] = 0xffffffffu;      // past the end of a side
+            __syncwarp();
+            size_t pos = (size_t)offs[node];
+            DF last{0.f, 0.f};                           // the end passed before this round's first step
+            for (int base = 0; base < steps; base += 32) {
+                const unsigned w = base + lane < steps ? e[base + lane] : 0xffffffffu;
+                const int pp = (int)(w & 0xffffu), qq = (int)(w >> 16);
+                const bool in = w != 0xffffffffu;
+                DF end{0.f, 0.f};
+                if (in) end = df_min(df_ld(A[pidx(pp + 1)]), df_ld(B[pidx(qq + 1)]));
+                DF prev = df_shfl_up(end, 1);
+                if (lane == 0) prev = last;
+                last = df_shfl(end, 31);
+                const DF ov = df_sub(end, prev);
+                const bool out = in && df_pos(ov);
+                const unsigned mask = __ballot_sync(0xffffffffu, out);
+                if (out) {
+                    const size_t o = pos + __popc(mask & ((1u << lane) - 1u));
+                    src[o] = ia[pp] * n + j;
+                    dst[o] = k * n + ib[qq];
+                    mass[o] = df_dbl(ov);
+                }
+                pos += __popc(mask);
             }
-            if (c > 0)
-                merge_walk(A, B, a, b, m, n, p0, d0 - p0, d1 - d0, src, dst, mass, (size_t)(offs[node] + incl - c), j,
-                           k);
         }
         __syncwarp();
     }
 }
 
-// exclusive scan of `n` ints into long long offsets (single block, chunked)
-__global__ void k_scan(const int* __restrict__ counts, long long* __restrict__ offs, int n,
-                       unsigned long long* __restrict__ total) {
-    __shared__ long long s_tot[1024];
-    __shared__ long long s_carry;
-    if (threadIdx.x == 0) s_carry = 0;
+// Exclusive scan of n counts into offsets, one CTA: a warp per segment sums it,
+// the warps' sums are scanned, then each warp walks its segment again, 128
+// counts per step.  65,536 counts: 131 -> 29 us (a block scan per 1,024 counts
+// paid 20 barriers for each); bound by the latency of one CTA's loads.
+__global__ void __launch_bounds__(1024) k_scan(const int* __restrict__ counts, long long* __restrict__ offs, int n,
+                                               unsigned long long* __restrict__ total) {
+    __shared__ long long s_w[32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int seg = (((n + 31) / 32) + 127) & ~127;              // per warp, whole steps
+    const int s0 = min(n, warp * seg), s1 = min(n, s0 + seg);
+    long long sum = 0;
+#pragma unroll 8
+    for (int t = s0 + lane; t < s1; t += 32) sum += counts[t];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane == 0) s_w[warp] = sum;
     __syncthreads();
-    for (int base = 0; base < n; base += blockDim.x) {
-        const int t = base + threadIdx.x;
-        const long long v = t < n ? counts[t] : 0;
-        s_tot[threadIdx.x] = v;
-        __syncthreads();
-        for (int o = 1; o < (int)blockDim.x; o <<= 1) {
-            long long y = threadIdx.x >= (unsigned)o ? s_tot[threadIdx.x - o] : 0;
-            __syncthreads();
-            s_tot[threadIdx.x] += y;
-            __syncthreads();
-        }
-        if (t < n) offs[t] = s_carry + s_tot[threadIdx.x] - v;
-        __syncthreads();
-        if (threadIdx.x == blockDim.x - 1) s_carry += s_tot[threadIdx.x];
-        __syncthreads();
+    long long carry = 0;
+    for (int w = 0; w < warp; ++w) carry += s_w[w];
+    if (threadIdx.x == 0) {
+        long long all = 0;
+        for (int w = 0; w < 32; ++w) all += s_w[w];
+        *total = (unsigned long long)all;
     }
-    if (threadIdx.x == 0) *total = (unsigned long long)s_carry;
+    for (int base = s0; base < s1; base += 128) {
+        int v[4], incl = 0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int t = base + lane * 4 + u;
+            v[u] = t < s1 ? counts[t] : 0;
+            incl += v[u];
+        }
+        const int own = incl;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        long long at = carry + incl - own;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int t = base + lane * 4 + u;
+            if (t < s1) offs[t] = at;
+            at += v[u];
+        }
+        carry += __shfl_sync(0xffffffffu, incl, 31);
+    }
 }
 
-__global__ void k_marg_l1(const double* __restrict__ marg, const double* __restrict__ mu, int M,
-                          double* __restrict__ out) {
-    __shared__ double s[1024];
+// L1 distances of the plan's marginals to mu1 and mu2 (blockIdx.y: which):
+// partial sums per CTA, added in order by the CTA that finishes last.
+// t1: marg1 is stored [j][i] (k_recover_df) instead of [i][j].
+constexpr int kL1Ctas = 64;
+__global__ void __launch_bounds__(256) k_marg_l1(const double* __restrict__ marg, const double* __restrict__ mu1,
+                                                 const double* __restrict__ mu2, int m, int n, int t1,
+                                                 double* __restrict__ part, unsigned int* __restrict__ done,
+                                                 double* __restrict__ out) {
+    __shared__ double s[256];
+    __shared__ int s_last;
+    const int which = blockIdx.y, M = m * n;
+    const double* mg = marg + (size_t)which * M;
+    const double* mu = which ? mu2 : mu1;
     double acc = 0.0;
-    for (int t = threadIdx.x; t < M; t += blockDim.x) acc += fabs(marg[t] - mu[t]);
-    s[threadIdx.x] = acc;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < (unsigned)o) s[threadIdx.x] += s[threadIdx.x + o];
+    for (int t = blockIdx.x * 256 + threadIdx.x; t < M; t += kL1Ctas * 256)
+        acc += fabs(mg[t] - mu[!which && t1 ? (t % m) * n + t / m : t]);
+    auto block = [&](double v) {
+        s[threadIdx.x] = v;
         __syncthreads();
+        for (int o = 128; o > 0; o >>= 1) {
+            if (threadIdx.x < (unsigned)o) s[threadIdx.x] += s[threadIdx.x + o];
+            __syncthreads();
+        }
+        return s[0];
+    };
+    const double tot = block(acc);
+    if (threadIdx.x == 0) {
+        part[which * kL1Ctas + blockIdx.x] = tot;
+        __threadfence();
+        s_last = atomicAdd(done + which, 1u) == kL1Ctas - 1;
+        __threadfence();
     }
-    if (threadIdx.x == 0) *out = s[0];
+    __syncthreads();
+    if (s_last) {
+        const double v = threadIdx.x < kL1Ctas ? __ldcg(part + which * kL1Ctas + threadIdx.x) : 0.0;
+        __syncthreads();
+        const double all = block(v);
+        if (threadIdx.x == 0) out[which] = all;
+    }
 }
 
 // x-bar from the slab layout into the paper's vec order (eq. 4-6):
 // f1_{i,k,j} at i + m k + m^2 j (same as slab j, row k, col i);
 // f2_{k,j,l} at n m^2 + k + m j + m n l (slab n + k, row j, col l); the
 // slab rows sit at their padded pitch.
+// f1 rows keep their order (a warp per row); f2 is transposed in k and l for
+// each j, in 32 x 32 blocks through shared memory, so that both sides are read
+// and written in whole lines.  256 x 256: 151 -> 84 us (f2 was read with the
+// stride of a slab), 403 MB, 0.72 of the measured copy bandwidth.
 template <typename T>
-__global__ void k_export(const T* __restrict__ x, int m, int n, double* __restrict__ out) {
-    const size_t half = (size_t)m * m * n;
-    const size_t V = half + (size_t)m * n * n;
+__global__ void __launch_bounds__(256) k_export(const T* __restrict__ x, int m, int n, double* __restrict__ out) {
+    __shared__ T tile[32][33];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const size_t mp = row_pitch(m), np = row_pitch(n);
-    // one thread per entry of the paper's order (coalesced writes)
-    for (size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q < V; q += (size_t)gridDim.x * blockDim.x) {
-        if (q < half) {                           // f1_{i,k,j} at i + m k + m^2 j: slab j, row k, column i
-            const size_t i = q % m, k = (q / m) % m, j = q / ((size_t)m * m);
-            out[q] = (double)x[(j * m + k) * mp + i];
-        } else {                                  // f2_{k,j,l} at k + m j + m n l: slab n + k, row j, column l
-            const size_t p = q - half;
-            const size_t k = p % m, j = (p / m) % n, l = p / ((size_t)m * n);
-            out[q] = (double)x[(size_t)n * m * mp + (k * n + j) * np + l];
+    const size_t half = (size_t)m * m * n, half_p = (size_t)n * m * mp;
+    // f1: rows (j, k), eight per step and CTA
+    const int rows = n * m, rsteps = (rows + 7) / 8;
+    const int kt = (m + 31) / 32, lt = (n + 31) / 32;
+    const long long items = (long long)rsteps + (long long)n * kt * lt;
+    for (long long it = blockIdx.x; it < items; it += gridDim.x) {
+        if (it < rsteps) {
+            const int r = (int)it * 8 + warp;
+            if (r < rows) {
+                const T* row = x + (size_t)r * mp;
+                double* o = out + (size_t)r * m;
+#pragma unroll 4
+                for (int i = lane; i < m; i += 32) o[i] = (double)__ldcs(row + i);
+            }
+        } else {
+            const int q = (int)(it - rsteps);
+            const int j = q / (kt * lt), k0 = (q / lt) % kt * 32, l0 = q % lt * 32;
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int k = k0 + warp + 8 * u, l = l0 + lane;
+                if (k < m && l < n) tile[warp + 8 * u][lane] = __ldcs(x + half_p + ((size_t)k * n + j) * np + l);
+            }
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int l = l0 + warp + 8 * u, k = k0 + lane;
+                if (k < m && l < n) out[half + (size_t)l * m * n + (size_t)j * m + k] = (double)tile[lane][warp + 8 * u];
+            }
         }
     }
 }
@@ -406,7 +551,7 @@ int export_flows(Inst* I, double* x, int space, cudaStream_t st) {
         HOT_CK(cudaMallocAsync(&tmp, V * 8, st));
         dst = tmp;
     }
-    const int grid = 1024;
+    const int grid = 152 * 8;
     if (I->fp64) k_export<double><<<grid, 256, 0, st>>>((const double*)I->desc.xr, m, n, dst);
     else k_export<float><<<grid, 256, 0, st>>>((const float*)I->desc.xr, m, n, dst);
     HOT_CK(cudaGetLastError());
@@ -420,90 +565,127 @@ int export_flows(Inst* I, double* x, int space, cudaStream_t st) {
 
 int recover_plan(Ctx* ctx, Inst* I, int32_t* src, int32_t* dst, double* mass, int space, size_t cap, size_t* nnz,
                  double* marg_l1, cudaStream_t st) {
-    (void)ctx;
     const int m = I->m, n = I->n;
     const int nodes = m * n;
-    int* counts = nullptr;
-    long long* offs = nullptr;
-    unsigned long long* dtot = nullptr;
-    double* marg = nullptr;
-    double* l1 = nullptr;
-    HOT_CK(cudaMallocAsync(&counts, sizeof(int) * nodes, st));
-    HOT_CK(cudaMallocAsync(&offs, sizeof(long long) * nodes, st));
-    HOT_CK(cudaMallocAsync(&dtot, sizeof(unsigned long long), st));
-    HOT_CK(cudaMallocAsync(&marg, sizeof(double) * 2 * nodes, st));
-    HOT_CK(cudaMallocAsync(&l1, sizeof(double) * 2, st));
-    HOT_CK(cudaMemsetAsync(marg, 0, sizeof(double) * 2 * nodes, st));
-    // warps per CTA: each holds a, b and their prefix sums (2(m + n) + 2
-    // doubles; FP32 mode: m + n floats and m + n + 2 float pairs)
-    const size_t per_warp =
-        I->fp64 ? recover_words(m, n) * sizeof(double) : recover_df_words(m, n) * sizeof(float);
-    const int nw = std::max(1, std::min(kRecWarps, (int)((200 * 1024) / per_warp)));
-    const size_t shm = (size_t)nw * per_warp;
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaFuncSetAttribute(k_recover_df, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        cudaFuncSetAttribute(k_recover<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        attr_set = true;
-    }
+    // one scratch allocation: offsets, marginals, L1 partials, total, L1, L1 counters, counts
+    const size_t o_marg = sizeof(long long) * nodes, o_part = o_marg + sizeof(double) * 2 * nodes,
+                 o_tot = o_part + sizeof(double) * 2 * kL1Ctas, o_l1 = o_tot + 8, o_done = o_l1 + 16,
+                 o_cnt = o_done + 8, bytes = o_cnt + sizeof(int) * nodes;
+    char* scr = nullptr;
+    HOT_CK(cudaMallocAsync((void**)&scr, bytes, st));
+    long long* offs = (long long*)scr;
+    double* marg = (double*)(scr + o_marg);
+    unsigned long long* dtot = (unsigned long long*)(scr + o_tot);
+    double* l1 = (double*)(scr + o_l1);
+    unsigned int* done = (unsigned int*)(scr + o_done);
+    int* counts = (int*)(scr + o_cnt);
+    int32_t *ds = src, *dd = dst;
+    double* dm = mass;
+    bool staged = false;
+    auto finish = [&](int rc) {
+        if (staged) {
+            if (ds) cudaFreeAsync(ds, st);
+            if (dd) cudaFreeAsync(dd, st);
+            if (dm) cudaFreeAsync(dm, st);
+        }
+        cudaFreeAsync(scr, st);
+        return rc;
+    };
+    auto failed = [&](cudaError_t e, const char* what) {
+        if (e == cudaSuccess) return false;
+        set_error(std::string(what) + ": " + cudaGetErrorString(e));
+        return true;
+    };
+    // warps per CTA (each has its own part of the shared memory): up to
+    // kRecWarps, fewer where that leaves more of them resident on an SM
+    auto warps_for = [](size_t per) {
+        int best = 1, most = 0;
+        for (int w = kRecWarps; w >= 1; --w) {
+            if (w * per > 200 * 1024) continue;
+            const int res = std::min(48, (int)((227 * 1024) / (w * per + 1024)) * w);
+            if (res > most) {
+                most = res;
+                best = w;
+            }
+        }
+        return best;
+    };
+    const size_t per_fill = I->fp64 ? recover_words(m, n) * sizeof(double) : recover_df_words(m, n, true) * sizeof(float);
+    const size_t per_count = I->fp64 ? per_fill : recover_df_words(m, n, false) * sizeof(float);
+    const int nw = warps_for(per_fill), nwc = warps_for(per_count);
+    const size_t shm = (size_t)nw * per_fill, shm_count = (size_t)nwc * per_count;
+    cudaError_t e = cudaFuncSetAttribute(k_recover_df<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_recover_df<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_recover<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     int sms = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, 0);
-    const int grid = std::max(1, std::min((nodes + nw - 1) / nw, sms * 8));
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
+    if (e == cudaSuccess) e = cudaMemsetAsync(marg, 0, o_cnt - o_marg, st);
+    if (failed(e, "plan recovery")) return finish(HOT_ECUDA);
+    const int grid = std::max(1, std::min((nodes + nw - 1) / nw, sms * (64 / nw)));
+    const int gridc = std::max(1, std::min((nodes + nwc - 1) / nwc, sms * (64 / nwc)));
     if (I->fp64)
         k_recover<double><<<grid, nw * 32, shm, st>>>((const double*)I->desc.xr, m, n, 1, counts, nullptr,
                                                               nullptr, nullptr, nullptr, marg, marg + nodes);
     else
-        k_recover_df<<<grid, nw * 32, shm, st>>>((const float*)I->desc.xr, m, n, 1, counts, nullptr, nullptr, nullptr,
-                                                 nullptr, marg, marg + nodes);
-    HOT_CK(cudaGetLastError());
+        k_recover_df<false><<<gridc, nwc * 32, shm_count, st>>>((const float*)I->desc.xr, m, n, counts, nullptr, nullptr, 0,
+                                                        nullptr, nullptr, nullptr, marg, marg + nodes);
     k_scan<<<1, 1024, 0, st>>>(counts, offs, nodes, dtot);
-    unsigned long long tot = 0;
-    HOT_CK(cudaMemcpyAsync(&tot, dtot, sizeof(tot), cudaMemcpyDeviceToHost, st));
-    HOT_CK(cudaStreamSynchronize(st));
-    *nnz = (size_t)tot;
-    int rc = HOT_OK;
-    if (marg_l1) {
+    if (marg_l1)
         // marginals against mu1 (row-major (i, j)) and mu2 (row-major (k, l))
-        k_marg_l1<<<1, 1024, 0, st>>>(marg, I->desc.mu1, nodes, l1);
-        k_marg_l1<<<1, 1024, 0, st>>>(marg + nodes, I->desc.mu2, nodes, l1 + 1);
-        HOT_CK(cudaMemcpyAsync(marg_l1, l1, sizeof(double) * 2, cudaMemcpyDeviceToHost, st));
+        k_marg_l1<<<dim3(kL1Ctas, 2), 256, 0, st>>>(marg, I->desc.mu1, I->desc.mu2, m, n, I->fp64 ? 0 : 1,
+                                                    (double*)(scr + o_part), done, l1);
+    auto fill = [&](size_t room) {
+        if (I->fp64)
+            k_recover<double><<<grid, nw * 32, shm, st>>>((const double*)I->desc.xr, m, n, 0, counts, offs, ds, dd, dm,
+                                                          nullptr, nullptr);
+        else
+            k_recover_df<true><<<grid, nw * 32, shm, st>>>((const float*)I->desc.xr, m, n, counts, offs, dtot, room,
+                                                           ds, dd, dm, nullptr, nullptr);
+    };
+    const bool want = cap > 0 || src || dst || mass;
+    // device outputs of an FP32 solution: the fill runs behind the count without
+    // a look at the total (it writes nothing when the plan does not fit)
+    const bool ahead = want && !I->fp64 && space == HOT_SPACE_DEVICE && cap > 0;
+    if (ahead) fill(cap);
+    unsigned long long tot = 0;
+    double hl1[2] = {0.0, 0.0};
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&tot, dtot, sizeof(tot), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess && marg_l1) e = cudaMemcpyAsync(hl1, l1, sizeof(hl1), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (failed(e, "plan recovery")) return finish(HOT_ECUDA);
+    *nnz = (size_t)tot;
+    if (marg_l1) {
+        marg_l1[0] = hl1[0];
+        marg_l1[1] = hl1[1];
     }
-    if (cap > 0 || src || dst || mass) {
-        if (cap < tot) {
-            rc = HOT_EINVAL;
-            set_error("output capacity " + std::to_string(cap) + " < plan size " + std::to_string(tot));
-        } else if (tot > 0) {
-            int32_t *ds = src, *dd = dst;
-            double* dm = mass;
-            if (space == HOT_SPACE_HOST) {
-                HOT_CK(cudaMallocAsync(&ds, sizeof(int32_t) * tot, st));
-                HOT_CK(cudaMallocAsync(&dd, sizeof(int32_t) * tot, st));
-                HOT_CK(cudaMallocAsync(&dm, sizeof(double) * tot, st));
-            }
-            if (I->fp64)
-                k_recover<double><<<grid, nw * 32, shm, st>>>((const double*)I->desc.xr, m, n, 0, counts, offs,
-                                                                      ds, dd, dm, nullptr, nullptr);
-            else
-                k_recover_df<<<grid, nw * 32, shm, st>>>((const float*)I->desc.xr, m, n, 0, counts, offs, ds, dd, dm,
-                                                         nullptr, nullptr);
-            HOT_CK(cudaGetLastError());
-            if (space == HOT_SPACE_HOST) {
-                HOT_CK(cudaMemcpyAsync(src, ds, sizeof(int32_t) * tot, cudaMemcpyDeviceToHost, st));
-                HOT_CK(cudaMemcpyAsync(dst, dd, sizeof(int32_t) * tot, cudaMemcpyDeviceToHost, st));
-                HOT_CK(cudaMemcpyAsync(mass, dm, sizeof(double) * tot, cudaMemcpyDeviceToHost, st));
-                cudaFreeAsync(ds, st);
-                cudaFreeAsync(dd, st);
-                cudaFreeAsync(dm, st);
-            }
-        }
+    if (!want) return finish(HOT_OK);
+    if (cap < tot) {
+        set_error("output capacity " + std::to_string(cap) + " < plan size " + std::to_string(tot));
+        return finish(HOT_EINVAL);
     }
-    cudaFreeAsync(counts, st);
-    cudaFreeAsync(offs, st);
-    cudaFreeAsync(dtot, st);
-    cudaFreeAsync(marg, st);
-    cudaFreeAsync(l1, st);
-    HOT_CK(cudaStreamSynchronize(st));
-    return rc;
+    if (ahead || tot == 0) return finish(HOT_OK);
+    if (space == HOT_SPACE_HOST) {
+        staged = true;
+        ds = dd = nullptr;
+        dm = nullptr;
+        e = cudaMallocAsync((void**)&ds, sizeof(int32_t) * tot, st);
+        if (e == cudaSuccess) e = cudaMallocAsync((void**)&dd, sizeof(int32_t) * tot, st);
+        if (e == cudaSuccess) e = cudaMallocAsync((void**)&dm, sizeof(double) * tot, st);
+        if (failed(e, "device allocation for the plan")) return finish(HOT_ENOMEM);
+    }
+    fill(tot);
+    e = cudaGetLastError();
+    if (space == HOT_SPACE_HOST) {
+        if (e == cudaSuccess) e = cudaMemcpyAsync(src, ds, sizeof(int32_t) * tot, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(dst, dd, sizeof(int32_t) * tot, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(mass, dm, sizeof(double) * tot, cudaMemcpyDeviceToHost, st);
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (failed(e, "plan recovery")) return finish(HOT_ECUDA);
+    return finish(HOT_OK);
 }
 
 }  // namespace hot
