@@ -425,6 +425,7 @@ int inst_create(const PairHost& p, int fp64, const hot_config& cfg, double tol, 
     c.rprev = -1.0;
     c.max_iter = max_iter;
     c.status = ST_RUNNING;
+    c.dzero = fp64 ? 0 : 1;      // the delta starts at zero, not stored in FP32 mode
     I->ctl_host = c;
 
     cudaError_t ee = cudaMemsetAsync(sm, 0, o_zero_end, st);
@@ -465,7 +466,7 @@ int inst_create(const PairHost& p, int fp64, const hot_config& cfg, double tol, 
         // pageable sources: the copies are staged before cudaMemcpyAsync returns
     }
     if (ee == cudaSuccess) {
-        launch_init(d, c.sigma, st);   // u = -sigma0 c (w0 = 0), delta and restart references 0
+        launch_init(d, c.sigma, st);   // u = -sigma0 c (w0 = 0)
         ee = cudaGetLastError();
     }
     // the staging vectors above are pageable: cudaMemcpyAsync from pageable

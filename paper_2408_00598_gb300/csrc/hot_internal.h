@@ -72,7 +72,7 @@ struct HotCtl {
     int just_finished;     // set at the check that ends the solve
     int cancel;            // host asks the instance to stop at the next check
     unsigned int ymax_bits;// max |alpha|, |beta| (float bits, scaled units)
-    int dzero;             // FP32: a restart left the delta zero (not stored); the
+    int dzero;             // FP32: the start or a restart left the delta zero (not stored); the
                            // next block's first sweep reads no d (cleared at the check)
 };
 
@@ -290,7 +290,7 @@ cudaError_t group_init();
 LaunchDims make_launch_dims(int device, int fp64);
 // resident CTAs of the (non-check) sweep on the current device
 int sweep_grid(int fp64);
-// u = -sigma0 c, d = 0, x_r = z_r = 0 and the FP64 sums of u for a new instance
+// u = -sigma0 c and its FP64 sums for a new instance (FP64 mode: also d0 = 0)
 // (the initial point w0 = 0: v0 = 0, y0 = 0).
 void launch_init(const HotInst& I, double sigma0, cudaStream_t st);
 cudaError_t kernels_init(int device);

@@ -1123,6 +1123,7 @@ __device__ __forceinline__ void restart_tile(const HotInst& I, int slab, int ban
     // k_restart_sigma has replaced it (kept in sigma_old)
     const double sig_old = (MODE == 1) ? I.ctl->sigma_old : I.ctl->sigma;
     const double sig_new = I.ctl->sigma;
+    const bool origin = I.ctl->restarts == 0;        // MODE 0: the reference point is still w0 = 0 (not stored)
     const int c0 = cg * NV;
     const int nval = S - c0;                         // columns inside the slab (pad columns after)
     const int cr = F32 ? I.coord_real : 0;           // real-valued coordinates: the cost term in pairs
@@ -1197,8 +1198,13 @@ __device__ __forceinline__ void restart_tile(const HotInst& I, int slab, int ban
                 if (e >= nval) xbv[e] = zbv[e] = rv[e] = T(0);   // pad columns: zero in every array
             if constexpr (MODE == 0) {
                 T xo[NV], zo[NV];
-                V::ld(xr + (size_t)r * Sp + c0, xo);
-                V::ld(zr + (size_t)r * Sp + c0, zo);
+                if (origin) {
+#pragma unroll
+                    for (int e = 0; e < NV; ++e) xo[e] = zo[e] = T(0);
+                } else {
+                    V::ld(xr + (size_t)r * Sp + c0, xo);
+                    V::ld(zr + (size_t)r * Sp + c0, zo);
+                }
 #pragma unroll
                 for (int e = 0; e < NV; ++e) {
                     if constexpr (F32) {
@@ -1380,8 +1386,13 @@ __global__ void __launch_bounds__(kThreads, 3) k_restart(const WorkDev* __restri
 }
 
 // Initial point w0 = 0 of a new instance: v0 = 0 and y0 = 0, so
-// u = v0 - sigma0 (c - A^T y0) = -sigma0 c; d = 0; x_r = z_r = 0; FP64 slab
-// sums of u.  One launch per instance (descriptor by value).
+// u = v0 - sigma0 (c - A^T y0) = -sigma0 c, with its sums in FP64.  The cost is
+// the same in every slab of a half: k_init forms the first slab of each, and
+// k_init_copy repeats it (FP64 arithmetic on every element, at a 64th of the
+// FP32 rate, took most of the set-up).  d = 0 and x_r = z_r = 0 are not stored:
+// the first sweep takes the delta as zero (HotCtl::dzero; FP64 mode clears d0)
+// and the first restart the reference point (restart_tile).  256 x 256: 549 us,
+// 537 MB written -> 45 + 25 us, 134 MB.  One launch per instance (descriptor by value).
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_init(HotInst I, double sigma0) {
     using V = VecT<T>;
@@ -1390,9 +1401,8 @@ __global__ void __launch_bounds__(kThreads) k_init(HotInst I, double sigma0) {
     __shared__ double s_col[kThreads * 4];
     __shared__ double s_red[32];
     const int TR = I.TR;
-    for (int t = blockIdx.x; t < g_ntiles(I); t += gridDim.x) {
-        int slab, band;
-        g_tile_slab(I, t, slab, band);
+    for (int t = blockIdx.x; t < I.nb1 + I.nb2; t += gridDim.x) {
+        const int slab = t < I.nb1 ? 0 : I.n, band = t < I.nb1 ? t : t - I.nb1;
         const int S = g_side(I, slab), Sp = g_pitch(I, slab);   // this slab's side and row pitch
         const int NC = Sp / NV;
         const int P = kThreads / NC;
@@ -1411,7 +1421,7 @@ __global__ void __launch_bounds__(kThreads) k_init(HotInst I, double sigma0) {
         }
         if (active) {
             for (int r = r0 + ro; r < r1; r += P) {
-                T uu[NV], zero[NV];
+                T uu[NV];
                 DF rsf{0.f, 0.f};
                 double rs = 0.0;
 #pragma unroll
@@ -1420,7 +1430,6 @@ __global__ void __launch_bounds__(kThreads) k_init(HotInst I, double sigma0) {
                     const bool v = c0 + e < S;                 // pad columns: 0
                     const double dc = v ? I.X64[xb0 + r] - I.X64[xb0 + c0 + e] : 0.0;
                     uu[e] = v ? (T)(-sigma0 * (dc * dc * I.h)) : T(0);
-                    zero[e] = T(0);
                     if constexpr (std::is_same<T, float>::value) {
                         rsf = df_add(rsf, (float)uu[e]);
                         fcol[e] = df_add(fcol[e], (float)uu[e]);
@@ -1438,9 +1447,6 @@ __global__ void __launch_bounds__(kThreads) k_init(HotInst I, double sigma0) {
                 }
                 if constexpr (std::is_same<T, float>::value) rs = df_val(rsf);
                 V::st((T*)I.u + off + (size_t)r * Sp + c0, uu);
-                V::st((T*)I.d0 + off + (size_t)r * Sp + c0, zero);
-                V::st((T*)I.xr + off + (size_t)r * Sp + c0, zero);
-                V::st((T*)I.zr + off + (size_t)r * Sp + c0, zero);
                 s_row[(r - r0) * NC + cg] = rs;
             }
         }
@@ -1462,6 +1468,31 @@ __global__ void __launch_bounds__(kThreads) k_init(HotInst I, double sigma0) {
             if (threadIdx.x == 0) reinterpret_cast<float2*>(I.cu_part)[g_tile(I, slab, band)] = df_st(cu[0]);
         }
         __syncthreads();
+    }
+}
+
+// The first slab of each half (k_init) repeated into the others: blockIdx.y the
+// slab, blockIdx.x a part of it; the slab's sums with part 0.
+constexpr int kCopyPart = 16;               // 16-byte words per thread
+template <typename T>
+__global__ void __launch_bounds__(kThreads) k_init_copy(HotInst I) {
+    const int slab = blockIdx.y, first = slab < I.n ? 0 : I.n;
+    if (slab == first) return;
+    const int S = g_side(I, slab), nb = g_nb(I, slab);
+    const size_t words = (size_t)S * g_pitch(I, slab) * sizeof(T) / 16;
+    const float4* __restrict__ src = reinterpret_cast<const float4*>((const T*)I.u + g_elem(I, first));
+    float4* __restrict__ dst = reinterpret_cast<float4*>((T*)I.u + g_elem(I, slab));
+    const size_t q0 = (size_t)blockIdx.x * kThreads * kCopyPart + threadIdx.x;
+#pragma unroll 4
+    for (int u = 0; u < kCopyPart; ++u) {
+        const size_t q = q0 + (size_t)u * kThreads;
+        if (q < words) __stcs(dst + q, src[q]);
+    }
+    if (blockIdx.x == 0) {
+        for (int q = threadIdx.x; q < S; q += kThreads) I.rs0[g_row(I, slab) + q] = I.rs0[g_row(I, first) + q];
+        for (int q = threadIdx.x; q < S * nb; q += kThreads)
+            I.cs0_part[g_colp(I, slab, 0) + q] = I.cs0_part[g_colp(I, first, 0) + q];
+        for (int q = threadIdx.x; q < nb; q += kThreads) I.cu_part[g_tile(I, slab, q)] = I.cu_part[g_tile(I, first, q)];
     }
 }
 
@@ -1824,10 +1855,17 @@ void launch_init(const HotInst& I, double sigma0, cudaStream_t st) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int tiles = g_ntiles(I);
-    const int grid = tiles < sms * 4 ? tiles : sms * 4;
-    if (I.fp64) k_init<double><<<grid, kThreads, 0, st>>>(I, sigma0);
-    else k_init<float><<<grid, kThreads, 0, st>>>(I, sigma0);
+    const int L = g_L(I), Lp = (L + 3) & ~3;
+    const size_t words = (size_t)L * Lp * (I.fp64 ? 8 : 4) / 16;               // of the larger slab
+    const dim3 copy((unsigned)((words + kThreads * kCopyPart - 1) / (kThreads * kCopyPart)), (unsigned)g_nslab(I));
+    if (I.fp64) {
+        k_init<double><<<I.nb1 + I.nb2, kThreads, 0, st>>>(I, sigma0);
+        k_init_copy<double><<<copy, kThreads, 0, st>>>(I);
+        cudaMemsetAsync(I.d0, 0, g_state_len(I) * sizeof(double), st);
+    } else {
+        k_init<float><<<I.nb1 + I.nb2, kThreads, 0, st>>>(I, sigma0);
+        k_init_copy<float><<<copy, kThreads, 0, st>>>(I);
+    }
     k_anchor_one<<<g_nslab(I) < sms * 4 ? g_nslab(I) : sms * 4, kThreads, 0, st>>>(I, sigma0);
 }
 
