@@ -249,7 +249,7 @@ int inst_create(const PairHost& p, int fp64, const hot_config& cfg, double tol, 
     const size_t o_rs2b = take(2 * MN * F2);
     const size_t o_cs32b = fp64 ? 0 : take(CP * 4);
     const size_t o_tp = fp64 ? 0 : take((size_t)NS * sizeof(float4));
-    const size_t o_gcount = fp64 ? 0 : take(sizeof(unsigned int));
+    const size_t o_gcount = fp64 ? 0 : take(2 * sizeof(unsigned int));
     const size_t o_vcnt = take(sizeof(unsigned int));
     const size_t o_zero_end = off;                 // everything above starts at 0
     const size_t o_mu1f = take(MN * F2);
@@ -584,8 +584,7 @@ int Batch::set_instances(const std::vector<Inst*>& v, cudaStream_t st, bool grou
     int* pv = h_pre + 2 * (cap + 1);
     int* pk = h_pre + 3 * (cap + 1);
     int* pa = h_pre + 4 * (cap + 1);
-    int* pw = h_pre + 5 * (cap + 1);
-    pt[0] = ps[0] = pv[0] = pk[0] = pa[0] = pw[0] = 0;
+    pt[0] = ps[0] = pv[0] = pk[0] = pa[0] = 0;
     int running = 0;
     size_t swept = 0;                 // bytes one sweep of the chain streams: u, d read, d written
     n_group = n_chain = 0;
@@ -617,11 +616,10 @@ int Batch::set_instances(const std::vector<Inst*>& v, cudaStream_t st, bool grou
             pad |= odd;
             swept += 3 * (v[i]->big_bytes / 5);
         }
-        pt[i + 1] = pt[i] + tiles;
-        pw[i + 1] = pw[i] + (g ? 0 : tiles);
-        ps[i + 1] = ps[i] + m + nn;
+        pt[i + 1] = pt[i] + (g ? 0 : tiles);
+        ps[i + 1] = ps[i] + (g ? 0 : m + nn);
         pv[i + 1] = pv[i] + (g ? 0 : v[i]->fp64 ? 2 * (m + nn) : vec32_items(m, nn));
-        pk[i + 1] = pk[i] + v[i]->n_k1 + (g ? v[i]->desc.n_achunk : 0);
+        pk[i + 1] = pk[i] + (g ? 0 : v[i]->n_k1);
         pa[i + 1] = pa[i] + (g ? 0 : v[i]->desc.n_achunk);
         if (v[i]->ctl_host.status == ST_RUNNING) ++running;
     }
@@ -640,7 +638,6 @@ int Batch::set_instances(const std::vector<Inst*>& v, cudaStream_t st, bool grou
     h_work->pre_vec = d_pre + 2 * (cap + 1);
     h_work->pre_k1 = d_pre + 3 * (cap + 1);
     h_work->pre_achunk = d_pre + 4 * (cap + 1);
-    h_work->pre_swp = d_pre + 5 * (cap + 1);
     h_work->gstart = d_gstart;
     h_work->gent = d_gent;
     h_work->n_running = d_running;
@@ -667,14 +664,14 @@ int Batch::set_instances(const std::vector<Inst*>& v, cudaStream_t st, bool grou
 }
 
 int Batch::launches() const {
-    return (n_group > 0 ? 1 : 0) + (n_chain > 0 ? launches_per_block(fp64, K, n_chain == 1) : 0) + kLaunchesBlockEnd;
+    return (n_group > 0 ? 1 : 0) + (n_chain > 0 ? launches_per_block(fp64, K, n_chain == 1) + kLaunchesBlockEnd : 0);
 }
 
 // The K iterations of a block: k_group32 for the grouped instances, the chain
 // of kernels for the others; with ev, an event pair around the sweep of
 // iteration timed_iter().
 void Batch::launch_iterations(cudaStream_t st, cudaEvent_t* ev) const {
-    if (n_group > 0) launch_group(d_work, ggrid, K, gpad != 0, st);
+    if (n_group > 0) launch_group(d_work, ggrid, K, group_blocks(), a1, a2, a3, gpad != 0, st);
     if (n_chain == 0) return;
     for (int j = 0; j < K; ++j) {
         launch_solve_kernels(d_work, ld, fp64, j, j == K - 1, n_chain == 1, st);
@@ -690,7 +687,7 @@ void Batch::launch_iterations(cudaStream_t st, cudaEvent_t* ev) const {
 int Batch::capture(cudaGraphExec_t* out, cudaEvent_t* ev) {
     HOT_CK(cudaStreamBeginCapture(cap_stream, cudaStreamCaptureModeThreadLocal));
     launch_iterations(cap_stream, ev);
-    launch_block_end(d_work, ld, fp64, K, a1, a2, a3, cap_stream);
+    if (n_chain > 0) launch_block_end(d_work, ld, fp64, K, a1, a2, a3, cap_stream);
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamEndCapture(cap_stream, &g);
     if (e != cudaSuccess) {
@@ -825,7 +822,7 @@ int run_solve(Ctx* ctx, const std::vector<PairHost>& pairs, double tol, long lon
     // finished pairs from the tables as they go, see below)
     std::vector<int> live(insts.size());
     for (size_t q = 0; q < insts.size(); ++q) live[q] = (int)q;
-    long long launches = 0;
+    long long launches = 0, blocks = 0;
     const auto th0 = std::chrono::steady_clock::now();
     auto note_finished = [&](const int* sts) {
         const double now = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - th0).count();
@@ -840,6 +837,7 @@ int run_solve(Ctx* ctx, const std::vector<PairHost>& pairs, double tol, long lon
                 break;
             }
             launches += B.launches();
+            blocks += B.group_blocks();
             cudaMemcpyAsync((void*)B.running(nb), B.d_running, 2 * sizeof(int), cudaMemcpyDeviceToHost, st);
             if (track)
                 cudaMemcpyAsync(B.h_stb + (size_t)(nb & 1) * B.cap, B.d_st, sizeof(int) * live.size(),
@@ -978,7 +976,10 @@ int run_solve(Ctx* ctx, const std::vector<PairHost>& pairs, double tol, long lon
         cleanup();
         return HOT_ECUDA;
     }
-    if (kt) launches = nb * B.launches();
+    if (kt) {
+        launches = nb * B.launches();
+        blocks = nb;
+    }
     for (size_t q = 0; q < insts.size(); ++q) {
         Inst* I = insts[q];
         cudaMemcpy(&I->ctl_host, I->desc.ctl, sizeof(HotCtl), cudaMemcpyDeviceToHost);
@@ -987,7 +988,7 @@ int run_solve(Ctx* ctx, const std::vector<PairHost>& pairs, double tol, long lon
         // the start of the batch); a single solve the device time of the solve
         out[q].solve_ms = track ? (fin_ms[q] >= 0.0 ? fin_ms[q] : (double)ms) : ms;
         out[q].kernel_launches = launches;
-        out[q].blocks = nb;
+        out[q].blocks = blocks;
         if (keep) {
             const unsigned long long id = ctx->next_id++;
             ctx->solutions[id].inst = I;

@@ -71,8 +71,8 @@ int inst_create(const PairHost& p, int fp64, const hot_config& cfg, double tol, 
 void inst_destroy(Inst* I, cudaStream_t st);
 
 // Device work tables plus the instantiated block graph that reads them.
-// Prefix tables (cap + 1 ints each): tiles, slabs, k_vec items, k_kkt1 chunks, k_alpha32 chunks, sweep tiles.
-constexpr int kPreTables = 6;
+// Prefix tables (cap + 1 ints each): tiles, slabs, k_vec items, k_kkt1 chunks, k_alpha32 chunks.
+constexpr int kPreTables = 5;
 // CTAs of k_group32 for the grouped instances of a batch, by a cost model of
 // one iteration: entries (instance, rank, group size) per CTA.
 struct GroupPlan {
@@ -119,6 +119,8 @@ struct Batch {
     // some instance of that kind needs the general sweep: a side that is not
     // a multiple of 4, or (FP32) real-valued bin coordinates
     int n_group = 0, n_chain = 0;
+    int max_group_blocks = 4;       // check blocks per launch of k_group32 when it runs alone (the host looks in between)
+    int group_blocks() const { return n_chain > 0 ? 1 : max_group_blocks; }
     int pad = 0, gpad = 0;
     int shape() const {             // what a captured graph depends on
         return (n_group > 0) | (n_chain > 0) << 1 | (n_chain == 1) << 2 | (pad != 0) << 3 | (gpad != 0) << 4;

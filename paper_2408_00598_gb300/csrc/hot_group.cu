@@ -22,7 +22,7 @@
 // The groups of one launch are independent.  The grid is launched
 // cooperatively, so that the CTAs of a group are resident together; every
 // wait is bounded and sets W->err when it runs out.
-#include "hot_dev.cuh"
+#include "hot_block.cuh"
 
 namespace hot {
 
@@ -65,18 +65,20 @@ struct GroupSmem {
     // (mvA, sy) of column j at j, (mvS, sp) of row k at n + k
     float4 vec[2 * kMaxGroupSide];
     float2 mar[2 * kMaxGroupSide];        // column totals of mu (cm2), row totals of nu (rm2)
-    float2 red[(kNK - 1) * 32];
+    float2 red[8 * 32];                   // block sums, up to eight at once (check_instance)
     HotInst I;
     CycleK C;
     GTile tile[kTileTable];
     StageK K;
+    PieceK PK;
+    DF F[2];                              // half totals
     DF sm1, sm2;                          // the marginals' sums
     P32 p[64];                            // of every iteration of the block (check_every <= 64)
     int dead;
 };
 
 // All CTAs of the group have arrived for the `epoch`-th time in this launch
-// (k_block_end clears the counter).  One thread per CTA arrives with a release
+// (the last CTA to leave clears the counter).  One thread per CTA arrives with a release
 // and polls with an acquire: 2,300 cycles with 32 CTAs, 2,800 with 304 (a flag
 // per CTA polled by whole warps took 2,000 and 8,200: the polls hold up the
 // arrivals).  The barrier at the top orders the CTA's writes before thread 0's
@@ -162,37 +164,42 @@ __device__ __forceinline__ DF slab_sum(const HotInst& I, const float2* __restric
     return c;
 }
 
-// Half totals F1, F2 (the order of k_vec32's item totals and alpha32_stage's
-// block sum: the items of 8 slabs left to right, the shuffle tree over 32
-// items, then the warps' totals) and the stage's scalars, by one warp.
-__device__ __forceinline__ void group_stage(GroupSmem& s, float kdl, int lane) {
+// Half total F1 (half 0: the f1 slabs' T) or F2 by one warp each, in the order
+// of k_vec32's item totals and alpha32_stage's block sum: the items of 8 slabs
+// left to right, the shuffle tree over 32 items (the f2 items after the f1
+// ones), then the warps' totals.
+__device__ __forceinline__ void group_half_total(GroupSmem& s, int half, int lane) {
     const int m = s.I.m, n = s.I.n;
     const int t1 = (n + 7) / 8, t2 = (m + 7) / 8;                 // t1 + t2 <= 64
-    DF F1{0.f, 0.f}, F2{0.f, 0.f};
+    const int cnt = half ? m : n;
+    const float4* tp = s.vec + (half ? n : 0);
+    DF F{0.f, 0.f};
 #pragma unroll 1
     for (int q = lane; q - lane < t1 + t2; q += 32) {
-        DF a{0.f, 0.f}, b{0.f, 0.f};
-        const bool first = q < t1;
-        const int s0 = (first ? q : q - t1) * 8, cnt = first ? n : m;
-        const float4* tp = s.vec + (first ? 0 : n);
-        DF tot{0.f, 0.f};
-#pragma unroll 1
-        for (int w = 0; w < 8; ++w)
-            if (s0 + w < cnt) tot = df_add(tot, DF{tp[s0 + w].x, tp[s0 + w].y});
-        if (first) a = tot;
-        else b = tot;
-#pragma unroll 1
-        for (int o = 16; o > 0; o >>= 1) {
-            a = df_add(a, df_shfl_down(a, o));
-            b = df_add(b, df_shfl_down(b, o));
+        const int item = half ? q - t1 : q;
+        const int s0 = item * 8;
+        float2 v[8];
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+            const bool in = item >= 0 && s0 + w < cnt;
+            const float4 t = in ? tp[s0 + w] : make_float4(0.f, 0.f, 0.f, 0.f);
+            v[w] = make_float2(t.x, t.y);
         }
-        F1 = df_add(F1, a);
-        F2 = df_add(F2, b);
+        DF a = df_ld(v[0]);
+#pragma unroll
+        for (int w = 1; w < 8; ++w) a = df_add(a, df_ld(v[w]));
+#pragma unroll 1
+        for (int o = 16; o > 0; o >>= 1) a = df_add(a, df_shfl_down(a, o));
+        F = df_add(F, a);
     }
-    F1 = DF{__shfl_sync(0xffffffffu, F1.hi, 0), __shfl_sync(0xffffffffu, F1.lo, 0)};
-    F2 = DF{__shfl_sync(0xffffffffu, F2.hi, 0), __shfl_sync(0xffffffffu, F2.lo, 0)};
+    if (lane == 0) s.F[half] = F;
+}
+
+// The stage's scalars, by one warp.
+__device__ __forceinline__ void group_stage(GroupSmem& s, float kdl, int lane) {
+    const int m = s.I.m, n = s.I.n;
     const float4 last = s.vec[n + m - 1];
-    const StageK K = stage_scalars(m, n, s.C, s.sm1, s.sm2, F1, F2, DF{last.x, last.y}, DF{last.z, last.w},
+    const StageK K = stage_scalars(m, n, s.C, s.sm1, s.sm2, s.F[0], s.F[1], DF{last.x, last.y}, DF{last.z, last.w},
                                    df_ld(s.mar[n + m - 1]), kdl);
     if (lane == 0) s.K = K;
 }
@@ -264,7 +271,7 @@ __device__ __forceinline__ PieceLd piece_load(const HotInst& I, const GTile& g, 
 __device__ __forceinline__ void piece_finish(GroupSmem& s, const GTile& g, int S, int item, const PieceLd& p,
                                              const float* __restrict__ cs, bool out) {
     const HotInst& I = s.I;
-    const PieceK K = piece_consts(I, s.C);
+    const PieceK& K = s.PK;
     const int n = I.n;
     const bool f1 = g.slab < n, row = item < g.nr;
     const int e = row ? g.r0 + item : item - g.nr;
@@ -526,27 +533,90 @@ __device__ __forceinline__ void group_sweep(GroupSmem& s, const GTile& g, const 
     }
 }
 
-template <bool PAD>
-__device__ __forceinline__ void group_instance(GroupSmem& s, int rank, int G, int K, int* err) {
+// The end of a check block (the kernels k_kkt1 ... k_block_end of the chain),
+// shared out over the group's CTAs.  Returns true when the instance goes on.
+// Out of line: its code is large and runs once in K iterations.
+struct BlockRule {
+    int K;
+    double a1, a2, a3;
+};
+__device__ __noinline__ bool group_block_end(GroupSmem& s, const WorkDev* W, int inst, int rank, int G,
+                                             unsigned& epoch, BlockRule rule) {
     const HotInst& I = s.I;
+    double* s_row = reinterpret_cast<double*>(s.row);        // row and xrow
+    double* s_col = reinterpret_cast<double*>(s.col);        // col and xcol
+    double* s_red = reinterpret_cast<double*>(s.red);
+    const int nt = g_ntiles(I);
+    if (!group_wait(s, G, ++epoch, W->err)) return false;
+#pragma unroll 1
+    for (int c = rank; c < I.n_k1 + I.n_achunk; c += G) {
+        if (c < I.n_k1) residual_chunk<true>(I, c, s_red);
+        else objective_chunk(I, c - I.n_k1, s.red, s.col);
+        __syncthreads();
+    }
+    if (!group_wait(s, G, ++epoch, W->err)) return false;
+    if (rank == 0) check_instance<true>(I, W, inst, rule.K, rule.a1, rule.a2, rule.a3, s_red);
+    if (!group_wait(s, G, ++epoch, W->err)) return false;
+    const int status = __ldcg(&I.ctl->status), restart = __ldcg(&I.ctl->restart_pending);
+    auto tiles = [&](auto mode) {
+#pragma unroll 1
+        for (int t = rank; t < nt; t += G) {
+            int slab, band;
+            g_tile_slab(I, t, slab, band);
+            restart_tile<float, decltype(mode)::value>(I, slab, band, s_row, s_col, s_red);
+            __syncthreads();
+        }
+    };
+    if (status != ST_RUNNING) {
+        tiles(std::integral_constant<int, 2>());             // x-bar and <c, d> of the final iteration
+        if (!group_wait(s, G, ++epoch, W->err)) return false;
+        if (rank == 0) end_instance(I, s.red);
+        return false;
+    }
+    if (!restart) return true;
+    tiles(std::integral_constant<int, 0>());
+    if (!group_wait(s, G, ++epoch, W->err)) return false;
+    if (rank == 0) sigma_instance<true>(I, s_red);
+    if (!group_wait(s, G, ++epoch, W->err)) return false;
+    tiles(std::integral_constant<int, 1>());
+    if (!group_wait(s, G, ++epoch, W->err)) return false;
+    const double sigma = __ldcg(&I.ctl->sigma);
+#pragma unroll 1
+    for (int slab = rank; slab < g_nslab(I); slab += G) anchor_slab(I, slab, sigma);
+    if (rank == 0 && threadIdx.x == 0) I.ctl->restart_pending = 0;   // read by every CTA before the waits above
+    return group_wait(s, G, ++epoch, W->err);
+}
+
+template <bool PAD>
+__device__ __forceinline__ void group_instance(GroupSmem& s, const WorkDev* __restrict__ W, int inst, int rank, int G,
+                                               int blocks, BlockRule rule) {
+    const HotInst& I = s.I;
+    const int K = rule.K;
+    int* err = W->err;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int ns = I.m + I.n, nt = g_ntiles(I);
     const int nq = (nt - rank + G - 1) / G;            // tiles of this CTA: rank, rank + G, ...
-    const bool dz = I.ctl->dzero != 0;
     const float* u = (const float*)I.u;
     float* d0 = (float*)I.d0;
     float* d1 = (float*)I.d1;
     const Half h1 = half_of(I.m), h2 = half_of(I.n);
-    if (tid < K) s.p[tid] = make_p32(I.ctl->sigma, I.ctl->k + tid, I.h, I.gadmm, I.relax);
     if (tid == 64) {
         s.sm1 = df_from(I.sum_mu1);
         s.sm2 = df_from(I.sum_mu2);
     }
 #pragma unroll 1
     for (int q = tid; q < ns; q += kThreads) s.mar[q] = q < I.n ? I.cm2[q] : I.rm2[q - I.n];
-    if (tid >= 128 && tid - 128 < min(nq, kTileTable)) s.tile[tid - 128] = gtile(I, rank + (tid - 128) * G);
-    __syncthreads();
     unsigned epoch = 0;
+#pragma unroll 1
+  for (int blk = 0; blk < blocks; ++blk) {
+    const bool dz = __ldcg(&I.ctl->dzero) != 0;
+    if (tid < K) s.p[tid] = make_p32(__ldcg(&I.ctl->sigma), __ldcg(&I.ctl->k) + tid, I.h, I.gadmm, I.relax);
+    if (tid >= 128 && tid - 128 < min(nq, kTileTable)) s.tile[tid - 128] = gtile(I, rank + (tid - 128) * G);
+#pragma unroll 1
+    for (int q = tid; q < (int)(sizeof(CycleK) / 8); q += kThreads)
+        reinterpret_cast<double*>(&s.C)[q] = __ldcg(reinterpret_cast<const double*>(I.cyc) + q);
+    __syncthreads();
+    if (tid == 96) s.PK = piece_consts(I, s.C);        // read after the first wait
 #pragma unroll 1
     for (int it = 0; it < K; ++it) {
         // iteration it reads the delta of it - 1: d0 at the block's start, then
@@ -586,6 +656,8 @@ __device__ __forceinline__ void group_instance(GroupSmem& s, int rank, int G, in
 #pragma unroll 1
                 for (int w = tid; w < ns; w += kThreads) s.vec[w] = __ldcg(I.tp + w);
                 __syncthreads();
+                if (warp < 2) group_half_total(s, warp, lane);
+                __syncthreads();
                 if (warp == 0) group_stage(s, kdl, lane);
                 __syncthreads();
                 group_vectors(s);
@@ -624,10 +696,13 @@ __device__ __forceinline__ void group_instance(GroupSmem& s, int rank, int G, in
             }
         }
     }
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    if (!group_block_end(s, W, inst, rank, G, epoch, rule)) return;
+  }
 }
 
 template <bool PAD>
-__global__ void __launch_bounds__(kThreads, 2) k_group32(const WorkDev* __restrict__ W, int K) {
+__global__ void __launch_bounds__(kThreads, 2) k_group32(const WorkDev* __restrict__ W, int blocks, BlockRule rule) {
     extern __shared__ __align__(16) unsigned char s_raw[];
     GroupSmem& s = *reinterpret_cast<GroupSmem*>(s_raw);
     const int tid = threadIdx.x;
@@ -641,14 +716,18 @@ __global__ void __launch_bounds__(kThreads, 2) k_group32(const WorkDev* __restri
 #pragma unroll 1
         for (int q = tid; q < (int)(sizeof(HotInst) / 8); q += kThreads)
             reinterpret_cast<double*>(&s.I)[q] = reinterpret_cast<const double*>(src)[q];
-        const CycleK* cyc = src->cyc;
-#pragma unroll 1
-        for (int q = tid; q < (int)(sizeof(CycleK) / 8); q += kThreads)
-            reinterpret_cast<double*>(&s.C)[q] = reinterpret_cast<const double*>(cyc)[q];
         __syncthreads();
         if (s.I.ctl->status != ST_RUNNING) continue;   // the same for the whole group
-        group_instance<PAD>(s, ge.y, ge.z, K, W->err);
+        group_instance<PAD>(s, W, ge.x, ge.y, ge.z, blocks, rule);
         asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+        if (ge.z > 1 && tid == 0 && s.dead == 0) {
+            // the last CTA to leave (all have left their waits) clears the counters for the next launch
+            __threadfence();
+            if (atomicAdd(s.I.gcount + 1, 1u) == (unsigned)ge.z - 1u) {
+                s.I.gcount[0] = 0u;
+                s.I.gcount[1] = 0u;
+            }
+        }
     }
 }
 
@@ -682,7 +761,8 @@ int group_grid() {
     return cache[dev];
 }
 
-void launch_group(const WorkDev* w, int grid, int K, bool pad, cudaStream_t st) {
+void launch_group(const WorkDev* w, int grid, int K, int blocks, double a1, double a2, double a3, bool pad,
+                  cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(kThreads);
@@ -693,7 +773,7 @@ void launch_group(const WorkDev* w, int grid, int K, bool pad, cudaStream_t st) 
     at[0].val.cooperative = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, pad ? k_group32<true> : k_group32<false>, w, K);
+    cudaLaunchKernelEx(&cfg, pad ? k_group32<true> : k_group32<false>, w, blocks, BlockRule{K, a1, a2, a3});
 }
 
 }  // namespace hot

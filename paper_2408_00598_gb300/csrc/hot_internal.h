@@ -165,7 +165,7 @@ struct HotInst {
     float2* rs2b;          // [2mn]
     float* cs32b;          // [slab][band][column]
     float4* tp;            // [m + n]
-    unsigned int* gcount;  // arrivals of the group's CTAs in the running launch (0 between launches)
+    unsigned int* gcount;  // [2] arrivals and departures of the group's CTAs in the running launch (0 between launches)
     unsigned int* vcount;  // k_vec32 items of this instance finished in the running launch (0 between launches)
     float2* mu1f;          // [m][n] mu1 as pairs
     float2* mu2f;          // [m][n] mu2 as pairs
@@ -230,12 +230,12 @@ struct WorkDev {
     int ninst;
     int alternate;         // the sweeps' state exceeds L2: odd iterations take the tiles in reverse
     HotInst* inst;         // [ninst]
-    int* pre_tile;         // restart tiles: n nb1 + m nb2 per instance
-    int* pre_swp;          // sweep tiles: the same, 0 for instances that k_group32 runs
+    // (0 for the instances that k_group32 runs)
+    int* pre_tile;         // sweep / restart tiles: n nb1 + m nb2 per instance
     int* pre_slab;         // k_alpha: m + n slabs per instance
-    int* pre_vec;          // k_vec: 2(m + n) per instance (one warp each); k_vec32: vec32_items(m, n) CTA items (0 for k_group32's)
-    int* pre_k1;           // k_kkt1: n_k1 per instance, and n_achunk more for k_group32's
-    int* pre_achunk;       // k_alpha32: n_achunk per instance (0 for k_group32's)
+    int* pre_vec;          // k_vec: 2(m + n) per instance (one warp each); k_vec32: vec32_items(m, n) CTA items
+    int* pre_k1;           // k_kkt1: n_k1 per instance
+    int* pre_achunk;       // k_alpha32: n_achunk per instance
     int* gstart;           // k_group32: entries of CTA c are gent[gstart[c]] ... gent[gstart[c + 1] - 1]
     int4* gent;            // instance, rank in its group, group size
     int* n_running;        // instances still running
@@ -283,8 +283,9 @@ void launch_solve_kernels(const WorkDev* w, const LaunchDims& ld, int fp64, int 
 void launch_sweep(const WorkDev* w, const LaunchDims& ld, int fp64, int j, bool check, bool pad, cudaStream_t st);
 void launch_block_end(const WorkDev* w, const LaunchDims& ld, int fp64, int K, double a1, double a2, double a3,
                       cudaStream_t st);
-// k_group32 (hot_group.cu): K iterations of every grouped instance in one cooperative launch
-void launch_group(const WorkDev* w, int grid, int K, bool pad, cudaStream_t st);
+// k_group32 (hot_group.cu): up to `blocks` check blocks of every grouped instance in one cooperative launch
+void launch_group(const WorkDev* w, int grid, int K, int blocks, double a1, double a2, double a3, bool pad,
+                  cudaStream_t st);
 int group_grid();                          // CTAs resident at once on the current device (0: not available)
 cudaError_t group_init();
 LaunchDims make_launch_dims(int device, int fp64);

@@ -236,6 +236,7 @@ static int serve_start(Ctx* ctx) {
     s->batch->device = ctx->device;
     s->batch->fp64 = ctx->cfg.precision == HOT_FP64 ? 1 : 0;
     s->batch->K = ctx->cfg.check_every;
+    s->batch->max_group_blocks = 1;          // admissions and cancellations wait for the launches in flight
     s->batch->a1 = ctx->cfg.restart_sufficient;
     s->batch->a2 = ctx->cfg.restart_necessary;
     s->batch->a3 = ctx->cfg.restart_long;
