@@ -1,12 +1,173 @@
-// The end of a check block, as device functions of one CTA: the KKT partial
-// sums, the stopping and restart rules, the sigma update, the restart passes
-// over the state, and the anchor constants of the new cycle.  hot_kernels.cu
-// launches them as kernels, hot_group.cu calls them inside k_group32.
+// Device functions of one CTA that hot_kernels.cu launches as kernels and
+// hot_group.cu calls inside its kernels: the FP64 sweep of a tile, and the end of
+// a check block (the KKT partial sums, the stopping and restart rules, the
+// sigma update, the restart passes over the state, and the anchor constants of
+// the new cycle).
 #pragma once
 
 #include "hot_dev.cuh"
 
 namespace hot {
+
+// ----------------------------------------------------------- FP64 sweep --
+constexpr int kMaxTR64 = 64;               // FP64 tiles: TR <= side and TR * (longer row pitch) <= 4096
+struct Sweep64Smem {
+    double row[kRowSmemBytes / 8 + 256];
+    double xrow[kRowSmemBytes / 8 + 256];
+    double col[kThreads * 2];
+    double xcol[kThreads * 2];
+    double red[kNK * 32];
+    double3 a[kMaxTR64];                   // per row: h x^2 - alpha, -2 h x, dalpha
+};
+
+// a > b for doubles, on the integer pipe (FP64 comparisons run at a 64th of the
+// FP32 rate, like all FP64 instructions here); a NaN compares as larger.
+__device__ __forceinline__ bool gt64(double a, double b) {
+    long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+    x ^= (x >> 63) & 0x7fffffffffffffffLL;
+    y ^= (y >> 63) & 0x7fffffffffffffffLL;
+    return x > y;
+}
+
+// -a on the integer pipe, for the same reason
+__device__ __forceinline__ double neg64(double a) {
+    return __hiloint2double(__double2hiint(a) ^ 0x80000000, __double2loint(a));
+}
+
+// Steps 2-4 of Algorithm 2 on one tile (TR rows of a slab) in FP64, and the
+// tile's row and column sums.  ab, dab: the slab's pieces, rows then columns.
+// Bound: the FP64 pipe (2 lanes per clock and SM).  An element takes 8.5 FP64
+// instructions (about 13 before): the cost is separable, h (x_r - x_c)^2 - alpha -
+// beta = (h x_r^2 - alpha) + (h x_c^2 - beta) - 2 h x_r x_c with the first term per
+// row and the second per column (x taken from the middle bin, so that the
+// squares stay below the largest cost), and comparisons run on integers.
+// FP64 pipe 81 % busy.  One sweep: 128 x 128 125 -> 92 us, 256 x 256 947 -> 651 us;
+// on check iterations 224 -> 193 and 1,748 -> 1,424 us.
+template <bool CHECK>
+__device__ __forceinline__ void sweep64_tile(const HotInst& I, int slab, int band, const double* __restrict__ din_,
+                                             double* __restrict__ dout_, const P64& p, const double* __restrict__ ab,
+                                             const double* __restrict__ dab, double* __restrict__ rs_out,
+                                             double* __restrict__ cs_out, Sweep64Smem& s) {
+    constexpr int NV = 2;
+    const int S = g_side(I, slab), Sp = g_pitch(I, slab), TR = I.TR;       // this slab's side and row pitch
+    const int NC = Sp / NV;
+    const int P = kThreads / NC;
+    const int tid = threadIdx.x;
+    const int cg = tid % NC, ro = tid / NC;
+    const bool active = ro < P;
+    const int r0 = band * TR, nr = min(S, r0 + TR) - r0;
+    const size_t off = g_elem(I, slab) + (size_t)r0 * Sp;
+    const double* __restrict__ u = (const double*)I.u + off;
+    const double* __restrict__ din = din_ + off;
+    double* __restrict__ dout = dout_ + off;
+    const double* __restrict__ X = I.X64 + g_xbase(I, slab);               // bin coordinates of this half
+    const double mid = X[S / 2], h = p.h;
+    if (tid < nr) {
+        const double x = X[r0 + tid] - mid;
+        s.a[tid] = make_double3(fma(h * x, x, -ab[r0 + tid]), -2.0 * h * x, dab[r0 + tid]);
+    }
+    const int c0 = cg * NV;
+    const int nval = S - c0;                                               // columns inside the slab (pad after)
+    double B[NV], db[NV], xc[NV], cacc[NV], xacc[NV];
+#pragma unroll
+    for (int e = 0; e < NV; ++e) {
+        const bool v = active && e < nval;
+        xc[e] = v ? X[c0 + e] - mid : 0.0;
+        B[e] = v ? fma(h * xc[e], xc[e], -ab[S + c0 + e]) : 0.0;
+        db[e] = v ? dab[S + c0 + e] : 0.0;
+        cacc[e] = xacc[e] = 0.0;
+    }
+    double k64[kNK] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    const double nis = -p.is, rho = p.rho, trs = p.trs, sg = p.s;
+    __syncthreads();
+    if (active) {
+        double un[NV], dn[NV];
+        if (ro < nr) {
+            VecT<double>::ld(u + (size_t)ro * Sp + c0, un);
+            VecT<double>::ld(din + (size_t)ro * Sp + c0, dn);
+        }
+        for (int r = ro; r < nr; r += P) {
+            const double uu[NV] = {un[0], un[1]}, dd[NV] = {dn[0], dn[1]};
+            if (r + P < nr) {                                              // the next row's loads
+                VecT<double>::ld(u + (size_t)(r + P) * Sp + c0, un);
+                VecT<double>::ld(din + (size_t)(r + P) * Sp + c0, dn);
+            }
+            const double3 a = s.a[r];
+            double out[NV], xo[NV];
+#pragma unroll
+            for (int e = 0; e < NV; ++e) {
+                const double g = fma(a.y, xc[e], a.x + B[e]);              // c - A^T y-bar
+                const double D = a.z + db[e];                              // A^T (y-bar - y0)
+                const double sv = uu[e] + dd[e];
+                const double w = fma(nis, sv, -D);                         // g - v / sigma
+                const double mg = neg64(g);
+                const bool pos = gt64(w, mg);                              // z-bar > 0
+                const double r_ = pos ? w : mg;                            // z-bar - g
+                out[e] = fma(trs, r_, rho * dd[e]);
+                xo[e] = 0.0;
+                if (e >= nval) {
+                    out[e] = 0.0;                                          // pad columns stay 0
+                    continue;
+                }
+                if constexpr (CHECK) {
+                    const double zb = pos ? g + w : 0.0, xb = fma(sg, D, sv);
+                    const double mn = gt64(xb, zb) ? zb : xb;
+                    const double dx = X[r0 + r] - X[c0 + e];
+                    xo[e] = xb;
+                    k64[0] = fma(r_, r_, k64[0]);
+                    k64[1] = fma(mn, mn, k64[1]);
+                    k64[2] = fma(xb, xb, k64[2]);
+                    k64[3] = fma(zb, zb, k64[3]);
+                    k64[4] = fma(dx * dx, xb, k64[4]);
+                    xacc[e] += xb;
+                }
+                cacc[e] += out[e];
+            }
+            VecT<double>::st(dout + (size_t)r * Sp + c0, out);
+            s.row[r * (NC + 1) + cg] = out[0] + out[1];
+            if constexpr (CHECK) s.xrow[r * (NC + 1) + cg] = xo[0] + xo[1];
+        }
+#pragma unroll
+        for (int e = 0; e < NV; ++e) {
+            s.col[ro * Sp + c0 + e] = cacc[e];
+            if constexpr (CHECK) s.xcol[ro * Sp + c0 + e] = xacc[e];
+        }
+    }
+    __syncthreads();
+    const size_t cbase = g_colp(I, slab, band), rbase = g_row(I, slab) + r0;
+    for (int c = tid; c < S; c += kThreads) {
+        cs_out[cbase + c] = sum_f64_strided(s.col + c, P, Sp);
+        if constexpr (CHECK) I.xcs_part[cbase + c] = sum_f64_strided(s.xcol + c, P, Sp);
+    }
+    // rows: eight lanes per row, each every eighth partial, then the lanes' sums
+    // (one thread per row was a chain of NC dependent adds on one warp)
+    for (int q = tid; q < ((nr * 8 + 31) & ~31); q += kThreads) {
+        const int r = q >> 3, l = q & 7;
+        double acc = 0.0, xac = 0.0;
+        if (r < nr)
+            for (int c = l; c < NC; c += 8) {
+                acc += s.row[r * (NC + 1) + c];
+                if constexpr (CHECK) xac += s.xrow[r * (NC + 1) + c];
+            }
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) {
+            acc += __shfl_down_sync(0xffffffffu, acc, o, 8);
+            if constexpr (CHECK) xac += __shfl_down_sync(0xffffffffu, xac, o, 8);
+        }
+        if (l == 0 && r < nr) {
+            rs_out[rbase + r] = acc;
+            if constexpr (CHECK) I.xrs[rbase + r] = xac;
+        }
+    }
+    if constexpr (CHECK) {
+        block_sum<kNK>(k64, s.red);
+        if (tid == 0) {
+            double* o = I.tile_kkt + (size_t)g_tile(I, slab, band) * kNK;
+#pragma unroll
+            for (int q = 0; q < kNK; ++q) o[q] = k64[q];
+        }
+    }
+}
 
 // Once per cycle (after a restart, and at the start): the anchor parts of the
 // right-hand side, per slab: R1a along the slab's rows and the column totals

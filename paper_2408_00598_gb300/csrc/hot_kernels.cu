@@ -586,17 +586,12 @@ __global__ void __launch_bounds__(kThreads) k_anchor_one(HotInst I, double sigma
 }
 
 // --------------------------------------------------------------- k_sweep --
-// FP64 mode: Steps 2-4 of Algorithm 2 on one tile (TR rows of one slab) per
-// loop trip.
-__global__ void __launch_bounds__(kThreads, 2) k_sweep64(const WorkDev* __restrict__ W, int j, int check) {
+// FP64 mode: Steps 2-4 of Algorithm 2, tiles in a grid-stride loop
+// (sweep64_tile, hot_block.cuh).
+template <bool CHECK>
+__global__ void __launch_bounds__(kThreads, 2) k_sweep64(const WorkDev* __restrict__ W, int j) {
     pdl_enter();
-    constexpr int NV = 2;
-    constexpr int kRowN = kRowSmemBytes / sizeof(double) + 256;
-    __shared__ __align__(16) double s_row[kRowN];
-    __shared__ __align__(16) double s_col[kThreads * NV];
-    __shared__ __align__(16) double s_xrow[kRowN];
-    __shared__ __align__(16) double s_xcol[kThreads * NV];
-    __shared__ double s_red[kNK * 32];
+    __shared__ Sweep64Smem sm;
     __shared__ int s_tile[4];
     __shared__ P64 s_p64;
     const int ninst = W->ninst;
@@ -609,99 +604,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_sweep64(const WorkDev* __restri
             continue;
         }
         const HotInst& I = W->inst[tc.inst];
-        const int slab = tc.slab, band = tc.band;
-        const int S = g_side(I, slab), Sp = g_pitch(I, slab), TR = I.TR;   // this slab's side and row pitch
-        const int NC = Sp / NV;
-        const int P = kThreads / NC;
-        const int cg = threadIdx.x % NC, ro = threadIdx.x / NC;
-        const bool active = ro < P;
-        const int r0 = band * TR, r1 = min(S, r0 + TR);
-        const size_t off = g_elem(I, slab);
-        const double* __restrict__ u = (const double*)I.u + off;
-        const double* __restrict__ din = (const double*)((j & 1) ? I.d1 : I.d0) + off;
-        double* __restrict__ dout = (double*)((j & 1) ? I.d0 : I.d1) + off;
         if (threadIdx.x == 0) s_p64 = make_p64(I.ctl->sigma, I.ctl->k + j, I.h, I.gadmm, I.relax);
         __syncthreads();
-        const int c0 = cg * NV;
-        double cacc[NV], xacc[NV];
-#pragma unroll
-        for (int e = 0; e < NV; ++e) cacc[e] = xacc[e] = 0.0;
-        double k64[kNK] = {0.0, 0.0, 0.0, 0.0, 0.0};
-        const P64 p = s_p64;
-        const double* ab = I.ab64 + 2 * g_row(I, slab);
-        const double* dab = I.dab64 + 2 * g_row(I, slab);
-        const double* X = I.X64 + g_xbase(I, slab);            // bin coordinates of this half
-        double bb[NV], db[NV], cf[NV];
-        const int nval = S - c0;                                // columns inside the slab (pad after)
-#pragma unroll
-        for (int e = 0; e < NV; ++e) {
-            bb[e] = active && e < nval ? ab[S + c0 + e] : 0.0;
-            db[e] = active && e < nval ? dab[S + c0 + e] : 0.0;
-            cf[e] = active && e < nval ? X[c0 + e] : 0.0;
-        }
-        if (active) {
-            for (int r = r0 + ro; r < r1; r += P) {
-                const double a = ab[r], da = dab[r];
-                const double rf = X[r];
-                double uu[NV], dd[NV], out[NV], xo[NV];
-                VecT<double>::ld(u + (size_t)r * Sp + c0, uu);
-                VecT<double>::ld(din + (size_t)r * Sp + c0, dd);
-#pragma unroll
-                for (int e = 0; e < NV; ++e) {
-                    const double dc = rf - cf[e];
-                    const double cq = dc * dc;
-                    const E64 el = elem64(uu[e], dd[e], cq, a, bb[e], da, db[e], p);
-                    out[e] = p.rho * dd[e] + p.trs * el.r;
-                    xo[e] = 0.0;
-                    if (e >= nval) {
-                        out[e] = 0.0;                               // pad columns stay 0
-                        continue;
-                    }
-                    if (check) {
-                        double xb, zb;
-                        xz64(el, p, xb, zb);
-                        xo[e] = xb;
-                        const double mn = fmin(xb, zb);
-                        k64[0] += el.r * el.r;
-                        k64[1] += mn * mn;
-                        k64[2] += xb * xb;
-                        k64[3] += zb * zb;
-                        k64[4] += cq * xb;
-                        xacc[e] += xb;
-                    }
-                    cacc[e] += out[e];
-                }
-                VecT<double>::st(dout + (size_t)r * Sp + c0, out);
-                s_row[(r - r0) * (NC + 1) + cg] = out[0] + out[1];
-                if (check) s_xrow[(r - r0) * (NC + 1) + cg] = xo[0] + xo[1];
-            }
-        }
-        __syncthreads();
-        if (active) {
-#pragma unroll
-            for (int e = 0; e < NV; ++e) {
-                s_col[ro * Sp + c0 + e] = cacc[e];
-                if (check) s_xcol[ro * Sp + c0 + e] = xacc[e];
-            }
-        }
-        __syncthreads();
-        const size_t cbase = g_colp(I, slab, band);
-        for (int c = threadIdx.x; c < S; c += blockDim.x) {
-            I.cs_part[cbase + c] = sum_f64_strided(s_col + c, P, Sp);
-            if (check) I.xcs_part[cbase + c] = sum_f64_strided(s_xcol + c, P, Sp);
-        }
-        for (int rr = threadIdx.x; rr < r1 - r0; rr += blockDim.x) {
-            I.rs[g_row(I, slab) + r0 + rr] = sum_f64_strided(s_row + rr * (NC + 1), NC, 1);
-            if (check) I.xrs[g_row(I, slab) + r0 + rr] = sum_f64_strided(s_xrow + rr * (NC + 1), NC, 1);
-        }
-        if (check) {
-            block_sum<kNK>(k64, s_red);
-            if (threadIdx.x == 0) {
-                double* o = I.tile_kkt + (size_t)g_tile(I, slab, band) * kNK;
-#pragma unroll
-                for (int q = 0; q < kNK; ++q) o[q] = k64[q];
-            }
-        }
+        const size_t o = 2 * g_row(I, tc.slab);
+        sweep64_tile<CHECK>(I, tc.slab, tc.band, (const double*)((j & 1) ? I.d1 : I.d0),
+                            (double*)((j & 1) ? I.d0 : I.d1), s_p64, I.ab64 + o, I.dab64 + o, I.rs, I.cs_part, sm);
         __syncthreads();
     }
 }
@@ -1274,8 +1181,8 @@ LaunchDims make_launch_dims(int device, int fp64) {
     if (sms <= 0) sms = 1;
     LaunchDims d;
     if (fp64) {
-        d.grid_tile = occ_grid(k_sweep64, sms, 0, 8);
-        d.grid_tile_chk = d.grid_tile;
+        d.grid_tile = occ_grid(k_sweep64<false>, sms, 0, 8);
+        d.grid_tile_chk = occ_grid(k_sweep64<true>, sms, 0, 8);
         d.grid_rst = std::min(occ_grid(k_restart<double, 0>, sms, 0, 8), occ_grid(k_restart<double, 1>, sms, 0, 8));
         d.grid_slab = occ_grid(k_alpha<true>, sms, 0, 4);
         d.grid_alpha = d.grid_slab;
@@ -1377,7 +1284,7 @@ void launch_solve_kernels(const WorkDev* w, const LaunchDims& ld, int fp64, int 
 
 void launch_sweep(const WorkDev* w, const LaunchDims& ld, int fp64, int j, bool check, bool pad, cudaStream_t st) {
     if (fp64)
-        launch(ld, k_sweep64, check ? ld.grid_tile_chk : ld.grid_tile, 0, st, w, j, check ? 1 : 0);
+        launch(ld, check ? k_sweep64<true> : k_sweep64<false>, check ? ld.grid_tile_chk : ld.grid_tile, 0, st, w, j);
     else if (check)
         launch(ld, pad ? k_sweep32<true, true> : k_sweep32<true, false>, ld.grid_tile_chk, kSweepSmemChk, st, w, j);
     else if (j == 0)
