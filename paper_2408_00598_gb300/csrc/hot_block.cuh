@@ -336,12 +336,11 @@ __device__ __forceinline__ void restart_tile(const HotInst& I, int slab, int ban
 #pragma unroll
                 for (int e = 0; e < NV; ++e) {
                     if constexpr (F32) {
-                        // (a - b)^2 exactly as a pair: the difference is exact to
-                        // rounding, its square split by fma
+                        // (a - b)^2: the difference is exact to rounding, its square
+                        // split by fma
                         const float dx = xbv[e] - xo[e], dz = zbv[e] - zo[e];
-                        const float px = dx * dx, pz = dz * dz;
-                        fr[0] = df_add(fr[0], DF{px, fmaf(dx, dx, -px)});
-                        fr[1] = df_add(fr[1], DF{pz, fmaf(dz, dz, -pz)});
+                        fr[0] = df_dot(fr[0], dx, dx);
+                        fr[1] = df_dot(fr[1], dz, dz);
                     } else {
                         const double dx = xbv[e] - xo[e], dz = zbv[e] - zo[e];
                         racc[0] += dx * dx;
@@ -367,9 +366,8 @@ __device__ __forceinline__ void restart_tile(const HotInst& I, int slab, int ban
                         if (cr) {
                             fr[0] = df_add(fr[0], cost_times(cost_pair(X32[r], xc[e]), (float)nu_[e]));
                         } else {
-                            const float dc = X32[r] - xc[e], cq = dc * dc;
-                            const float p = cq * (float)nu_[e];
-                            fr[0] = df_add(fr[0], DF{p, fmaf(cq, (float)nu_[e], -p)});
+                            const float dc = X32[r] - xc[e];
+                            fr[0] = df_dot(fr[0], dc * dc, (float)nu_[e]);
                         }
                     } else {
                         rsd += nu_[e];
@@ -393,9 +391,8 @@ __device__ __forceinline__ void restart_tile(const HotInst& I, int slab, int ban
                         if (cr) {
                             fr[0] = df_add(fr[0], cost_times(cost_pair(X32[r], xc[e]), (float)dd[e]));
                         } else {
-                            const float dc = X32[r] - xc[e], cq = dc * dc;
-                            const float pd = cq * (float)dd[e];
-                            fr[0] = df_add(fr[0], DF{pd, fmaf(cq, (float)dd[e], -pd)});
+                            const float dc = X32[r] - xc[e];
+                            fr[0] = df_dot(fr[0], dc * dc, (float)dd[e]);
                         }
                     }
                 }
@@ -561,6 +558,24 @@ __device__ __forceinline__ void residual_chunk(const HotInst& I, int chunk, doub
     }
 }
 
+// Chunk `chunk` (kThreads tiles) of the check sweep's KKT sums and of <c, u>
+// (FP32 mode): one pair each, so that k_check, a single CTA, adds few (512 x 512,
+// 16,384 tiles: 24 us; 20 us at 256 x 256 before, 11 now).
+__device__ __forceinline__ void tile_chunk(const HotInst& I, int chunk, float2* s_red) {
+    const int t = chunk * kThreads + (int)threadIdx.x;
+    const bool in = t < g_ntiles(I);
+    const float2* tk = reinterpret_cast<const float2*>(I.tile_kkt) + (size_t)t * kNK;
+    const float2 z = make_float2(0.f, 0.f);
+    DF v[kNK];
+#pragma unroll
+    for (int e = 0; e < kNK - 1; ++e) v[e] = df_ld(in ? tk[e] : z);
+    v[kNK - 1] = df_ld(in ? reinterpret_cast<const float2*>(I.cu_part)[t] : z);
+    block_sum_df<kNK>(v, s_red);
+    if (threadIdx.x == 0)
+#pragma unroll
+        for (int e = 0; e < kNK; ++e) I.kc_part[chunk * kNK + e] = df_st(v[e]);
+}
+
 // Sum of count pairs p[0], p[stride], ... of this thread's share (q = threadIdx.x,
 // q + blockDim.x, ...), the loads issued four at a time.
 __device__ __forceinline__ DF sum_pairs(const float2* __restrict__ p, int count, int stride) {
@@ -586,17 +601,17 @@ __device__ __forceinline__ void check_instance(const HotInst& I, const WorkDev* 
     const int ntile = g_ntiles(I), nslab = g_nslab(I);
     double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     if constexpr (F32) {
-        // eight sums of pairs, a warp each: the check sweep's per-tile KKT sums
-        // (0-3), k_alpha32's <c, A^T(y-bar - y0)> (4) and <b, y> (6) per chunk,
-        // the ||A x - b||^2 chunks (5) and <c, u> per tile (7); the objective's
+        // eight sums of pairs, a warp each: the check sweep's KKT sums (0-3) and
+        // <c, u> (7) per chunk of tiles, k_alpha32's <c, A^T(y-bar - y0)> (4) and
+        // <b, y> (6) per chunk, and the ||A x - b||^2 chunks (5); the objective's
         // <c, d> share is added when the instance ends.  (Short code: it runs
         // once a block, from cold instruction caches, while the grid waits.)
         float2* sh = reinterpret_cast<float2*>(s_red);
         const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        const float2* p = w < 4 ? reinterpret_cast<const float2*>(I.tile_kkt) + w
-                                : reinterpret_cast<const float2*>(w == 4 ? I.cD_part : w == 5 ? I.k1_part
-                                                                          : w == 6 ? I.dobj_part : I.cu_part);
-        const int count = w < 4 || w == 7 ? ntile : w == 5 ? I.n_k1 : I.n_achunk, stride = w < 4 ? kNK : 1;
+        const bool tile = w < 4 || w == 7;
+        const float2* p = tile ? I.kc_part + (w < 4 ? w : 4)
+                               : reinterpret_cast<const float2*>(w == 4 ? I.cD_part : w == 5 ? I.k1_part : I.dobj_part);
+        const int count = tile ? I.n_kc : w == 5 ? I.n_k1 : I.n_achunk, stride = tile ? kNK : 1;
         DF acc{0.f, 0.f};
 #pragma unroll 1
         for (int q0 = lane; q0 < count; q0 += 4 * 32) {

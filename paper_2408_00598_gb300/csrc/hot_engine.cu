@@ -236,6 +236,8 @@ int inst_create(const PairHost& p, int fp64, const hot_config& cfg, double tol, 
     const size_t o_xrs = take(2 * MN * 8);
     const size_t o_xcs = take(CP * 8);
     const size_t o_tk = take((size_t)ntiles * kNK * 8);
+    const int n_kc = fp64 ? 0 : (ntiles + kThreads - 1) / kThreads;
+    const size_t o_kc = take((size_t)n_kc * kNK * sizeof(float2));
     const size_t o_rp = take((size_t)ntiles * 2 * 8);
     const size_t o_vec = take(4 * (size_t)L * 8);
     const size_t o_mvec = take(4 * (size_t)L * 8);
@@ -293,6 +295,7 @@ int inst_create(const PairHost& p, int fp64, const hot_config& cfg, double tol, 
     d.nb2 = I->nb2;
     d.n_k1 = I->n_k1;
     d.n_achunk = n_achunk;
+    d.n_kc = n_kc;
     d.fp64 = fp64;
     d.gadmm = cfg.method == HOT_METHOD_GADMM ? 1 : 0;
     d.stop_abs = cfg.stop_rule == HOT_STOP_ABSOLUTE ? 1 : 0;
@@ -379,6 +382,7 @@ int inst_create(const PairHost& p, int fp64, const hot_config& cfg, double tol, 
     d.xcs_part = (double*)(sm + o_xcs);
     d.tile_kkt = (double*)(sm + o_tk);
     d.rst_part = (double*)(sm + o_rp);
+    d.kc_part = fp64 ? nullptr : (float2*)(sm + o_kc);
     d.vecs = (double*)(sm + o_vec);
     d.mvec = (double*)(sm + o_mvec);
     d.mu1 = (double*)(sm + o_mu1);
@@ -498,6 +502,7 @@ Batch::~Batch() {
             if (tev[p][q]) cudaEventDestroy(tev[p][q]);
     }
     if (cap_stream) cudaStreamDestroy(cap_stream);
+    cudaFree(d_tiles);
     cudaFree(d_work);
     cudaFree(d_inst);
     cudaFree(d_pre);
@@ -619,7 +624,7 @@ int Batch::set_instances(const std::vector<Inst*>& v, cudaStream_t st, bool grou
         pt[i + 1] = pt[i] + (g ? 0 : tiles);
         ps[i + 1] = ps[i] + (g ? 0 : m + nn);
         pv[i + 1] = pv[i] + (g ? 0 : v[i]->fp64 ? 2 * (m + nn) : vec32_items(m, nn));
-        pk[i + 1] = pk[i] + (g ? 0 : v[i]->n_k1);
+        pk[i + 1] = pk[i] + (g ? 0 : v[i]->n_k1 + v[i]->desc.n_kc);
         pa[i + 1] = pa[i] + (g ? 0 : v[i]->desc.n_achunk);
         if (v[i]->ctl_host.status == ST_RUNNING) ++running;
     }
@@ -638,6 +643,16 @@ int Batch::set_instances(const std::vector<Inst*>& v, cudaStream_t st, bool grou
     h_work->pre_vec = d_pre + 2 * (cap + 1);
     h_work->pre_k1 = d_pre + 3 * (cap + 1);
     h_work->pre_achunk = d_pre + 4 * (cap + 1);
+    const size_t swtiles = fp64 ? 0 : (size_t)pt[n];
+    if (swtiles > tiles_cap) {
+        cudaFree(d_tiles);
+        d_tiles = nullptr;
+        tiles_cap = 0;
+        const size_t want = std::max<size_t>(swtiles, 4096);
+        HOT_CK(cudaMalloc(&d_tiles, want * sizeof(SweepTile)));
+        tiles_cap = want;
+    }
+    h_work->tiles = d_tiles;
     h_work->gstart = d_gstart;
     h_work->gent = d_gent;
     h_work->n_running = d_running;
@@ -659,6 +674,10 @@ int Batch::set_instances(const std::vector<Inst*>& v, cudaStream_t st, bool grou
     HOT_CK(cudaMemcpyAsync(d_work, h_work, sizeof(WorkDev), cudaMemcpyHostToDevice, st));
     HOT_CK(cudaMemcpyAsync(d_running, h_running, sizeof(int) * 2, cudaMemcpyHostToDevice, st));
     if (n > 0) HOT_CK(cudaMemcpyAsync(d_st, h_st, sizeof(int) * n, cudaMemcpyHostToDevice, st));
+    if (swtiles > 0) {
+        launch_tile_table(d_work, (int)swtiles, st);
+        HOT_CK(cudaGetLastError());
+    }
     ninst = n;
     return HOT_OK;
 }

@@ -90,6 +90,8 @@ struct Batch {
     HotInst* d_inst = nullptr;
     int* d_pre = nullptr;
     int* d_running = nullptr;       // [2]: instances still running, error flag of the bounded waits
+    SweepTile* d_tiles = nullptr;   // [tiles_cap] the chain's sweep tiles (FP32 mode)
+    size_t tiles_cap = 0;
     int* d_gstart = nullptr;        // [ggrid + 1]
     int4* d_gent = nullptr;         // [ggrid + cap]
     int* h_gstart = nullptr;        // pinned

@@ -549,9 +549,10 @@ __device__ __noinline__ bool group_block_end(GroupSmem& s, const WorkDev* W, int
     const int nt = g_ntiles(I);
     if (!group_wait(s, G, ++epoch, W->err)) return false;
 #pragma unroll 1
-    for (int c = rank; c < I.n_k1 + I.n_achunk; c += G) {
+    for (int c = rank; c < I.n_k1 + I.n_achunk + I.n_kc; c += G) {
         if (c < I.n_k1) residual_chunk<true>(I, c, s_red);
-        else objective_chunk(I, c - I.n_k1, s.red, s.col);
+        else if (c < I.n_k1 + I.n_achunk) objective_chunk(I, c - I.n_k1, s.red, s.col);
+        else tile_chunk(I, c - I.n_k1 - I.n_achunk, s.red);
         __syncthreads();
     }
     if (!group_wait(s, G, ++epoch, W->err)) return false;

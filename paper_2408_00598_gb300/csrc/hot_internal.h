@@ -103,6 +103,7 @@ struct HotInst {
     int TR;                // rows per sweep tile
     int nb1, nb2;          // bands (tiles) per f1 slab = ceil(m / TR), per f2 slab = ceil(n / TR)
     int n_k1;              // chunks of the A x - b kernel
+    int n_kc;              // chunks of kThreads tiles (FP32 mode; 0 in FP64 mode)
     int n_achunk;          // chunks of k_alpha32 (kAlphaChunk pieces each; FP32 mode)
     int fp64;              // 1: FP64 state, 0: FP32 anchor + delta
     int gadmm;             // 1: Step 4 of the generalized ADMM instead of Halpern's
@@ -110,7 +111,6 @@ struct HotInst {
     int coord_real;        // FP32 mode: some bin coordinate is not an integer in [-2048, 2048], so the
                            // pieces carry h x^2 - alpha as pairs and the sweep forms the cost term in pairs
     int grp;               // 1: k_group32 runs this instance's iterations, not the chain of kernels
-    int pad0;
     double relax;          // rho of the generalized ADMM
     double h;              // 2^-E
     double norm_b;         // ||b||
@@ -140,6 +140,7 @@ struct HotInst {
     double* xrs;           // [2mn] row sums of x-bar (check iterations)
     double* xcs_part;      // [slab][band][column] partial sums of x-bar
     double* tile_kkt;      // [tiles][kNK], tiles = n nb1 + m nb2
+    float2* kc_part;       // [n_kc][kNK] sums of tile_kkt (first four) and of cu_part over chunks of tiles (FP32 mode)
     double* rst_part;      // [tiles][2]
     double* vecs;          // [4][max(m, n)]: T1, T2, P1, P2 (slab totals and cross-slab row sums)
     double* mvec;          // [4][max(m, n)]: instance-wide vectors of Prop. 3 (k_marg)
@@ -224,6 +225,25 @@ __host__ __device__ inline int g_xbase(const HotInst& I, int s) { return s < I.n
 // stride of the four instance-wide Prop. 3 vectors (indexed by j < n or k < m)
 __host__ __device__ inline int g_L(const HotInst& I) { return I.m > I.n ? I.m : I.n; }
 
+// One tile of the FP32 sweep (k_sweep32), resolved once when the work tables
+// are set: the sweep's threads read it from here instead of searching the
+// prefix table and dividing for every tile (about 1,000 cycles each, on the path
+// of the next copies; with rows and columns reduced side by side, one sweep of
+// 20 instances with sides 32 to 128: 95 -> 77 us, of 512 x 512: 516 -> 500 us).
+struct alignas(128) SweepTile {
+    int inst, slab, band, S, NC, P, r0, r1, npass;   // NC: column groups of the row pitch (S rounded up to 4)
+    int row;          // g_row: first row entry of the slab
+    int tile;         // g_tile: index of the tile within its instance
+    int colp;         // g_colp: first column-partial entry of (slab, band)
+    int dz;           // set by the sweep: the delta read is zero (first iteration after an FP32 restart): no loads
+    int pad;
+    long long elem;   // g_elem: first flow variable of the slab
+    const HotCtl* ctl;
+    const float *u, *d0, *d1;     // of the tile's first row
+    const float4* ab;             // alpha piece of the tile's first row
+    const P32* p32;
+};
+
 // Work tables of one batch, in device memory.  pre_* are prefix sums over the
 // instances of the number of work items each kernel family handles.
 struct WorkDev {
@@ -234,8 +254,9 @@ struct WorkDev {
     int* pre_tile;         // sweep / restart tiles: n nb1 + m nb2 per instance
     int* pre_slab;         // k_alpha: m + n slabs per instance
     int* pre_vec;          // k_vec: 2(m + n) per instance (one warp each); k_vec32: vec32_items(m, n) CTA items
-    int* pre_k1;           // k_kkt1: n_k1 per instance
+    int* pre_k1;           // k_kkt1: n_k1 + n_kc per instance
     int* pre_achunk;       // k_alpha32: n_achunk per instance
+    SweepTile* tiles;      // [pre_tile[ninst]] (FP32 mode)
     int* gstart;           // k_group32: entries of CTA c are gent[gstart[c]] ... gent[gstart[c + 1] - 1]
     int4* gent;            // instance, rank in its group, group size
     int* n_running;        // instances still running
@@ -244,6 +265,7 @@ struct WorkDev {
 };
 
 // Host-side launch helpers (hot_kernels.cu).
+void launch_tile_table(const WorkDev* w, int ntiles, cudaStream_t st);   // fills WorkDev::tiles
 struct LaunchDims {
     // persistent grids: SM count x resident CTAs per SM of each kernel, so
     // that every CTA of a grid-stride loop is resident from the start

@@ -635,41 +635,33 @@ __global__ void __launch_bounds__(kThreads, 2) k_sweep64(const WorkDev* __restri
 // floats (checked when the instance is created); zero-initialised at module load.
 __device__ __align__(16) float g_zero_tile[kMaxTileElems];
 
-struct TileD {
-    int inst, slab, band, S, NC, P, r0, r1, npass;   // NC: column groups of the row pitch (S rounded up to 4)
-    int row;          // g_row: first row entry of the slab
-    int tile;         // g_tile: index of the tile within its instance
-    int colp;         // g_colp: first column-partial entry of (slab, band)
-    int dz;           // the delta read is zero (first iteration after an FP32 restart): no loads
-    long long elem;   // g_elem: first flow variable of the slab
-};
-
-// Resolve tile t; npass = 0 marks a tile of an instance that is not running,
-// or t past the end.  PAD = false: every side of the batch is a multiple of 4,
-// so the pitch is the side.
-template <bool PAD>
-__device__ __forceinline__ TileD tile_desc(const WorkDev* __restrict__ W, int t, int ntiles, bool first) {
-    TileD d{};
-    if (t >= ntiles) return d;
+__global__ void __launch_bounds__(kThreads) k_tile_table(const WorkDev* __restrict__ W, int ntiles) {
+    const int t = blockIdx.x * kThreads + threadIdx.x;
+    if (t >= ntiles) return;
+    SweepTile d{};
     const int i = find_inst(W->pre_tile, W->ninst, t);
     const HotInst& I = W->inst[i];
-    const int loc = t - W->pre_tile[i];
     d.inst = i;
-    g_tile_slab(I, loc, d.slab, d.band);
+    g_tile_slab(I, t - W->pre_tile[i], d.slab, d.band);
     d.S = g_side(I, d.slab);
-    d.NC = (PAD ? g_pitch(I, d.slab) : d.S) / 4;
+    const int pitch = g_pitch(I, d.slab);
+    d.NC = pitch / 4;
     d.P = kThreads / d.NC;
     d.r0 = d.band * I.TR;
     d.r1 = min(d.S, d.r0 + I.TR);
+    d.npass = (d.r1 - d.r0 + d.P - 1) / d.P;
     d.row = (int)g_row(I, d.slab);
     d.tile = g_tile(I, d.slab, d.band);
     d.colp = (int)g_colp(I, d.slab, d.band);
-    d.elem = PAD ? (long long)g_elem(I, d.slab)
-                 : (d.slab < I.n ? (long long)d.slab * I.m * I.m
-                                 : (long long)I.n * I.m * I.m + (long long)(d.slab - I.n) * I.n * I.n);
-    if (I.ctl->status == ST_RUNNING) d.npass = (d.r1 - d.r0 + d.P - 1) / d.P;
-    if (first) d.dz = I.ctl->dzero;
-    return d;
+    d.elem = (long long)g_elem(I, d.slab);
+    d.ctl = I.ctl;
+    const size_t first = (size_t)d.elem + (size_t)d.r0 * pitch;
+    d.u = (const float*)I.u + first;
+    d.d0 = (const float*)I.d0 + first;
+    d.d1 = (const float*)I.d1 + first;
+    d.ab = I.ab32 + 2 * (size_t)d.row + d.r0;
+    d.p32 = I.p32;
+    W->tiles[t] = d;
 }
 
 // PAD: some slab side of the batch is not a multiple of 4, so a thread's
@@ -688,7 +680,9 @@ __global__ void __launch_bounds__(kThreads, CHECK ? 2 : 3) k_sweep32(const WorkD
     __shared__ __align__(16) float s_col[kThreads * NV];
     __shared__ __align__(16) float4 s_alpha[kStages][kMaxTR];
     __shared__ __align__(16) float2 s_rdf[kW][kMaxTR];            // per-warp row partial pairs
-    __shared__ TileD s_td[kStages];
+    // descriptors of the tiles in flight: the issue side starts tiles up to kStages
+    // ahead of the one being computed, so twice as many slots are never reused early
+    __shared__ SweepTile s_td[2 * kStages];
     __shared__ float2 s_red[kNK * 32];
     // dynamic: the pass ring [kStages][2][kThreads] float4, then (check
     // iterations) the x-bar row and column partials
@@ -715,31 +709,33 @@ __global__ void __launch_bounds__(kThreads, CHECK ? 2 : 3) k_sweep32(const WorkD
     // so a sweep starts on the tiles whose state the previous sweep touched
     // last (still in L2)
     const bool rev = (j & 1) && W->alternate;
+    auto at = [&](int t) { return W->tiles + (rev ? ntiles - 1 - t : t); };
     auto set_tile = [&](int t) {
-        TileD d = tile_desc<PAD>(W, rev && t < ntiles ? ntiles - 1 - t : t, ntiles, FIRST);
-        while (t < ntiles && d.npass == 0) {
-            t += G;
-            d = tile_desc<PAD>(W, rev && t < ntiles ? ntiles - 1 - t : t, ntiles, FIRST);
-        }
+        // tiles of an instance that is not running are passed over
+        while (t < ntiles && at(t)->ctl->status != ST_RUNNING) t += G;
         c.it = t;
         if (t < ntiles) {
-            const HotInst& I = W->inst[d.inst];
-            const int ro = tid / d.NC, cg = tid - ro * d.NC;
-            const int sp = PAD ? (d.S + 3) & ~3 : d.S;   // row pitch (without padded slabs, the side)
-            const size_t base = (size_t)d.elem + ((size_t)d.r0 + ro) * sp + (size_t)cg * NV;
-            c.u = (const float*)I.u + base;
+            const SweepTile* d = at(t);
+            // the next tile's descriptor on its way into L1
+            if (t + G < ntiles) asm volatile("prefetch.global.L1 [%0];\n" ::"l"(at(t + G)));
+            const int NC = d->NC, P = d->P;
+            const int ro = tid / NC, cg = tid - ro * NC;
+            const int sp = PAD ? (d->S + 3) & ~3 : d->S;   // row pitch (without padded slabs, the side)
+            const int base = ro * sp + cg * NV;
+            const bool dz = FIRST && d->ctl->dzero;
+            c.u = d->u + base;
             // a delta known to be zero (first iteration after an FP32 restart,
             // which stores none) is copied from a zero tile: L2 hits, no HBM read
-            c.d = (FIRST && d.dz) ? g_zero_tile + ((size_t)ro * sp + (size_t)cg * NV)
-                                  : (const float*)((j & 1) ? I.d1 : I.d0) + base;
-            const int nr = d.r1 - d.r0;
-            c.a = I.ab32 + 2 * (size_t)d.row + d.r0 + tid;
-            c.step = d.P * sp;
+            c.d = dz ? g_zero_tile + base : ((j & 1) ? d->d1 : d->d0) + base;
+            const int nr = d->r1 - d->r0;
+            c.a = d->ab + tid;
+            c.step = P * sp;
             // rows ro, ro + P, ... below nr (threads past P rows copy nothing)
-            c.mine = ro < d.P && ro < nr ? (nr - ro + d.P - 1) / d.P : 0;
-            c.left = d.npass;
+            c.mine = ro < P && ro < nr ? (nr - ro + P - 1) / P : 0;
+            c.left = d->npass;
             c.acopy = tid < nr;
-            if (tid == 0) s_td[c.ik % kStages] = d;
+            if (tid < (int)(sizeof(SweepTile) / 16))
+                reinterpret_cast<float4*>(&s_td[c.ik % (2 * kStages)])[tid] = reinterpret_cast<const float4*>(d)[tid];
         }
     };
     c.ik = 0;
@@ -776,11 +772,10 @@ __global__ void __launch_bounds__(kThreads, CHECK ? 2 : 3) k_sweep32(const WorkD
     // dbeta, x_c; loaded for the next tile during the current tile's epilogue
     float4 bq[NV];
     P32 p;
-    auto load_cols = [&](const TileD& d) {
-        const HotInst& I = W->inst[d.inst];
+    auto load_cols = [&](const SweepTile& d) {
         const int ro = tid / d.NC, c0 = (tid - ro * d.NC) * NV;
-        p = *I.p32;
-        const float4* ab = I.ab32 + 2 * (size_t)d.row + d.S;
+        p = *d.p32;
+        const float4* ab = d.ab - d.r0 + d.S;
 #pragma unroll
         for (int e = 0; e < NV; ++e)
             bq[e] = ro < d.P && (!PAD || c0 + e < d.S) ? ab[c0 + e] : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -794,7 +789,7 @@ __global__ void __launch_bounds__(kThreads, CHECK ? 2 : 3) k_sweep32(const WorkD
         __syncthreads();
         // the issue side has started every tile this CTA still has (it runs ahead)
         if (c.it >= ntiles && ck >= c.ik) break;
-        const TileD dc = s_td[ck % kStages];
+        const SweepTile& dc = s_td[ck % (2 * kStages)];
         if (!have) load_cols(dc);
         const HotInst& I = W->inst[dc.inst];
         const int S = dc.S, Sp = PAD ? (dc.S + 3) & ~3 : dc.S, NC = dc.NC, P = dc.P;
@@ -893,17 +888,8 @@ __global__ void __launch_bounds__(kThreads, CHECK ? 2 : 3) k_sweep32(const WorkD
         // issuing its first pass, before this barrier); the loads complete
         // under the reductions below
         have = !(c.it >= ntiles && ck + 1 >= c.ik);
-        if (have) load_cols(s_td[(ck + 1) % kStages]);
+        if (have) load_cols(s_td[(ck + 1) % (2 * kStages)]);
         const size_t cbase = dc.colp;
-        for (int cc = tid; cc < S; cc += kThreads) {
-            DF a{0.f, 0.f}, x{0.f, 0.f};
-            for (int qq = 0; qq < P; ++qq) {
-                a = df_add(a, s_col[qq * Sp + cc]);
-                if constexpr (CHECK) x = df_add(x, s_xcol[qq * Sp + cc]);
-            }
-            I.cs32[cbase + cc] = df_f(a);
-            if constexpr (CHECK) I.xcs_part[cbase + cc] = df_val(x);
-        }
         // rows: warp w sums partials [w NC/8, (w+1) NC/8) of rows lane, lane + 32, ...
         // (row stride NC + 1 keeps the lanes on distinct banks), then the 8
         // pairs of each row are combined in warp order
@@ -932,7 +918,9 @@ __global__ void __launch_bounds__(kThreads, CHECK ? 2 : 3) k_sweep32(const WorkD
         } else {
             __syncthreads();
         }
+        // rows on the first warps, columns on the last: side by side up to sides of 128
         for (int r = tid; r < nr; r += kThreads) {
+            const float2 u0 = I.rs02[dc.row + r0 + r];          // row sum of u
             DF a = df_ld(s_rdf[0][r]), x{0.f, 0.f};
             if constexpr (CHECK) x = df_ld(s_xdf[0][r]);
 #pragma unroll
@@ -940,9 +928,18 @@ __global__ void __launch_bounds__(kThreads, CHECK ? 2 : 3) k_sweep32(const WorkD
                 a = df_add(a, df_ld(s_rdf[w][r]));
                 if constexpr (CHECK) x = df_add(x, df_ld(s_xdf[w][r]));
             }
-            a = df_add(a, df_ld(I.rs02[dc.row + r0 + r]));      // + row sum of u
+            a = df_add(a, df_ld(u0));
             I.rs2[dc.row + r0 + r] = df_st(a);
             if constexpr (CHECK) I.xrs[dc.row + r0 + r] = df_val(x);
+        }
+        for (int cc = kThreads - 1 - tid; cc < S; cc += kThreads) {
+            DF a{0.f, 0.f}, x{0.f, 0.f};
+            for (int qq = 0; qq < P; ++qq) {
+                a = df_add(a, s_col[qq * Sp + cc]);
+                if constexpr (CHECK) x = df_add(x, s_xcol[qq * Sp + cc]);
+            }
+            I.cs32[cbase + cc] = df_f(a);
+            if constexpr (CHECK) I.xcs_part[cbase + cc] = df_val(x);
         }
     }
     cp_async_wait<0>();
@@ -1097,7 +1094,7 @@ __global__ void __launch_bounds__(kThreads) k_init_copy(HotInst I) {
 template <bool F32>
 __global__ void __launch_bounds__(kThreads) k_kkt1(const WorkDev* __restrict__ W) {
     pdl_enter();
-    __shared__ double s_red[32];
+    __shared__ double s_red[kNK * 32];
     __shared__ int s_t[3];
     const int ninst = W->ninst;
     const int nchunks = W->pre_k1[ninst];
@@ -1114,7 +1111,8 @@ __global__ void __launch_bounds__(kThreads) k_kkt1(const WorkDev* __restrict__ W
             continue;
         }
         const HotInst& I = W->inst[s_t[0]];
-        residual_chunk<F32>(I, s_t[1], s_red);
+        if (s_t[1] < I.n_k1) residual_chunk<F32>(I, s_t[1], s_red);
+        else tile_chunk(I, s_t[1] - I.n_k1, reinterpret_cast<float2*>(s_red));
         __syncthreads();
     }
 }
@@ -1210,6 +1208,10 @@ int sweep_grid(int fp64) {
     int& c = cache[fp64 ? 1 : 0][dev];
     if (c == 0) c = make_launch_dims(dev, fp64).grid_tile;
     return c;
+}
+
+void launch_tile_table(const WorkDev* w, int ntiles, cudaStream_t st) {
+    if (ntiles > 0) k_tile_table<<<(ntiles + kThreads - 1) / kThreads, kThreads, 0, st>>>(w, ntiles);
 }
 
 void launch_init(const HotInst& I, double sigma0, cudaStream_t st) {
