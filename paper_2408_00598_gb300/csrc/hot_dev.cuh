@@ -541,4 +541,165 @@ __device__ __forceinline__ void alpha32_stage(const HotInst& I, float2* __restri
     }
 }
 
+// ---------------------------------------------------------- k_marg/k_alpha --
+// Prop. 3 on R' = (b - A(u + d))/sigma, the right-hand side whose solution is
+// dy = y-bar - y0: with v = sigma g0 + u + d, the right-hand side of
+// eq. (update:y) is R = b/sigma - A(v/sigma - c) = AA^T y0 + R'.  R' comes
+// from the slab sums of u + d.  With j < n and k < m:
+//   a_j = sum_k R1(k,j), bb_j = sum_i R2(i,j), r3_k = sum_l R3(k,l), T3 = sum r3,
+//   y1-hat(k,j) = (R1(k,j) + a_j/n - (1/m+1/n) bb_j + r3_k/n + T3/n^2)/(m+n),
+//   s_k = sum_j y1-hat(k,j),  t = W-hat s,  y1^a = t + (1^T t / n) 1,
+//   y1 = y1-hat - y1^a,  y2(i,j) = (R2(i,j) - sum_k y1(k,j))/m,
+//   y3(k,l) = (R3(k,l) + sum_j y1(k,j))/n.
+// marg64 (one CTA) forms the O(m + n) vectors shared by all
+// slabs, at mv[w * L + index], L = max(m, n):
+//   w = 0: a_j / n - (1/m + 1/n) bb_j        (column part of y1-hat), j < n
+//   w = 1: r3_k / n + T3 / n^2 - (m+n) y1^a_k (row part of y1, times m+n), k < m
+//   w = 2: sum_k y1(k,j)                      (for y2), j < n
+//   w = 3: sum_j y1(k,j)                      (for y3), k < m
+// pieces64 then forms the slab's entries with products only
+// (FP64 division is slow on this part; reciprocals are taken once).
+// Reciprocals of a cycle (FP64 divisions take hundreds of cycles here: formed
+// once by the caller).
+struct Recip64 {
+    double is, im, in_, imn, dl, iw;
+};
+__device__ __forceinline__ Recip64 recip64(int mi, int ni, double sigma) {
+    const double m = mi, n = ni;
+    Recip64 r;
+    r.is = 1.0 / sigma;
+    r.in_ = 1.0 / n;
+    r.im = 1.0 / m;
+    r.imn = 1.0 / (m + n);
+    r.dl = (1.0 - r.in_) / (m + 1.0);
+    r.iw = 1.0 / (r.im - r.dl);                    // 1/w, w = 1/m - (1-1/n)/(m+1)
+    return r;
+}
+
+// The O(m + n) vectors mv of Prop. 3 in FP64 from T1, T2, P1, P2 (the first four
+// of the 7 L doubles sv); cs: column partials of the delta.  One CTA.
+__device__ __forceinline__ void marg64(const HotInst& I, const Recip64& R, const double* cs, double* mv, double* sv,
+                                       double* s_red) {
+    const int mi = I.m, ni = I.n, L = g_L(I);
+    const double m = mi, n = ni;
+    const double is = R.is, in_ = R.in_, im = R.im, imn = R.imn, dl = R.dl, iw = R.iw;
+    double* T1 = sv;
+    double* T2 = sv + L;
+    double* P1 = sv + 2 * L;
+    double* P2 = sv + 3 * L;
+    double* cm = sv + 4 * L;
+    double* rm = sv + 5 * L;
+    double* ss = sv + 6 * L;
+    for (int q = threadIdx.x; q < ni; q += blockDim.x) cm[q] = I.colmu1[q];
+    for (int q = threadIdx.x; q < mi; q += blockDim.x) rm[q] = I.rowmu2[q];
+    // the dropped (m, n) row of eq. (7): column n-1 of the last f2 slab
+    const int sl = g_nslab(I) - 1;
+    const double kap_last =
+        sum_bands(cs + g_colp(I, sl, 0) + (ni - 1), (size_t)ni, I.nb2, I.kapa[g_row(I, sl) + (ni - 1)]);
+    const double mu_last = I.mu2[(size_t)(mi - 1) * ni + (ni - 1)];
+    __syncthreads();
+    auto A_ = [&](int j) { return -(T1[j] - P2[j]) * is; };
+    auto B_ = [&](int j) { return (cm[j] - T1[j]) * is; };
+    auto R3_ = [&](int k) {
+        double r = (rm[k] - T2[k]) * is;
+        if (k == mi - 1) r -= (mu_last - kap_last) * is;
+        return r;
+    };
+    double red[3] = {0.0, 0.0, 0.0}, one[1];
+    for (int j = threadIdx.x; j < ni; j += blockDim.x) {
+        red[0] += A_(j);
+        red[1] += B_(j);
+    }
+    for (int k = threadIdx.x; k < mi; k += blockDim.x) red[2] += R3_(k);
+    block_sum<3>(red, s_red);
+    const double Asum = red[0], Bsum = red[1], T3 = red[2];
+    one[0] = 0.0;
+    for (int k = threadIdx.x; k < mi; k += blockDim.x) {
+        const double rowR1 = -(P1[k] - T2[k]) * is;
+        const double s = (rowR1 + Asum * in_ - (im + in_) * Bsum + R3_(k) + T3 * in_) * imn;   // s_k
+        ss[k] = s;
+        one[0] += (k == mi - 1 ? dl : im) * s;
+    }
+    block_sum<1>(one, s_red);
+    const double ds = one[0];
+    one[0] = 0.0;
+    for (int k = threadIdx.x; k < mi; k += blockDim.x) {
+        const double dq = (k == mi - 1 ? dl : im);
+        one[0] += -dq * ss[k] - dq * ds * iw;       // 1^T W-hat s
+    }
+    block_sum<1>(one, s_red);
+    const double tsum = one[0];
+    const double yasum = tsum + m * tsum * in_;    // 1^T y1^a over k < m
+    for (int k = threadIdx.x; k < mi; k += blockDim.x) {
+        const double dq = (k == mi - 1 ? dl : im);
+        const double ya = -dq * ss[k] - dq * ds * iw + tsum * in_;   // y1^a_k
+        mv[L + k] = R3_(k) * in_ + T3 * in_ * in_ - (m + n) * ya;
+        mv[3 * L + k] = ss[k] - n * ya;
+    }
+    for (int j = threadIdx.x; j < ni; j += blockDim.x) {
+        const double aq = A_(j), bq = B_(j);
+        mv[j] = aq * in_ - (im + in_) * bq;
+        mv[2 * L + j] = (aq - bq + T3 * in_) * in_ - yasum;
+    }
+}
+
+// The slab's pieces, in FP64: entries of dy = y-bar - y0 (dab) and of y-bar
+// itself (ab) for its rows [r0, r0 + nr) and, with cols, its columns (from the
+// slab's side on).  rs, cs: row sums and column partials of the delta; mv: the
+// vectors of marg64.  The anchor part of R (row sums and column totals of u) is
+// formed once per cycle by k_anchor.  CHECK: the slab's share of <b, y> (when it
+// has the columns) and max |A^T y|.
+template <bool CHECK>
+__device__ __forceinline__ void pieces64(const HotInst& I, const Recip64& R, int slab, int r0, int nr, bool first,
+                                         const double* __restrict__ rs, const double* __restrict__ cs,
+                                         const double* __restrict__ mv, double* ab, double* dab, double* s_red,
+                                         float* s_max) {
+    const int mi = I.m, ni = I.n, L = g_L(I), Ls = g_side(I, slab), nb = g_nb(I, slab);
+    const double is = R.is, im = R.im, in_ = R.in_, imn = R.imn;
+    const double* __restrict__ R1a = I.R1a + g_row(I, slab);
+    const double* __restrict__ kapa = I.kapa + g_row(I, slab);
+    const double* __restrict__ ab0 = I.ab0 + 2 * g_row(I, slab);
+    const size_t f2 = (size_t)ni * mi;            // first row of the f2 half
+    const bool f1 = slab < ni;
+    float ymax = 0.f;
+    double dob = 0.0;
+    // idx < Ls: alpha (row) entries, idx >= Ls: beta (column) entries; returns the full piece
+    auto put = [&](int idx, double dv) -> double {
+        dab[idx] = dv;
+        const double full = ab0[idx] + dv;
+        ab[idx] = full;
+        if (CHECK) ymax = fmaxf(ymax, fabsf((float)full));
+        return full;
+    };
+    for (int r = r0 + (int)threadIdx.x; r < r0 + nr; r += kThreads) {
+        const int j = f1 ? slab : r, k = f1 ? r : slab - ni;
+        const double R1 = R1a[r] - (__ldcg(rs + (size_t)j * mi + k) - __ldcg(rs + f2 + (size_t)k * ni + j)) * is;
+        const double y1 = (R1 + mv[j] + mv[L + k]) * imn;              // y1(k, j)
+        put(r, f1 ? y1 : -y1);                                         // A2 = -1_n^T kron I_M
+    }
+    const double sy = f1 ? mv[2 * L + slab] : mv[3 * L + slab - ni];
+    for (int c = threadIdx.x; c < Ls; c += kThreads) {
+        if (!f1 && slab == ni + mi - 1 && c == ni - 1) {
+            put(Ls + c, 0.0);                                          // no row: y3(m, n) = 0
+            continue;
+        }
+        double kd = 0.0;                                               // column total of the delta over the bands
+        for (int b = 0; b < nb; ++b) kd += __ldcg(cs + g_colp(I, slab, 0) + (size_t)b * Ls + c);
+        const double kap = kapa[c] + kd;
+        const double mu = f1 ? I.mu1[(size_t)c * ni + slab] : I.mu2[(size_t)(slab - ni) * ni + c];
+        const double full = f1 ? put(Ls + c, ((mu - kap) * is - sy) * im)       // y2(i, j)
+                               : put(Ls + c, ((mu - kap) * is + sy) * in_);     // y3(k, l)
+        if (CHECK) dob += mu * full;                                   // <b, y>: mu1 . y2, mu2 . y3
+    }
+    if (CHECK) {
+        double red[1] = {dob};
+        block_sum<1>(red, s_red);
+        const float bm = block_max(ymax, s_max);
+        if (threadIdx.x == 0) {
+            if (first) I.dobj_part[slab] = red[0];
+            atomicMax(&I.ctl->ymax_bits, __float_as_uint(bm));
+        }
+    }
+}
+
 }  // namespace hot

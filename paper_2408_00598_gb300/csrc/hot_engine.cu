@@ -117,11 +117,16 @@ int validate_pair(const double* mu, const double* nu, int m, int n, int space, i
     return HOT_OK;
 }
 
-constexpr size_t kGroupStateBytes = (size_t)120 << 20;   // u and one delta
-// k_group32 or the chain of kernels: the group kernel holds one column per
-// thread and one round of slab sums (sides up to 256).
+// k_group32 / k_group64 or the chain of kernels.  FP32: sides up to 256 (one
+// column per thread, one round of slab sums) while u and the delta fit in L2:
+// 192 x 192 (108 MB) 59.8 us per iteration against the chain's 64.7, 256 x 256
+// (256 MB) 114 against 99, since the chain's sweep keeps more CTAs per SM.
+// FP64 (u and two deltas): 96 x 96 (40 MB) 70 against 78 us, 127 x 100 (66 MB) 108
+// against 112, 128 x 128 (96 MB) 143 against 134.
+constexpr size_t kGroupStateBytes = (size_t)120 << 20, kGroupStateBytes64 = (size_t)72 << 20;
 static int group_rule(const Inst& I) {
-    return !I.fp64 && std::max(I.m, I.n) <= kMaxGroupSide && I.big_bytes / 5 * 2 <= kGroupStateBytes ? 1 : 0;
+    if (I.fp64) return std::max(I.m, I.n) <= kMaxGroupSide64 && I.big_bytes / 5 * 3 <= kGroupStateBytes64 ? 1 : 0;
+    return std::max(I.m, I.n) <= kMaxGroupSide && I.big_bytes / 5 * 2 <= kGroupStateBytes ? 1 : 0;
 }
 
 // Groups of CTAs for one launch of k_group32.  An iteration of an instance
@@ -129,11 +134,11 @@ static int group_rule(const Inst& I) {
 // takes the smallest time in which every instance fits into the grid: large
 // ones get as many CTAs as they need, small ones share a CTA (group size 1).
 GroupPlan plan_groups(const std::vector<int>& inst, const std::vector<int>& tiles, const std::vector<int>& elems,
-                      int grid) {
+                      int grid, int fp64) {
     GroupPlan P;
     const int n = (int)inst.size();
     const double wait = 4.0, self = 1.5;                      // microseconds: two waits and the stage; the stage alone
-    auto tile_us = [&](int q) { return 0.9 + elems[q] * 0.00015; };
+    auto tile_us = [&](int q) { return 0.9 + elems[q] * (fp64 ? 0.003 : 0.00015); };
     std::vector<int> order(n);
     for (int q = 0; q < n; ++q) order[q] = q;
     std::stable_sort(order.begin(), order.end(),
@@ -248,10 +253,12 @@ int inst_create(const PairHost& p, int fp64, const hot_config& cfg, double tol, 
     const size_t o_vec2 = take(vec2_entries(m, n) * F2);
     const size_t o_dab2 = take(4 * MN * F2);
     const size_t o_stg2 = take(4 * (size_t)L * F2);
+    const size_t o_rsb = fp64 ? take(2 * MN * 8) : 0;
+    const size_t o_csb = fp64 ? take(CP * 8) : 0;
     const size_t o_rs2b = take(2 * MN * F2);
     const size_t o_cs32b = fp64 ? 0 : take(CP * 4);
     const size_t o_tp = fp64 ? 0 : take((size_t)NS * sizeof(float4));
-    const size_t o_gcount = fp64 ? 0 : take(2 * sizeof(unsigned int));
+    const size_t o_gcount = take(2 * sizeof(unsigned int));
     const size_t o_vcnt = take(sizeof(unsigned int));
     const size_t o_zero_end = off;                 // everything above starts at 0
     const size_t o_mu1f = take(MN * F2);
@@ -403,7 +410,9 @@ int inst_create(const PairHost& p, int fp64, const hot_config& cfg, double tol, 
     d.rs2b = fp64 ? nullptr : (float2*)(sm + o_rs2b);
     d.cs32b = fp64 ? nullptr : (float*)(sm + o_cs32b);
     d.tp = fp64 ? nullptr : (float4*)(sm + o_tp);
-    d.gcount = fp64 ? nullptr : (unsigned int*)(sm + o_gcount);
+    d.gcount = (unsigned int*)(sm + o_gcount);
+    d.rsb = fp64 ? (double*)(sm + o_rsb) : nullptr;
+    d.cs_partb = fp64 ? (double*)(sm + o_csb) : nullptr;
     d.mu1f = fp64 ? nullptr : (float2*)(sm + o_mu1f);
     d.mu2f = fp64 ? nullptr : (float2*)(sm + o_mu2f);
     d.cm2 = fp64 ? nullptr : (float2*)(sm + o_cm2);
@@ -558,7 +567,7 @@ int Batch::reserve(int n) {
     d_gent = nullptr;
     h_gstart = nullptr;
     h_gent = nullptr;
-    ggrid = fp64 ? 0 : group_grid();
+    ggrid = group_grid(fp64);
     HOT_CK(cudaMalloc(&d_gstart, sizeof(int) * (ggrid + 1)));
     HOT_CK(cudaMalloc(&d_gent, sizeof(int4) * (ggrid + ncap)));
     HOT_CK(cudaMallocHost(&h_gstart, sizeof(int) * (ggrid + 1)));
@@ -614,7 +623,7 @@ int Batch::set_instances(const std::vector<Inst*>& v, cudaStream_t st, bool grou
             if (v[i]->ctl_host.status == ST_RUNNING) {
                 gi.push_back(i);
                 gt.push_back(tiles);
-                ge.push_back((int)(v[i]->big_bytes / 20 / tiles));
+                ge.push_back((int)(v[i]->big_bytes / (fp64 ? 40 : 20) / tiles));
             }
         } else {
             ++n_chain;
@@ -662,7 +671,7 @@ int Batch::set_instances(const std::vector<Inst*>& v, cudaStream_t st, bool grou
     h_running[0] = running;
     h_running[1] = 0;
     if (n_group > 0) {
-        const GroupPlan gp = plan_groups(gi, gt, ge, ggrid);
+        const GroupPlan gp = plan_groups(gi, gt, ge, ggrid, fp64);
         std::copy(gp.start.begin(), gp.start.end(), h_gstart);
         std::copy(gp.entries.begin(), gp.entries.end(), h_gent);
         HOT_CK(cudaMemcpyAsync(d_gstart, h_gstart, sizeof(int) * gp.start.size(), cudaMemcpyHostToDevice, st));
@@ -690,7 +699,7 @@ int Batch::launches() const {
 // of kernels for the others; with ev, an event pair around the sweep of
 // iteration timed_iter().
 void Batch::launch_iterations(cudaStream_t st, cudaEvent_t* ev) const {
-    if (n_group > 0) launch_group(d_work, ggrid, K, group_blocks(), a1, a2, a3, gpad != 0, st);
+    if (n_group > 0) launch_group(d_work, ggrid, fp64, K, group_blocks(), a1, a2, a3, gpad != 0, st);
     if (n_chain == 0) return;
     for (int j = 0; j < K; ++j) {
         launch_solve_kernels(d_work, ld, fp64, j, j == K - 1, n_chain == 1, st);

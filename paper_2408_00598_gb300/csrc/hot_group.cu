@@ -75,6 +75,10 @@ struct GroupSmem {
     DF sm1, sm2;                          // the marginals' sums
     P32 p[64];                            // of every iteration of the block (check_every <= 64)
     int dead;
+    // buffers of the block end
+    __device__ double* rows() { return reinterpret_cast<double*>(row); }      // row and xrow
+    __device__ double* cols() { return reinterpret_cast<double*>(col); }      // col and xcol
+    __device__ double* reds() { return reinterpret_cast<double*>(red); }
 };
 
 // All CTAs of the group have arrived for the `epoch`-th time in this launch
@@ -86,7 +90,8 @@ struct GroupSmem {
 // (through L2, __ldcg).  Without the __syncwarp the first warp stayed split
 // after the poll, and what it runs alone next (group_stage) took three times
 // as long.
-__device__ __forceinline__ bool group_wait(GroupSmem& s, int G, unsigned epoch, int* err) {
+template <typename S>
+__device__ __forceinline__ bool group_wait(S& s, int G, unsigned epoch, int* err) {
     __syncthreads();
     if (G == 1) return true;
     if (threadIdx.x == 0) {
@@ -540,23 +545,25 @@ struct BlockRule {
     int K;
     double a1, a2, a3;
 };
-__device__ __noinline__ bool group_block_end(GroupSmem& s, const WorkDev* W, int inst, int rank, int G,
+template <typename T, typename S>
+__device__ __noinline__ bool group_block_end(S& s, const WorkDev* W, int inst, int rank, int G,
                                              unsigned& epoch, BlockRule rule) {
     const HotInst& I = s.I;
-    double* s_row = reinterpret_cast<double*>(s.row);        // row and xrow
-    double* s_col = reinterpret_cast<double*>(s.col);        // col and xcol
-    double* s_red = reinterpret_cast<double*>(s.red);
+    constexpr bool F32 = std::is_same<T, float>::value;
+    double* s_row = s.rows();
+    double* s_col = s.cols();
+    double* s_red = s.reds();
     const int nt = g_ntiles(I);
     if (!group_wait(s, G, ++epoch, W->err)) return false;
 #pragma unroll 1
-    for (int c = rank; c < I.n_k1 + I.n_achunk + I.n_kc; c += G) {
-        if (c < I.n_k1) residual_chunk<true>(I, c, s_red);
-        else if (c < I.n_k1 + I.n_achunk) objective_chunk(I, c - I.n_k1, s.red, s.col);
-        else tile_chunk(I, c - I.n_k1 - I.n_achunk, s.red);
+    for (int c = rank; c < I.n_k1 + (F32 ? I.n_achunk + I.n_kc : 0); c += G) {
+        if (c < I.n_k1) residual_chunk<F32>(I, c, s_red);
+        else if (c < I.n_k1 + I.n_achunk) objective_chunk(I, c - I.n_k1, reinterpret_cast<float2*>(s_red), reinterpret_cast<float*>(s_col));
+        else tile_chunk(I, c - I.n_k1 - I.n_achunk, reinterpret_cast<float2*>(s_red));
         __syncthreads();
     }
     if (!group_wait(s, G, ++epoch, W->err)) return false;
-    if (rank == 0) check_instance<true>(I, W, inst, rule.K, rule.a1, rule.a2, rule.a3, s_red);
+    if (rank == 0) check_instance<F32>(I, W, inst, rule.K, rule.a1, rule.a2, rule.a3, s_red);
     if (!group_wait(s, G, ++epoch, W->err)) return false;
     const int status = __ldcg(&I.ctl->status), restart = __ldcg(&I.ctl->restart_pending);
     auto tiles = [&](auto mode) {
@@ -564,20 +571,20 @@ __device__ __noinline__ bool group_block_end(GroupSmem& s, const WorkDev* W, int
         for (int t = rank; t < nt; t += G) {
             int slab, band;
             g_tile_slab(I, t, slab, band);
-            restart_tile<float, decltype(mode)::value>(I, slab, band, s_row, s_col, s_red);
+            restart_tile<T, decltype(mode)::value>(I, slab, band, s_row, s_col, s_red);
             __syncthreads();
         }
     };
     if (status != ST_RUNNING) {
         tiles(std::integral_constant<int, 2>());             // x-bar and <c, d> of the final iteration
         if (!group_wait(s, G, ++epoch, W->err)) return false;
-        if (rank == 0) end_instance(I, s.red);
+        if (rank == 0) end_instance(I, reinterpret_cast<float2*>(s_red));
         return false;
     }
     if (!restart) return true;
     tiles(std::integral_constant<int, 0>());
     if (!group_wait(s, G, ++epoch, W->err)) return false;
-    if (rank == 0) sigma_instance<true>(I, s_red);
+    if (rank == 0) sigma_instance<F32>(I, s_red);
     if (!group_wait(s, G, ++epoch, W->err)) return false;
     tiles(std::integral_constant<int, 1>());
     if (!group_wait(s, G, ++epoch, W->err)) return false;
@@ -698,14 +705,14 @@ __device__ __forceinline__ void group_instance(GroupSmem& s, const WorkDev* __re
         }
     }
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-    if (!group_block_end(s, W, inst, rank, G, epoch, rule)) return;
+    if (!group_block_end<float>(s, W, inst, rank, G, epoch, rule)) return;
   }
 }
 
-template <bool PAD>
-__global__ void __launch_bounds__(kThreads, 2) k_group32(const WorkDev* __restrict__ W, int blocks, BlockRule rule) {
-    extern __shared__ __align__(16) unsigned char s_raw[];
-    GroupSmem& s = *reinterpret_cast<GroupSmem*>(s_raw);
+// The entries of one CTA: each names an instance, the CTA's rank in its group
+// and the group's size.  run(s, entry) takes the instance through its blocks.
+template <typename S, typename F>
+__device__ __forceinline__ void group_entries(S& s, const WorkDev* __restrict__ W, F run) {
     const int tid = threadIdx.x;
     const int e0 = W->gstart[blockIdx.x], e1 = W->gstart[blockIdx.x + 1];
     if (tid == 0) s.dead = 0;
@@ -719,7 +726,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_group32(const WorkDev* __restri
             reinterpret_cast<double*>(&s.I)[q] = reinterpret_cast<const double*>(src)[q];
         __syncthreads();
         if (s.I.ctl->status != ST_RUNNING) continue;   // the same for the whole group
-        group_instance<PAD>(s, W, ge.x, ge.y, ge.z, blocks, rule);
+        run(ge);
         asm volatile("cp.async.wait_group 0;\n" ::: "memory");
         if (ge.z > 1 && tid == 0 && s.dead == 0) {
             // the last CTA to leave (all have left their waits) clears the counters for the next launch
@@ -732,49 +739,174 @@ __global__ void __launch_bounds__(kThreads, 2) k_group32(const WorkDev* __restri
     }
 }
 
+template <bool PAD>
+__global__ void __launch_bounds__(kThreads, 2) k_group32(const WorkDev* __restrict__ W, int blocks, BlockRule rule) {
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    GroupSmem& s = *reinterpret_cast<GroupSmem*>(s_raw);
+    group_entries(s, W, [&](int4 ge) { group_instance<PAD>(s, W, ge.x, ge.y, ge.z, blocks, rule); });
+}
+
+// -------------------------------------------------------------- k_group64 --
+// The same for FP64 mode: slab sums (k_vec's), wait, the vectors of Prop. 3 in
+// every CTA (marg64), then per tile the pieces (pieces64) and the sweep
+// (sweep64_tile), wait; the block end.  The arithmetic and its order are the
+// chain's (k_vec, k_marg, k_alpha, k_sweep64).  us per iteration of a solve,
+// chain -> group: 16 x 16 31.4 -> 21.9, 64 x 64 58 -> 47, 96 x 96 80 -> 71; bound by
+// FP64 latency (about 60 cycles an operation, 440 a conversion) and the waits.
+struct Group64Smem {
+    Sweep64Smem sw;
+    double red[8 * 32];
+    double sv[7 * kMaxGroupSide64];        // T1 T2 P1 P2, then the work vectors of marg64
+    double mv[4 * kMaxGroupSide64];
+    double ab[2 * kMaxGroupSide64], dab[2 * kMaxGroupSide64];   // pieces of the tile's slab
+    float mx[32];
+    HotInst I;
+    Recip64 R;
+    P64 p[64];
+    int dead;
+    __device__ double* rows() { return sw.row; }             // row and xrow
+    __device__ double* cols() { return sw.col; }             // col and xcol
+    __device__ double* reds() { return red; }
+};
+
+// T1[j], T2[k], P1[k], P2[j] (k_vec's order), one warp; valid in lane 0.
+__device__ __forceinline__ double vec64(const HotInst& I, const double* __restrict__ rs, int q, int lane, int& out) {
+    const int m = I.m, n = I.n, L = g_L(I), f2 = n * m;      // f2: first row of the f2 half
+    int at, step, len;
+    if (q < n) {                                             // T1[j]: f1 slab j, its m rows
+        at = q * m, step = 1, len = m, out = q;
+    } else if ((q -= n) < m) {                               // T2[k]: f2 slab k, its n rows
+        at = f2 + q * n, step = 1, len = n, out = L + q;
+    } else if ((q -= m) < m) {                               // P1[k]: row k of every f1 slab
+        at = q, step = m, len = n, out = 2 * L + q;
+    } else {                                                 // P2[j]: row j of every f2 slab
+        q -= m;
+        at = f2 + q, step = n, len = m, out = 3 * L + q;
+    }
+    double acc = 0.0;
+#pragma unroll 4
+    for (int t = lane; t < len; t += 32) acc += __ldcg(rs + at + t * step) + I.rs0[at + t * step];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    return acc;
+}
+
+__device__ __forceinline__ void group_instance64(Group64Smem& s, const WorkDev* __restrict__ W, int inst, int rank,
+                                                 int G, int blocks, BlockRule rule) {
+    const HotInst& I = s.I;
+    const int K = rule.K;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int L = g_L(I), nv = 2 * (I.m + I.n), nt = g_ntiles(I);
+    unsigned epoch = 0;
+#pragma unroll 1
+    for (int blk = 0; blk < blocks; ++blk) {
+        const double sigma = __ldcg(&I.ctl->sigma);
+        if (tid < K) s.p[tid] = make_p64(sigma, __ldcg(&I.ctl->k) + tid, I.h, I.gadmm, I.relax);
+        if (tid == kThreads - 1) s.R = recip64(I.m, I.n, sigma);
+        __syncthreads();
+#pragma unroll 1
+        for (int it = 0; it < K; ++it) {
+            const bool check = it == K - 1;
+            const double* din = (const double*)(it & 1 ? I.d1 : I.d0);
+            double* dout = (double*)(it & 1 ? I.d0 : I.d1);
+            const double* rs = it & 1 ? I.rsb : I.rs;
+            double* rs_out = it & 1 ? I.rs : I.rsb;
+            const double* cs = it & 1 ? I.cs_partb : I.cs_part;
+            double* cs_out = it & 1 ? I.cs_part : I.cs_partb;
+            if (it > 0 && !group_wait(s, G, ++epoch, W->err)) return;
+#pragma unroll 1
+            for (int q = rank + G * warp; q < nv; q += G * kW) {
+                int out = 0;
+                const double v = vec64(I, rs, q, lane, out);
+                if (lane == 0) __stcg(I.vecs + out, v);
+            }
+            if (!group_wait(s, G, ++epoch, W->err)) return;
+#pragma unroll 1
+            for (int q = tid; q < 4 * L; q += kThreads) s.sv[q] = __ldcg(I.vecs + q);
+            marg64(I, s.R, cs, s.mv, s.sv, s.red);
+            __syncthreads();
+#pragma unroll 1
+            for (int t = rank; t < nt; t += G) {
+                int slab, band;
+                g_tile_slab(I, t, slab, band);
+                const int S = g_side(I, slab), r0 = band * I.TR, nr = min(S, r0 + I.TR) - r0;
+                const size_t o = 2 * g_row(I, slab);
+                if (check) {
+                    pieces64<true>(I, s.R, slab, r0, nr, band == 0, rs, cs, s.mv, s.ab, s.dab, s.red, s.mx);
+                    __syncthreads();
+                    // the block end reads the pieces in global memory
+                    for (int q = tid; q < 2 * S; q += kThreads)
+                        if (q >= S ? band == 0 : q >= r0 && q < r0 + nr) {
+                            I.ab64[o + q] = s.ab[q];
+                            I.dab64[o + q] = s.dab[q];
+                        }
+                    sweep64_tile<true>(I, slab, band, din, dout, s.p[it], s.ab, s.dab, rs_out, cs_out, s.sw);
+                } else {
+                    pieces64<false>(I, s.R, slab, r0, nr, band == 0, rs, cs, s.mv, s.ab, s.dab, s.red, s.mx);
+                    __syncthreads();
+                    sweep64_tile<false>(I, slab, band, din, dout, s.p[it], s.ab, s.dab, rs_out, cs_out, s.sw);
+                }
+                __syncthreads();
+            }
+        }
+        if (!group_block_end<double>(s, W, inst, rank, G, epoch, rule)) return;
+    }
+}
+
+__global__ void __launch_bounds__(kThreads, 2) k_group64(const WorkDev* __restrict__ W, int blocks, BlockRule rule) {
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    Group64Smem& s = *reinterpret_cast<Group64Smem*>(s_raw);
+    group_entries(s, W, [&](int4 ge) { group_instance64(s, W, ge.x, ge.y, ge.z, blocks, rule); });
+}
+
 }  // namespace
 
 static_assert(sizeof(HotInst) % 8 == 0 && sizeof(CycleK) % 8 == 0, "descriptors are copied in 8-byte words");
-
-size_t group_smem() { return sizeof(GroupSmem); }
 
 cudaError_t group_init() {
     cudaError_t e =
         cudaFuncSetAttribute(k_group32<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GroupSmem));
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_group32<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GroupSmem));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_group64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Group64Smem));
     return e;
 }
 
-int group_grid() {
-    static int cache[64];                    // per device ordinal; 0 = not yet queried
+int group_grid(int fp64) {
+    static int cache[2][64];                 // per precision and device ordinal; 0 = not yet queried
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-    if (cache[dev] == 0) {
+    int& c = cache[fp64 ? 1 : 0][dev];
+    if (c == 0) {
         int sms = 0, a = 0, b = 0;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (group_init() != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_group32<false>, kThreads, sizeof(GroupSmem)) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_group32<true>, kThreads, sizeof(GroupSmem)) != cudaSuccess)
-            return 0;
-        cache[dev] = sms * (a < b ? a : b);
+        if (group_init() != cudaSuccess) return 0;
+        cudaError_t e = fp64 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_group64, kThreads, sizeof(Group64Smem))
+                             : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_group32<false>, kThreads, sizeof(GroupSmem));
+        b = a;
+        if (e == cudaSuccess && !fp64)
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_group32<true>, kThreads, sizeof(GroupSmem));
+        if (e != cudaSuccess) return 0;
+        c = sms * (a < b ? a : b);
     }
-    return cache[dev];
+    return c;
 }
 
-void launch_group(const WorkDev* w, int grid, int K, int blocks, double a1, double a2, double a3, bool pad,
+void launch_group(const WorkDev* w, int grid, int fp64, int K, int blocks, double a1, double a2, double a3, bool pad,
                   cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = sizeof(GroupSmem);
+    cfg.dynamicSmemBytes = fp64 ? sizeof(Group64Smem) : sizeof(GroupSmem);
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeCooperative;       // the CTAs of a group wait on one another
     at[0].val.cooperative = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, pad ? k_group32<true> : k_group32<false>, w, blocks, BlockRule{K, a1, a2, a3});
+    const BlockRule rule{K, a1, a2, a3};
+    cudaLaunchKernelEx(&cfg, fp64 ? k_group64 : pad ? k_group32<true> : k_group32<false>, w, blocks, rule);
 }
 
 }  // namespace hot

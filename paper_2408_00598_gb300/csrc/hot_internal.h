@@ -41,6 +41,7 @@ constexpr int kAlphaChunk = kThreads * kAPT;
 constexpr int kMaxTR = 128;            // FP32 tiles: TR * max(m, n) <= kRowSmemBytes / 4
 constexpr int kMaxTileElems = 16384;   // FP32 tiles: TR * (longer row pitch) <= this
 constexpr int kMaxGroupSide = 256;     // k_group32: longest side (one column per thread)
+constexpr int kMaxGroupSide64 = 128;   // k_group64: longest side
 constexpr int kMaxGroup = 512;         // k_group32: most CTAs of one instance
 
 enum : int {
@@ -161,9 +162,12 @@ struct HotInst {
     float2* vec2;          // rows of max(m, n): T1, T2, then ceil(n/64) partials of P1 and ceil(m/64) of P2, of u + d
     float2* dab2;          // [4mn] pieces of A^T(y-bar - y0)
     float2* stg2;          // [4][max(m, n)] Prop. 3 stage of the current iteration: mvA, mvS, sy, sp (k_stage32)
-    // k_group32 only: the other row-sum and column-partial buffers (odd
-    // iterations read them), T and P of every slab, the arrival counter
-    float2* rs2b;          // [2mn]
+    // k_group32 and k_group64 only: the other row-sum and column-partial
+    // buffers (odd iterations read them), T and P of every slab (FP32 mode),
+    // the arrival counter
+    double* rsb;           // FP64 mode: [2mn], and
+    double* cs_partb;      // [slab][band][column]
+    float2* rs2b;          // FP32 mode: [2mn], and
     float* cs32b;          // [slab][band][column]
     float4* tp;            // [m + n]
     unsigned int* gcount;  // [2] arrivals and departures of the group's CTAs in the running launch (0 between launches)
@@ -305,10 +309,10 @@ void launch_solve_kernels(const WorkDev* w, const LaunchDims& ld, int fp64, int 
 void launch_sweep(const WorkDev* w, const LaunchDims& ld, int fp64, int j, bool check, bool pad, cudaStream_t st);
 void launch_block_end(const WorkDev* w, const LaunchDims& ld, int fp64, int K, double a1, double a2, double a3,
                       cudaStream_t st);
-// k_group32 (hot_group.cu): up to `blocks` check blocks of every grouped instance in one cooperative launch
-void launch_group(const WorkDev* w, int grid, int K, int blocks, double a1, double a2, double a3, bool pad,
+// k_group32, k_group64 (hot_group.cu): up to `blocks` check blocks of every grouped instance in one cooperative launch
+void launch_group(const WorkDev* w, int grid, int fp64, int K, int blocks, double a1, double a2, double a3, bool pad,
                   cudaStream_t st);
-int group_grid();                          // CTAs resident at once on the current device (0: not available)
+int group_grid(int fp64);                  // CTAs resident at once on the current device (0: not available)
 cudaError_t group_init();
 LaunchDims make_launch_dims(int device, int fp64);
 // resident CTAs of the (non-check) sweep on the current device

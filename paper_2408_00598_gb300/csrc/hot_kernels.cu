@@ -137,24 +137,6 @@ __global__ void __launch_bounds__(kThreads) k_vec(const WorkDev* __restrict__ W)
     }
 }
 
-// ---------------------------------------------------------- k_marg/k_alpha --
-// Prop. 3 on R' = (b - A(u + d))/sigma, the right-hand side whose solution is
-// dy = y-bar - y0: with v = sigma g0 + u + d, the right-hand side of
-// eq. (update:y) is R = b/sigma - A(v/sigma - c) = AA^T y0 + R'.  R' comes
-// from the slab sums of u + d.  With j < n and k < m:
-//   a_j = sum_k R1(k,j), bb_j = sum_i R2(i,j), r3_k = sum_l R3(k,l), T3 = sum r3,
-//   y1-hat(k,j) = (R1(k,j) + a_j/n - (1/m+1/n) bb_j + r3_k/n + T3/n^2)/(m+n),
-//   s_k = sum_j y1-hat(k,j),  t = W-hat s,  y1^a = t + (1^T t / n) 1,
-//   y1 = y1-hat - y1^a,  y2(i,j) = (R2(i,j) - sum_k y1(k,j))/m,
-//   y3(k,l) = (R3(k,l) + sum_j y1(k,j))/n.
-// k_marg (one CTA per instance) forms the O(m + n) vectors shared by all
-// slabs, at mv[w * L + index], L = max(m, n):
-//   w = 0: a_j / n - (1/m + 1/n) bb_j        (column part of y1-hat), j < n
-//   w = 1: r3_k / n + T3 / n^2 - (m+n) y1^a_k (row part of y1, times m+n), k < m
-//   w = 2: sum_k y1(k,j)                      (for y2), j < n
-//   w = 3: sum_j y1(k,j)                      (for y3), k < m
-// k_alpha (one CTA per slab) then forms the slab's entries with products only
-// (FP64 division is slow on this part; reciprocals are taken once).
 __global__ void __launch_bounds__(kThreads) k_marg(const WorkDev* __restrict__ W) {
     pdl_enter();
     extern __shared__ double sv[];                   // 7 L: T1 T2 P1 P2 colmu1 rowmu2, then s
@@ -162,73 +144,10 @@ __global__ void __launch_bounds__(kThreads) k_marg(const WorkDev* __restrict__ W
     const int ninst = W->ninst;
     for (int inst = blockIdx.x; inst < ninst; inst += gridDim.x) {
         const HotInst& I = W->inst[inst];
-        if (I.ctl->status != ST_RUNNING) continue;     // block-uniform
-        const int mi = I.m, ni = I.n, L = g_L(I);
-        const double m = mi, n = ni;
-        const double is = 1.0 / I.ctl->sigma;
-        const double in_ = 1.0 / n, im = 1.0 / m, imn = 1.0 / (m + n);
-        double* T1 = sv;
-        double* T2 = sv + L;
-        double* P1 = sv + 2 * L;
-        double* P2 = sv + 3 * L;
-        double* cm = sv + 4 * L;
-        double* rm = sv + 5 * L;
-        double* ss = sv + 6 * L;
+        if (I.grp || I.ctl->status != ST_RUNNING) continue;     // block-uniform
+        const int L = g_L(I);
         for (int q = threadIdx.x; q < 4 * L; q += blockDim.x) sv[q] = I.vecs[q];
-        for (int q = threadIdx.x; q < ni; q += blockDim.x) cm[q] = I.colmu1[q];
-        for (int q = threadIdx.x; q < mi; q += blockDim.x) rm[q] = I.rowmu2[q];
-        // the dropped (m, n) row of eq. (7): column n-1 of the last f2 slab
-        const int sl = g_nslab(I) - 1;
-        const double kap_last =
-            sum_bands(I.cs_part + g_colp(I, sl, 0) + (ni - 1), (size_t)ni, I.nb2, I.kapa[g_row(I, sl) + (ni - 1)]);
-        const double mu_last = I.mu2[(size_t)(mi - 1) * ni + (ni - 1)];
-        __syncthreads();
-        auto A_ = [&](int j) { return -(T1[j] - P2[j]) * is; };
-        auto B_ = [&](int j) { return (cm[j] - T1[j]) * is; };
-        auto R3_ = [&](int k) {
-            double r = (rm[k] - T2[k]) * is;
-            if (k == mi - 1) r -= (mu_last - kap_last) * is;
-            return r;
-        };
-        double red[4] = {0.0, 0.0, 0.0, 0.0};
-        for (int j = threadIdx.x; j < ni; j += blockDim.x) {
-            red[0] += A_(j);
-            red[1] += B_(j);
-        }
-        for (int k = threadIdx.x; k < mi; k += blockDim.x) red[2] += R3_(k);
-        block_sum<4>(red, s_red);
-        const double Asum = red[0], Bsum = red[1], T3 = red[2];
-        const double dl = (1.0 - in_) / (m + 1.0);
-        const double iw = 1.0 / (im - dl);             // 1/w, w = 1/m - (1-1/n)/(m+1)
-        red[0] = red[1] = red[2] = red[3] = 0.0;
-        for (int k = threadIdx.x; k < mi; k += blockDim.x) {
-            const double rowR1 = -(P1[k] - T2[k]) * is;
-            const double s = (rowR1 + Asum * in_ - (im + in_) * Bsum + R3_(k) + T3 * in_) * imn;   // s_k
-            ss[k] = s;
-            red[0] += (k == mi - 1 ? dl : im) * s;
-        }
-        block_sum<4>(red, s_red);
-        const double ds = red[0];
-        red[0] = red[1] = red[2] = red[3] = 0.0;
-        for (int k = threadIdx.x; k < mi; k += blockDim.x) {
-            const double dq = (k == mi - 1 ? dl : im);
-            red[0] += -dq * ss[k] - dq * ds * iw;       // 1^T W-hat s
-        }
-        block_sum<4>(red, s_red);
-        const double tsum = red[0];
-        const double yasum = tsum + m * tsum * in_;    // 1^T y1^a over k < m
-        double* mv = I.mvec;
-        for (int k = threadIdx.x; k < mi; k += blockDim.x) {
-            const double dq = (k == mi - 1 ? dl : im);
-            const double ya = -dq * ss[k] - dq * ds * iw + tsum * in_;   // y1^a_k
-            mv[L + k] = R3_(k) * in_ + T3 * in_ * in_ - (m + n) * ya;
-            mv[3 * L + k] = ss[k] - n * ya;
-        }
-        for (int j = threadIdx.x; j < ni; j += blockDim.x) {
-            const double aq = A_(j), bq = B_(j);
-            mv[j] = aq * in_ - (im + in_) * bq;
-            mv[2 * L + j] = (aq - bq + T3 * in_) * in_ - yasum;
-        }
+        marg64(I, recip64(I.m, I.n, I.ctl->sigma), I.cs_part, I.mvec, sv, s_red);
         __syncthreads();
     }
 }
@@ -257,74 +176,9 @@ __global__ void __launch_bounds__(kThreads) k_alpha(const WorkDev* __restrict__ 
             continue;
         }
         const HotInst& I = W->inst[s_t[0]];
-        const int slab = s_t[1];
-        const int mi = I.m, ni = I.n, L = g_L(I), Ls = g_side(I, slab), nb = g_nb(I, slab);
-        const double m = mi, n = ni;
-        const double is = 1.0 / I.ctl->sigma;
-        const double im = 1.0 / m, in_ = 1.0 / n, imn = 1.0 / (m + n);
-        const double* __restrict__ rs = I.rs;
-        const double* __restrict__ mv = I.mvec;
-        const double* __restrict__ R1a = I.R1a + g_row(I, slab);
-        const double* __restrict__ kapa = I.kapa + g_row(I, slab);
+        const int slab = s_t[1], Ls = g_side(I, slab);
         const size_t o = 2 * g_row(I, slab);
-        const size_t f2 = (size_t)ni * mi;            // first row of the f2 half
-        float ymax = 0.f;
-        double dob = 0.0;
-        // idx < Ls: alpha (row) entries, idx >= Ls: beta (column) entries; returns the full piece
-        auto put = [&](int idx, double dv) -> double {
-            I.dab64[o + idx] = dv;
-            const double full = I.ab0[o + idx] + dv;
-            I.ab64[o + idx] = full;
-            if (CHECK) ymax = fmaxf(ymax, fabsf((float)full));
-            return full;
-        };
-        auto kap_delta = [&](int c) -> double {           // column total of the delta over the bands
-            double k = 0.0;
-            k += sum_bands(I.cs_part + g_colp(I, slab, 0) + c, (size_t)Ls, nb);
-            return k;
-        };
-        if (slab < ni) {
-            const int j = slab;
-            const double colj = mv[j];
-            for (int k = threadIdx.x; k < mi; k += blockDim.x) {
-                const double R1 = R1a[k] - (rs[(size_t)j * mi + k] - rs[f2 + (size_t)k * ni + j]) * is;
-                put(k, (R1 + colj + mv[L + k]) * imn);        // y1(k, j)
-            }
-            const double sy = mv[2 * L + j];
-            for (int i = threadIdx.x; i < mi; i += blockDim.x) {
-                const double kap = kapa[i] + kap_delta(i);
-                const double mu = I.mu1[(size_t)i * ni + j];
-                const double full = put(Ls + i, ((mu - kap) * is - sy) * im);  // y2(i, j)
-                if (CHECK) dob += mu * full;                                    // <b, y>: mu1 . y2
-            }
-        } else {
-            const int k = slab - ni;
-            const double rowk = mv[L + k];
-            for (int j = threadIdx.x; j < ni; j += blockDim.x) {
-                const double R1 = R1a[j] - (rs[(size_t)j * mi + k] - rs[f2 + (size_t)k * ni + j]) * is;
-                put(j, -(R1 + mv[j] + rowk) * imn);            // -y1(k, j): A2 = -1_n^T kron I_M
-            }
-            const double sp = mv[3 * L + k];
-            for (int l = threadIdx.x; l < ni; l += blockDim.x) {
-                if (k == mi - 1 && l == ni - 1) {
-                    put(Ls + l, 0.0);                          // no row: y3(m, n) = 0
-                    continue;
-                }
-                const double kap = kapa[l] + kap_delta(l);
-                const double mu = I.mu2[(size_t)k * ni + l];
-                const double full = put(Ls + l, ((mu - kap) * is + sp) * in_); // y3(k, l)
-                if (CHECK) dob += mu * full;                                    // mu2 . y3
-            }
-        }
-        if (CHECK) {
-            double red[4] = {dob, 0.0, 0.0, 0.0};
-            block_sum<4>(red, s_red);
-            const float bm = block_max(ymax, s_max);
-            if (threadIdx.x == 0) {
-                I.dobj_part[slab] = red[0];
-                atomicMax(&I.ctl->ymax_bits, __float_as_uint(bm));
-            }
-        }
+        pieces64<CHECK>(I, recip64(I.m, I.n, I.ctl->sigma), slab, 0, Ls, true, I.rs, I.cs_part, I.mvec, I.ab64 + o, I.dab64 + o, s_red, s_max);
         __syncthreads();
     }
 }
@@ -534,7 +388,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_alpha32(const WorkDev* __restri
             const DF dv = piece_dv(I, K, slab, idx, a, zero);
             const bool col = idx >= Ls;
             const size_t o = 2 * g_row(I, slab) + idx;
-            dab2[o] = df_st(dv);
+            if (CHECK) dab2[o] = df_st(dv);          // read at the block's end only
             ab32[o] = piece_pack(a, dv, K, I.coord_real);
             if (CHECK) {
                 const DF full = df_add(DF{a.a0.x, a.a0.y}, dv);

@@ -66,6 +66,7 @@ static size_t inst_bytes_estimate(Ctx* ctx, int m, int n, int fp64) {
     const size_t CP = (size_t)n * ((m + tr - 1) / tr) * m + (size_t)m * ((n + tr - 1) / tr) * n;
     // pieces 3 x 32 MN, slab-row sums 5 x 16 MN, marginals 16 MN, column partials 28 CP
     size_t small = MN * (96 + 80 + 16) + CP * 28 + 1024 * 64;
+    if (fp64) small += MN * 16 + CP * 8;                                              // group buffers
     if (!fp64) small += MN * 208 + CP * 4 + (size_t)(m + n) * 16;   // double-float arrays and group buffers of FP32 mode
     return big + small;
 }

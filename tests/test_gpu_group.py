@@ -1,4 +1,4 @@
-"""k_group32 (one kernel per check block for small instances) against the chain of
+"""k_group32 and k_group64 (one kernel for the check blocks of small instances) against the chain of
 kernels: the same iterates and results, bit for bit.
 
 The live sweep timing mode times the chain's kernels and therefore runs the chain at
@@ -50,6 +50,15 @@ def test_group_kernel_equals_the_chain_at_real_positions(m, n):
     mu, nu = syn.make_pair("white", m, 2, n)
     with hot.Context(precision="fp32") as ctx:
         _same(_both(ctx, mu, nu, xs=np.sort(rng.random(m)), ys=np.sort(rng.random(n))))
+
+
+@pytest.mark.parametrize("m,n,kind", [(2, 2, "white"), (3, 2, "white"), (5, 7, "gauss"), (16, 16, "shapes"), (17, 23, "white"),
+                                      (33, 31, "white"), (65, 63, "white"), (20, 90, "white"), (128, 3, "white")])
+def test_fp64_group_kernel_equals_the_chain(m, n, kind):
+    from paper_2408_00598_gb300 import hot
+    mu, nu = syn.make_pair(kind, m, 1, n)
+    with hot.Context(precision="fp64") as ctx:
+        _same(_both(ctx, mu, nu))
 
 
 @pytest.mark.parametrize("check_every", [2, 4, 64])
