@@ -79,13 +79,13 @@ __device__ __forceinline__ void sweep64_tile(const HotInst& I, int slab, int ban
     }
     double k64[kNK] = {0.0, 0.0, 0.0, 0.0, 0.0};
     const double nis = -p.is, rho = p.rho, trs = p.trs, sg = p.s;
+    double un[NV] = {0.0, 0.0}, dn[NV] = {0.0, 0.0};
+    if (active && ro < nr) {                                               // in flight across the barrier
+        VecT<double>::ld(u + (size_t)ro * Sp + c0, un);
+        VecT<double>::ld(din + (size_t)ro * Sp + c0, dn);
+    }
     __syncthreads();
     if (active) {
-        double un[NV], dn[NV];
-        if (ro < nr) {
-            VecT<double>::ld(u + (size_t)ro * Sp + c0, un);
-            VecT<double>::ld(din + (size_t)ro * Sp + c0, dn);
-        }
         for (int r = ro; r < nr; r += P) {
             const double uu[NV] = {un[0], un[1]}, dd[NV] = {dn[0], dn[1]};
             if (r + P < nr) {                                              // the next row's loads
@@ -252,9 +252,19 @@ __device__ __forceinline__ void anchor_slab(const HotInst& I, int slab, double s
 //         (FP32 mode) the tile's share of <c, d> of that iteration, which
 //         completes the reported objective (k_block_end).
 // The check iteration (index K-1, odd) read delta buffer d1.
-template <typename T, int MODE>
+// FP32 mode streams the state through a ring of SLOTS passes per thread in
+// shared memory (u and d; MODE 0 also x_r and z_r), a commit group per pass:
+// more bytes in flight than registers can hold beside the double-float sums.
+// 512 x 512, before -> with the ring: MODE 0 975 -> 737 us (5.8 TB/s of its 16 B per
+// variable), MODE 2 642 -> 572 us, MODE 1 1,450 us either way: its epilogue adds a
+// row's partials in one chain, whose order the iterates depend on.
+constexpr int kRestartSlots = 4;
+__host__ __device__ constexpr size_t restart_ring(int mode) {
+    return (size_t)kRestartSlots * (mode == 0 ? 4 : 2) * kThreads * sizeof(float4);
+}
+template <typename T, int MODE, int SLOTS>
 __device__ __forceinline__ void restart_tile(const HotInst& I, int slab, int band, double* s_row, double* s_col,
-                                             double* s_red) {
+                                             double* s_red, float4* s_ring) {
     using V = VecT<T>;
     constexpr int NV = V::N;
     constexpr bool F32 = std::is_same<T, float>::value;
@@ -316,13 +326,42 @@ __device__ __forceinline__ void restart_tile(const HotInst& I, int slab, int ban
             }
         }
         const float fsig = (float)sig_new;
-        // two rows in flight per thread: the pass streams 16-24 B per variable
-        // and needs the loads of several rows outstanding to reach HBM speed
-#pragma unroll 2
-        for (int r = r0 + ro; r < r1; r += P) {
+        constexpr int NA = MODE == 0 ? 4 : 2;            // arrays in a slot
+        float4* ring = s_ring + threadIdx.x;
+        unsigned long long pol = 0;
+        if constexpr (F32) asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;\n" : "=l"(pol));
+        auto issue = [&](int q, int r) {                 // row r into slot q % SLOTS
+            if constexpr (F32) {
+                if (r < r1) {
+                    const size_t o = (size_t)r * Sp + c0;
+                    float4* p = ring + (q % SLOTS) * NA * kThreads;
+                    cp_async16_ef(p, (const float*)u + o, pol);
+                    cp_async16_ef(p + kThreads, (const float*)d1 + o, pol);
+                    if (MODE == 0 && !origin) {
+                        cp_async16_ef(p + 2 * kThreads, (const float*)xr + o, pol);
+                        cp_async16_ef(p + 3 * kThreads, (const float*)zr + o, pol);
+                    }
+                }
+                cp_async_commit();
+            }
+        };
+#pragma unroll 1
+        for (int q = 0; q < SLOTS - 1; ++q) issue(q, r0 + ro + q * P);
+        int q = 0;
+#pragma unroll 1
+        for (int r = r0 + ro; r < r1; r += P, ++q) {
             T uu[NV], dd[NV], xbv[NV], zbv[NV], rv[NV];
-            V::ld(u + (size_t)r * Sp + c0, uu);
-            V::ld(d1 + (size_t)r * Sp + c0, dd);
+            const float4* slot = ring + (q % SLOTS) * NA * kThreads;
+            if constexpr (F32) {
+                issue(q + SLOTS - 1, r + (SLOTS - 1) * P);
+                cp_async_wait<SLOTS - 1>();
+                const float4 a = slot[0], b = slot[kThreads];
+                uu[0] = a.x, uu[1] = a.y, uu[2] = a.z, uu[3] = a.w;
+                dd[0] = b.x, dd[1] = b.y, dd[2] = b.z, dd[3] = b.w;
+            } else {
+                V::ld(u + (size_t)r * Sp + c0, uu);
+                V::ld(d1 + (size_t)r * Sp + c0, dd);
+            }
             if constexpr (F32) {
                 const float4 a = ab32[r];
                 const float xrow = X32[r];
@@ -352,6 +391,10 @@ __device__ __forceinline__ void restart_tile(const HotInst& I, int slab, int ban
                 if (origin) {
 #pragma unroll
                     for (int e = 0; e < NV; ++e) xo[e] = zo[e] = T(0);
+                } else if constexpr (F32) {
+                    const float4 a = slot[2 * kThreads], b = slot[3 * kThreads];
+                    xo[0] = a.x, xo[1] = a.y, xo[2] = a.z, xo[3] = a.w;
+                    zo[0] = b.x, zo[1] = b.y, zo[2] = b.z, zo[3] = b.w;
                 } else {
                     V::ld(xr + (size_t)r * Sp + c0, xo);
                     V::ld(zr + (size_t)r * Sp + c0, zo);

@@ -57,6 +57,29 @@ __device__ __forceinline__ void block_sum(double (&v)[NV], double* sh) {
     __syncthreads();
 }
 
+// block_sum when only the first n threads hold values: up to a warp of them the
+// other warps' sums are zeros, so the first warp's is the result (the same bits)
+template <int NV>
+__device__ __forceinline__ void block_sum_first(double (&v)[NV], int n, double* sh) {
+    if (n > 32) {
+        block_sum<NV>(v, sh);
+        return;
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int q = 0; q < NV; ++q) v[q] += __shfl_down_sync(0xffffffffu, v[q], o);
+        if (threadIdx.x == 0)
+#pragma unroll
+            for (int q = 0; q < NV; ++q) sh[q] = v[q];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < NV; ++q) v[q] = sh[q];
+}
+
 __device__ __forceinline__ float block_max(float v, float* sh) {
     for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_down_sync(0xffffffffu, v, o));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -262,6 +285,23 @@ template <> struct VecT<double> {
         __stcs(reinterpret_cast<double2*>(p), make_double2(x[0], x[1]));
     }
 };
+
+// Asynchronous global -> shared copies (16 B per thread, cached in L2 only).
+// A thread waits only for its own copies (cp.async.wait_group), so a pipeline
+// in which every thread reads back only what it copied needs no barrier.
+__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
+    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async16_ef(void* smem, const void* gmem, unsigned long long pol) {
+    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;\n" ::"r"(sa), "l"(gmem), "l"(pol) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
+}
 
 // Rows of a P partial (see k_vec32): P1 and P2 are formed from partial sums over
 // blocks of this many rows.
@@ -611,7 +651,7 @@ __device__ __forceinline__ void marg64(const HotInst& I, const Recip64& R, const
         red[1] += B_(j);
     }
     for (int k = threadIdx.x; k < mi; k += blockDim.x) red[2] += R3_(k);
-    block_sum<3>(red, s_red);
+    block_sum_first<3>(red, L, s_red);
     const double Asum = red[0], Bsum = red[1], T3 = red[2];
     one[0] = 0.0;
     for (int k = threadIdx.x; k < mi; k += blockDim.x) {
@@ -620,14 +660,14 @@ __device__ __forceinline__ void marg64(const HotInst& I, const Recip64& R, const
         ss[k] = s;
         one[0] += (k == mi - 1 ? dl : im) * s;
     }
-    block_sum<1>(one, s_red);
+    block_sum_first<1>(one, L, s_red);
     const double ds = one[0];
     one[0] = 0.0;
     for (int k = threadIdx.x; k < mi; k += blockDim.x) {
         const double dq = (k == mi - 1 ? dl : im);
         one[0] += -dq * ss[k] - dq * ds * iw;       // 1^T W-hat s
     }
-    block_sum<1>(one, s_red);
+    block_sum_first<1>(one, L, s_red);
     const double tsum = one[0];
     const double yasum = tsum + m * tsum * in_;    // 1^T y1^a over k < m
     for (int k = threadIdx.x; k < mi; k += blockDim.x) {

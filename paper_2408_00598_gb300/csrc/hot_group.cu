@@ -79,6 +79,7 @@ struct GroupSmem {
     __device__ double* rows() { return reinterpret_cast<double*>(row); }      // row and xrow
     __device__ double* cols() { return reinterpret_cast<double*>(col); }      // col and xcol
     __device__ double* reds() { return reinterpret_cast<double*>(red); }
+    __device__ float4* ring() { return &st[0][0][0]; }                       // kRing slots of two arrays
 };
 
 // All CTAs of the group have arrived for the `epoch`-th time in this launch
@@ -571,7 +572,8 @@ __device__ __noinline__ bool group_block_end(S& s, const WorkDev* W, int inst, i
         for (int t = rank; t < nt; t += G) {
             int slab, band;
             g_tile_slab(I, t, slab, band);
-            restart_tile<T, decltype(mode)::value>(I, slab, band, s_row, s_col, s_red);
+            restart_tile<T, decltype(mode)::value, decltype(mode)::value == 0 ? kRing / 2 : kRing>(I, slab, band, s_row, s_col,
+                                                                                                s_red, s.ring());
             __syncthreads();
         }
     };
@@ -767,6 +769,7 @@ struct Group64Smem {
     __device__ double* rows() { return sw.row; }             // row and xrow
     __device__ double* cols() { return sw.col; }             // col and xcol
     __device__ double* reds() { return red; }
+    __device__ float4* ring() { return nullptr; }            // FP32 mode only
 };
 
 // T1[j], T2[k], P1[k], P2[j] (k_vec's order), one warp; valid in lane 0.

@@ -38,23 +38,6 @@
 
 namespace hot {
 
-// Asynchronous global -> shared copies (16 B per thread, cached in L2 only).
-// A thread waits only for its own copies (cp.async.wait_group), so a pipeline
-// in which every thread reads back only what it copied needs no barrier.
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async16_ef(void* smem, const void* gmem, unsigned long long pol) {
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;\n" ::"r"(sa), "l"(gmem), "l"(pol) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
-
 // Stages of the FP32 sweep pipeline: each holds one pass of P rows
 // (one float4 of u and one of the delta per thread).
 constexpr int kStages = 4;
@@ -802,6 +785,7 @@ __global__ void __launch_bounds__(kThreads, CHECK ? 2 : 3) k_sweep32(const WorkD
 template <typename T, int MODE>
 __global__ void __launch_bounds__(kThreads, 3) k_restart(const WorkDev* __restrict__ W) {
     pdl_enter();
+    extern __shared__ float4 s_ring[];               // FP32 mode: restart_ring<MODE>() passes in flight
     __shared__ double s_row[MODE == 1 ? kRowSmemBytes / 8 * 2 : 1];
     __shared__ double s_col[MODE == 1 ? kThreads * 4 : 1];
     __shared__ double s_red[2 * 32];
@@ -822,7 +806,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_restart(const WorkDev* __restri
         bool go;
         if (MODE == 2) go = I.ctl->just_finished != 0;
         else go = (s_tile[2] == ST_RUNNING) && (s_tile[3] != 0);
-        if (go) restart_tile<T, MODE>(I, tc.slab, tc.band, s_row, s_col, s_red);
+        if (go) restart_tile<T, MODE, kRestartSlots>(I, tc.slab, tc.band, s_row, s_col, s_red, s_ring);
         __syncthreads();
     }
 }
@@ -1043,7 +1027,8 @@ LaunchDims make_launch_dims(int device, int fp64) {
     } else {
         d.grid_tile = occ_grid(k_sweep32<false, false>, sms, kSweepSmem, 8);
         d.grid_tile_chk = occ_grid(k_sweep32<true, false>, sms, kSweepSmemChk, 8);
-        d.grid_rst = std::min(occ_grid(k_restart<float, 0>, sms, 0, 8), occ_grid(k_restart<float, 1>, sms, 0, 8));
+        d.grid_rst = std::min(occ_grid(k_restart<float, 0>, sms, restart_ring(0), 8),
+                              occ_grid(k_restart<float, 1>, sms, restart_ring(1), 8));
         d.grid_slab = occ_grid(k_anchor, sms, 0, 4);
         d.grid_alpha = occ_grid(k_alpha32<true>, sms, 0, 2);
         d.grid_vec = occ_grid(k_vec32<false>, sms, 0, 4);
@@ -1099,6 +1084,12 @@ cudaError_t kernels_init(int device) {
         e = cudaFuncSetAttribute(k_sweep32<false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSweepSmem);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_sweep32<false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSweepSmem);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_restart<float, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)restart_ring(0));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_restart<float, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)restart_ring(1));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_restart<float, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)restart_ring(2));
     if (e == cudaSuccess) e = group_init();
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_marg, cudaFuncAttributeMaxDynamicSharedMemorySize, 7 * kMaxS * 8);
     return e;
@@ -1162,11 +1153,11 @@ void launch_block_end(const WorkDev* w, const LaunchDims& ld, int fp64, int K, d
     } else {
         launch(ld, k_kkt1<true>, ld.grid_k1, 0, st, w);
         launch(ld, k_check<true>, ld.grid_inst, 0, st, w, K, a1, a2, a3);
-        launch(ld, k_restart<float, 0>, ld.grid_rst, 0, st, w);
+        launch(ld, k_restart<float, 0>, ld.grid_rst, restart_ring(0), st, w);
         launch(ld, k_restart_sigma<true>, ld.grid_inst, 0, st, w);
-        launch(ld, k_restart<float, 1>, ld.grid_rst, 0, st, w);
+        launch(ld, k_restart<float, 1>, ld.grid_rst, restart_ring(1), st, w);
         launch(ld, k_anchor, ld.grid_slab, 0, st, w);
-        launch(ld, k_restart<float, 2>, ld.grid_rst, 0, st, w);
+        launch(ld, k_restart<float, 2>, ld.grid_rst, restart_ring(2), st, w);
     }
     launch(ld, k_block_end, ld.grid_inst, 0, st, w);
 }
