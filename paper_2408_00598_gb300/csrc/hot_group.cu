@@ -1,23 +1,30 @@
-// One check block (K iterations of Algorithm 2, arXiv 2408.00598) of an FP32
-// bulk instance in one kernel: k_group32.
+// Check blocks (K iterations of Algorithm 2, arXiv 2408.00598, and the stopping
+// and restart rules) of small instances in one kernel: k_group32 (FP32 bulk
+// mode), k_group64.
 //
-// The chain k_vec32 -> k_alpha32 -> k_sweep32 costs three launch boundaries
-// per iteration, about 20 us on small grids whose sweep itself takes one or
-// two.  Here a group of CTAs takes an instance through the K iterations of a
-// block with two waits per iteration:
-//   A  slab sums: T and P of each slab (a warp per slab) from the row sums;
-//      wait 1
-//   B  every CTA forms the O(m + n) stage of Prop. 3 for itself (a few
-//      thousand cycles, the same bits in every CTA), then for each of its
-//      tiles the pieces of A^T y-bar (in shared memory), Steps 2-4, and the
-//      tile's row and column sums;
-//      wait 2
-// A CTA owns the same tiles in every iteration, so the flow state needs no
-// exchange: only the row sums (2mn pairs), column partials and slab sums go
-// through L2.  The first pass of the next iteration's state is loaded before
-// the waits.  Every sum that feeds the iterates is formed in the order of the
-// chain of kernels (hot_dev.cuh, k_vec32, k_sweep32), so an instance's iterates
-// do not depend on which of the two ran, nor on the size of its group.
+// The chain k_vec32 -> k_alpha32 -> k_sweep32 costs three launch boundaries per
+// iteration, about 20 us on small grids whose sweep itself takes one or two, and
+// eight more per block.  Here a group of CTAs takes an instance through its
+// blocks with two waits per iteration:
+//   A  slab sums: T and P of each slab (a warp per sum) from the row sums;
+//      wait
+//   B  every CTA forms the O(m + n) stage of Prop. 3 for itself (the same bits
+//      in every CTA), then for each of its tiles the pieces of A^T y-bar (in
+//      shared memory), Steps 2-4, and the tile's row and column sums;
+//      wait
+// and the block end (hot_block.cuh) with waits in place of its launches.  A CTA
+// owns the same tiles throughout, so the flow state needs no exchange: only the
+// row sums (2mn), column partials and slab sums go through L2.  The first
+// tile's state is copied to shared memory while the sums and the second wait
+// run, every further tile's under the sums of the one before.  Every sum that
+// feeds the iterates is formed in the order of the chain (hot_dev.cuh, k_vec32,
+// k_sweep32), so an instance's iterates do not depend on which of the two ran,
+// nor on the size of its group.
+//
+// Bound by latency: an iteration of a 32 x 32 pair takes 19,400 cycles, the two
+// waits 3,000 each with the CTAs' skew, slab sums 1,900, stage 3,000, pieces 2,000,
+// sweep and sums 3,000.  us per iteration of a solve, chain -> group: 32 x 32
+// 24.9 -> 11.3, 64 x 64 25.9 -> 13.2, 128 x 128 34.5 -> 23.1, 192 x 192 64.7 -> 59.8.
 //
 // The groups of one launch are independent.  The grid is launched
 // cooperatively, so that the CTAs of a group are resident together; every

@@ -16,7 +16,8 @@
 // FP64 mode runs the same solve as k_vec, k_marg (instance-wide vectors, one
 // CTA per instance) and k_alpha, in FP64.
 // A block of K iterations ends with the KKT check, the restart rule, and the
-// restart itself (new anchor), see launch_block_end.
+// restart itself (new anchor), see launch_block_end.  Small instances run the
+// same steps inside one kernel (hot_group.cu).
 //
 // FP32 bulk mode stores the anchor u (= v0 - sigma g0) and the delta d in FP32
 // and forms every element from small quantities (see hot_internal.h):
