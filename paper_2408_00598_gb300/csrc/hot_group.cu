@@ -29,6 +29,9 @@
 // The groups of one launch are independent.  The grid is launched
 // cooperatively, so that the CTAs of a group are resident together; every
 // wait is bounded and sets W->err when it runs out.
+
+#include <atomic>
+
 #include "hot_block.cuh"
 
 namespace hot {
@@ -884,11 +887,11 @@ cudaError_t group_init() {
 }
 
 int group_grid(int fp64) {
-    static int cache[2][64];                 // per precision and device ordinal; 0 = not yet queried
+    static std::atomic<int> cache[2][64];    // per precision and device ordinal; 0 = not yet queried
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-    int& c = cache[fp64 ? 1 : 0][dev];
-    if (c == 0) {
+    std::atomic<int>& c = cache[fp64 ? 1 : 0][dev];
+    if (c.load() == 0) {
         int sms = 0, a = 0, b = 0;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (group_init() != cudaSuccess) return 0;
@@ -898,9 +901,9 @@ int group_grid(int fp64) {
         if (e == cudaSuccess && !fp64)
             e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_group32<true>, kThreads, sizeof(GroupSmem));
         if (e != cudaSuccess) return 0;
-        c = sms * (a < b ? a : b);
+        c.store(sms * (a < b ? a : b));
     }
-    return c;
+    return c.load();
 }
 
 void launch_group(const WorkDev* w, int grid, int fp64, int K, int blocks, double a1, double a2, double a3, bool pad,

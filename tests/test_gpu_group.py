@@ -80,3 +80,29 @@ def test_groups_of_a_batch_equal_single_solves(count):
             a = ctx.solve(mu, nu, tol=1e-6, max_iter=300)
             ctx.release(a)
             assert (a["ot_value"], a["dual_value"], a["iters"]) == (b["ot_value"], b["dual_value"], b["iters"])
+
+
+@pytest.mark.parametrize("sizes", [(128, 128), (64, 128, 256, 16)])
+def test_contexts_of_several_threads_share_the_device(sizes):
+    """Each thread's groups fill the device; the launches of the others take turns with them."""
+    import threading
+    from paper_2408_00598_gb300 import hot
+    pairs = [syn.make_pair("white", S, q) for q, S in enumerate(sizes)]
+    out = [[] for _ in sizes]
+
+    def run(q, times):
+        with hot.Context(precision="fp32") as ctx:
+            for _ in range(times):
+                r = ctx.solve(*pairs[q], tol=1e-6, max_iter=200)
+                out[q].append((r["ot_value"], r["iters"], r["rel_kkt"], r["status"]))
+                ctx.release(r)
+
+    for q in range(len(sizes)):
+        run(q, 1)
+    threads = [threading.Thread(target=run, args=(q, 4)) for q in range(len(sizes))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join(120)
+    for got in out:
+        assert len(got) == 5 and all(g == got[0] for g in got)
