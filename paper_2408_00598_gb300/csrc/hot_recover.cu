@@ -28,12 +28,12 @@ constexpr int kRecWarps = 8;
 // 256), which would otherwise start in the same banks.
 __host__ __device__ constexpr int pidx(int i) { return i + (i >> 3); }
 // shared memory of one warp in k_recover_df, in floats: the pairs A (m + 1) and
-// B (n + 1), the entries' indices (16 bits each) and, to fill, the merge steps
-// (m + n), to an even count
-__host__ __device__ constexpr size_t recover_df_words(int m, int n, bool fill) {
-    return (2 * ((size_t)pidx(m) + 1) + 2 * ((size_t)pidx(n) + 1) + (m + 1) / 2 + (n + 1) / 2 + (fill ? m + n : 0) + 1) &
-           ~(size_t)1;
+// B (n + 1) and the entries' indices (16 bits each), to an even count
+__host__ __device__ constexpr size_t recover_df_words(int m, int n) {
+    return (2 * ((size_t)pidx(m) + 1) + 2 * ((size_t)pidx(n) + 1) + (m + 1) / 2 + (n + 1) / 2 + 1) & ~(size_t)1;
 }
+// longest walk (m + n - 1 merge steps) whose directions fit 32 bits per lane
+constexpr int kPathSteps = 32 * 32;
 // the same for k_recover, in doubles
 __host__ __device__ constexpr size_t recover_words(int m, int n) { return 2 * ((size_t)m + n) + 2; }
 
@@ -306,32 +306,65 @@ __device__ __forceinline__ int merge_split(const float2* A, const float2* B, int
     return lo;
 }
 
+// A lane's steps [d0, d1): bit t of the result is set where step d0 + t passes a
+// source's end (steps past the end of a side: 0).  COUNT: the entries are counted
+// into c.
+template <bool COUNT, class BITS>
+__device__ __forceinline__ BITS merge_walk(const float2* A, const float2* B, int ca, int cb, int d0, int d1, int& c) {
+    BITS bits = 0;
+    if (d0 >= d1) return bits;
+    int p = merge_split(A, B, ca, cb, d0), q = d0 - p;
+    if (p >= ca || q >= cb) return bits;
+    DF ae = df_ld(A[pidx(p + 1)]), be = df_ld(B[pidx(q + 1)]);
+    DF prev = COUNT ? df_max(df_ld(A[pidx(p)]), df_ld(B[pidx(q)])) : DF{0.f, 0.f};
+    BITS bit = 1;
+    for (int d = d0; d < d1 && p < ca && q < cb; ++d, bit <<= 1) {
+        const bool sf = !df_lt(be, ae);                  // source p ends first (or both end)
+        if (COUNT) {
+            const DF end = sf ? ae : be;
+            if (df_pos(df_sub(end, prev))) ++c;
+            prev = end;
+        }
+        if (sf) bits |= bit;
+        p += sf;
+        q += !sf;
+        const DF nx = df_ld(sf ? A[pidx(p + 1 < ca ? p + 1 : ca)] : B[pidx(q + 1 < cb ? q + 1 : cb)]);
+        if (sf) ae = nx;
+        else be = nx;
+    }
+    return bits;
+}
+
 // One node (k, j) per warp.  FILL = false: the node's entry count and the
-// plan's marginals.  FILL = true: its entries, 32 merge steps at a time: the
-// walk only notes where each step stands, then consecutive lanes form
-// consecutive steps' overlaps and write the entries next to each other.  (A
-// lane writing its own run put a partial 32-byte sector per entry and array
-// into L2.)  Nothing is written when the plan exceeds cap.
-// Bound: instruction issue (79 % of cycles in both).  256 x 256 after 30
-// iterations: count 0.45 -> 0.26 ms, fill 0.59 -> 0.31 ms; the whole call on a
-// converged pair (11.6 M entries) 1.28 -> 0.46 ms, 512 x 512 (71 M) 10.0 -> 3.3 ms.
-template <bool FILL>
+// plan's marginals.  FILL = true: its entries, 32 merge steps at a time:
+// consecutive lanes form consecutive steps' overlaps and write the entries next
+// to each other.  (A lane writing its own run put a partial 32-byte sector per
+// entry and array into L2.)  Where step d stands follows from the directions of
+// the steps before it: p is the number of sources among them.  PATH: the count
+// leaves them in `path`, 32 bits per lane and node, and the fill reads those
+// 128 bytes; otherwise (walks of more than kPathSteps, or no memory for `path`)
+// the fill walks again.  Nothing is written when the plan exceeds cap.
+// Bound: instruction issue (79 % of cycles).  256 x 256, a converged pair (11.6 M
+// entries): count 172 us, fill 169 us; the whole call 1.32 ms with the walk over
+// all m + n ends, 0.46 ms with both kernels walking and one CTA scanning, 0.41 ms
+// now; 512 x 512 (71 M) 10.0 -> 3.3 -> 2.7 ms.
+template <bool FILL, bool PATH>
 __global__ void __launch_bounds__(kRecWarps * 32) k_recover_df(const float* __restrict__ x, int m, int n,
-                                                               int* __restrict__ counts,
+                                                               int* __restrict__ counts, unsigned* __restrict__ path,
                                                                const long long* __restrict__ offs,
                                                                const unsigned long long* __restrict__ total,
                                                                unsigned long long cap, int32_t* __restrict__ src,
                                                                int32_t* __restrict__ dst, double* __restrict__ mass,
                                                                double* __restrict__ marg1,
                                                                double* __restrict__ marg2) {
+    using Bits = std::conditional_t<PATH, unsigned, unsigned long long>;
     if (FILL && *total > cap) return;
     extern __shared__ float4 shdf[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nw = blockDim.x >> 5;
-    float2* A = reinterpret_cast<float2*>(reinterpret_cast<float*>(shdf) + (size_t)warp * recover_df_words(m, n, FILL));
+    float2* A = reinterpret_cast<float2*>(reinterpret_cast<float*>(shdf) + (size_t)warp * recover_df_words(m, n));
     float2* B = A + pidx(m) + 1;
-    unsigned* e = reinterpret_cast<unsigned*>(B + pidx(n) + 1);
-    unsigned short* ia = reinterpret_cast<unsigned short*>(e + (FILL ? m + n : 0));
+    unsigned short* ia = reinterpret_cast<unsigned short*>(B + pidx(n) + 1);
     unsigned short* ib = ia + ((m + 1) & ~1);
     const int nodes = m * n;
     for (int r = blockIdx.x * nw + warp; r < nodes; r += gridDim.x * nw) {
@@ -340,35 +373,19 @@ __global__ void __launch_bounds__(kRecWarps * 32) k_recover_df(const float* __re
         const int node = k * n + j;
         const float* ra = x + node_row_a(m, k, j);
         const float* rb = x + node_row_b(m, n, k, j);
+        Bits bits = 0;
+        if (FILL && PATH) bits = path[(size_t)node * 32 + lane];
         const int ca = load_side_df(ra, m, ia, A);
         const int cb = load_side_df(rb, n, ib, B);
         const int steps = ca && cb ? ca + cb - 1 : 0;    // every step stands inside both sides until one ends
         const int span = (steps + 31) >> 5;              // merge steps per lane
-        const int d0 = min(steps, lane * span), d1 = min(steps, d0 + span);
-        int p = d0 < d1 ? merge_split(A, B, ca, cb, d0) : ca;
-        int q = d0 - p;
         int c = 0;
-        int d = d0;
-        if (p < ca && q < cb) {
-            DF ae = df_ld(A[pidx(p + 1)]), be = df_ld(B[pidx(q + 1)]);
-            DF prev = FILL ? DF{0.f, 0.f} : df_max(df_ld(A[pidx(p)]), df_ld(B[pidx(q)]));
-            for (; d < d1 && p < ca && q < cb; ++d) {
-                const bool sf = !df_lt(be, ae);          // source p ends first (or both end)
-                if (FILL) {
-                    e[d] = (unsigned)p | (unsigned)q << 16;
-                } else {
-                    const DF end = sf ? ae : be;
-                    if (df_pos(df_sub(end, prev))) ++c;
-                    prev = end;
-                }
-                p += sf;
-                q += !sf;
-                const DF nx = df_ld(sf ? A[pidx(p + 1 < ca ? p + 1 : ca)] : B[pidx(q + 1 < cb ? q + 1 : cb)]);
-                if (sf) ae = nx;
-                else be = nx;
-            }
+        if (!FILL || !PATH) {
+            const int d0 = min(steps, lane * span), d1 = min(steps, d0 + span);
+            bits = merge_walk<!FILL, Bits>(A, B, ca, cb, d0, d1, c);
         }
         if (!FILL) {
+            if (PATH) path[(size_t)node * 32 + lane] = (unsigned)bits;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) c += __shfl_down_sync(0xffffffffu, c, o);
             if (lane == 0) counts[node] = c;
@@ -377,14 +394,23 @@ __global__ void __launch_bounds__(kRecWarps * 32) k_recover_df(const float* __re
             side_marginal(marg1 + (size_t)j * m, ca, ra, ia, A, Bt);
             side_marginal(marg2 + (size_t)k * n, cb, rb, ib, B, At);
         } else {
-            for (; d < d1; ++d) e[d] = 0xffffffffu;      // past the end of a side
-            __syncwarp();
+            const int own = __popcll(bits);              // sources passed before a lane's steps
+            int before = own;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, before, o);
+                if (lane >= o) before += y;
+            }
+            before -= own;
+            const float inv = 1.f / (float)span;
             size_t pos = (size_t)offs[node];
             DF last{0.f, 0.f};                           // the end passed before this round's first step
             for (int base = 0; base < steps; base += 32) {
-                const unsigned w = base + lane < steps ? e[base + lane] : 0xffffffffu;
-                const int pp = (int)(w & 0xffffu), qq = (int)(w >> 16);
-                const bool in = w != 0xffffffffu;
+                const int d = base + lane;
+                const int w = (int)(((float)d + 0.5f) * inv);    // d / span: at least 0.5 / 64 from the next integer
+                const Bits ahead = __shfl_sync(0xffffffffu, bits, w & 31) & (((Bits)1 << ((d - w * span) & 63)) - 1);
+                const int pp = __shfl_sync(0xffffffffu, before, w & 31) + __popcll(ahead), qq = d - pp;
+                const bool in = d < steps && pp < ca && qq < cb;
                 DF end{0.f, 0.f};
                 if (in) end = df_min(df_ld(A[pidx(pp + 1)]), df_ld(B[pidx(qq + 1)]));
                 DF prev = df_shfl_up(end, 1);
@@ -393,8 +419,8 @@ __global__ void __launch_bounds__(kRecWarps * 32) k_recover_df(const float* __re
                 const DF ov = df_sub(end, prev);
                 const bool out = in && df_pos(ov);
                 const unsigned mask = __ballot_sync(0xffffffffu, out);
-                if (out) {
-                    const size_t o = pos + __popc(mask & ((1u << lane) - 1u));
+                const size_t o = pos + __popc(mask & ((1u << lane) - 1u));
+                if (out && o < cap) {
                     src[o] = ia[pp] * n + j;
                     dst[o] = k * n + ib[qq];
                     mass[o] = df_dbl(ov);
@@ -406,53 +432,47 @@ __global__ void __launch_bounds__(kRecWarps * 32) k_recover_df(const float* __re
     }
 }
 
-// Exclusive scan of n counts into offsets, one CTA: a warp per segment sums it,
-// the warps' sums are scanned, then each warp walks its segment again, 128
-// counts per step.  65,536 counts: 131 -> 29 us (a block scan per 1,024 counts
-// paid 20 barriers for each); bound by the latency of one CTA's loads.
+// Exclusive scan of n counts into offsets: each CTA adds up all counts before
+// its segment, then scans the segment, a count per thread and step.  The sums are
+// read from L2 once per CTA, which costs less than a second launch.  65,536
+// counts: 131 -> 12 us (29 on one CTA, whose loads' latency bound it).
+constexpr int kScanCtas = 64;
 __global__ void __launch_bounds__(1024) k_scan(const int* __restrict__ counts, long long* __restrict__ offs, int n,
                                                unsigned long long* __restrict__ total) {
     __shared__ long long s_w[32];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int seg = (((n + 31) / 32) + 127) & ~127;              // per warp, whole steps
-    const int s0 = min(n, warp * seg), s1 = min(n, s0 + seg);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int seg = ((n + kScanCtas - 1) / kScanCtas + 1023) & ~1023;
+    const int s0 = min(n, (int)blockIdx.x * seg), s1 = min(n, s0 + seg);
     long long sum = 0;
 #pragma unroll 8
-    for (int t = s0 + lane; t < s1; t += 32) sum += counts[t];
+    for (int t = tid; t < s0; t += 1024) sum += counts[t];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
     if (lane == 0) s_w[warp] = sum;
     __syncthreads();
     long long carry = 0;
-    for (int w = 0; w < warp; ++w) carry += s_w[w];
-    if (threadIdx.x == 0) {
-        long long all = 0;
-        for (int w = 0; w < 32; ++w) all += s_w[w];
-        *total = (unsigned long long)all;
-    }
-    for (int base = s0; base < s1; base += 128) {
-        int v[4], incl = 0;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int t = base + lane * 4 + u;
-            v[u] = t < s1 ? counts[t] : 0;
-            incl += v[u];
-        }
-        const int own = incl;
+    for (int w = 0; w < 32; ++w) carry += s_w[w];
+    for (int base = s0; base < s1; base += 1024) {
+        const int t = base + tid;
+        const int v = t < s1 ? counts[t] : 0;
+        int incl = v;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int y = __shfl_up_sync(0xffffffffu, incl, o);
             if (lane >= o) incl += y;
         }
-        long long at = carry + incl - own;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int t = base + lane * 4 + u;
-            if (t < s1) offs[t] = at;
-            at += v[u];
+        __syncthreads();                                 // s_w has been read
+        if (lane == 31) s_w[warp] = incl;
+        __syncthreads();
+        long long at = carry + incl - v;
+        for (int w = 0; w < 32; ++w) {
+            const long long x = s_w[w];
+            if (w < warp) at += x;
+            carry += x;
         }
-        carry += __shfl_sync(0xffffffffu, incl, 31);
+        if (t < s1) offs[t] = at;
     }
+    if (blockIdx.x == kScanCtas - 1 && tid == 0) *total = (unsigned long long)carry;
 }
 
 // L1 distances of the plan's marginals to mu1 and mu2 (blockIdx.y: which):
@@ -571,8 +591,17 @@ int recover_plan(Ctx* ctx, Inst* I, int32_t* src, int32_t* dst, double* mass, in
     const size_t o_marg = sizeof(long long) * nodes, o_part = o_marg + sizeof(double) * 2 * nodes,
                  o_tot = o_part + sizeof(double) * 2 * kL1Ctas, o_l1 = o_tot + 8, o_done = o_l1 + 16,
                  o_cnt = o_done + 8, bytes = o_cnt + sizeof(int) * nodes;
+    // and the merge directions that the count leaves for the fill (k_recover_df)
+    const bool want = cap > 0 || src || dst || mass;
+    const size_t o_path = (bytes + 127) & ~(size_t)127;
+    bool keep = want && !I->fp64 && m + n - 1 <= kPathSteps;
     char* scr = nullptr;
-    HOT_CK(cudaMallocAsync((void**)&scr, bytes, st));
+    if (keep && cudaMallocAsync((void**)&scr, o_path + sizeof(unsigned) * 32 * nodes, st) != cudaSuccess) {
+        cudaGetLastError();
+        keep = false;
+    }
+    if (!keep) HOT_CK(cudaMallocAsync((void**)&scr, bytes, st));
+    unsigned* path = keep ? (unsigned*)(scr + o_path) : nullptr;
     long long* offs = (long long*)scr;
     double* marg = (double*)(scr + o_marg);
     unsigned long long* dtot = (unsigned long long*)(scr + o_tot);
@@ -610,13 +639,13 @@ int recover_plan(Ctx* ctx, Inst* I, int32_t* src, int32_t* dst, double* mass, in
         }
         return best;
     };
-    const size_t per_fill = I->fp64 ? recover_words(m, n) * sizeof(double) : recover_df_words(m, n, true) * sizeof(float);
-    const size_t per_count = I->fp64 ? per_fill : recover_df_words(m, n, false) * sizeof(float);
-    const int nw = warps_for(per_fill), nwc = warps_for(per_count);
-    const size_t shm = (size_t)nw * per_fill, shm_count = (size_t)nwc * per_count;
-    cudaError_t e = cudaFuncSetAttribute(k_recover_df<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_recover_df<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    const size_t per = I->fp64 ? recover_words(m, n) * sizeof(double) : recover_df_words(m, n) * sizeof(float);
+    const int nw = warps_for(per);
+    const size_t shm = (size_t)nw * per;
+    const auto count_df = keep ? k_recover_df<false, true> : k_recover_df<false, false>;
+    const auto fill_df = keep ? k_recover_df<true, true> : k_recover_df<true, false>;
+    cudaError_t e = cudaFuncSetAttribute(count_df, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fill_df, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_recover<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     int sms = 0;
@@ -624,14 +653,13 @@ int recover_plan(Ctx* ctx, Inst* I, int32_t* src, int32_t* dst, double* mass, in
     if (e == cudaSuccess) e = cudaMemsetAsync(marg, 0, o_cnt - o_marg, st);
     if (failed(e, "plan recovery")) return finish(HOT_ECUDA);
     const int grid = std::max(1, std::min((nodes + nw - 1) / nw, sms * (64 / nw)));
-    const int gridc = std::max(1, std::min((nodes + nwc - 1) / nwc, sms * (64 / nwc)));
     if (I->fp64)
         k_recover<double><<<grid, nw * 32, shm, st>>>((const double*)I->desc.xr, m, n, 1, counts, nullptr,
                                                               nullptr, nullptr, nullptr, marg, marg + nodes);
     else
-        k_recover_df<false><<<gridc, nwc * 32, shm_count, st>>>((const float*)I->desc.xr, m, n, counts, nullptr, nullptr, 0,
-                                                        nullptr, nullptr, nullptr, marg, marg + nodes);
-    k_scan<<<1, 1024, 0, st>>>(counts, offs, nodes, dtot);
+        count_df<<<grid, nw * 32, shm, st>>>((const float*)I->desc.xr, m, n, counts, path, nullptr, nullptr, 0, nullptr,
+                                             nullptr, nullptr, marg, marg + nodes);
+    k_scan<<<kScanCtas, 1024, 0, st>>>(counts, offs, nodes, dtot);
     if (marg_l1)
         // marginals against mu1 (row-major (i, j)) and mu2 (row-major (k, l))
         k_marg_l1<<<dim3(kL1Ctas, 2), 256, 0, st>>>(marg, I->desc.mu1, I->desc.mu2, m, n, I->fp64 ? 0 : 1,
@@ -641,10 +669,9 @@ int recover_plan(Ctx* ctx, Inst* I, int32_t* src, int32_t* dst, double* mass, in
             k_recover<double><<<grid, nw * 32, shm, st>>>((const double*)I->desc.xr, m, n, 0, counts, offs, ds, dd, dm,
                                                           nullptr, nullptr);
         else
-            k_recover_df<true><<<grid, nw * 32, shm, st>>>((const float*)I->desc.xr, m, n, counts, offs, dtot, room,
-                                                           ds, dd, dm, nullptr, nullptr);
+            fill_df<<<grid, nw * 32, shm, st>>>((const float*)I->desc.xr, m, n, counts, path, offs, dtot, room, ds, dd, dm,
+                                                nullptr, nullptr);
     };
-    const bool want = cap > 0 || src || dst || mass;
     // device outputs of an FP32 solution: the fill runs behind the count without
     // a look at the total (it writes nothing when the plan does not fit)
     const bool ahead = want && !I->fp64 && space == HOT_SPACE_DEVICE && cap > 0;

@@ -13,7 +13,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("m,n,kind", [(2, 2, "white"), (31, 3, "white"), (32, 33, "shapes"), (33, 9, "white"),
-                                      (5, 129, "white"), (130, 7, "gauss"), (24, 24, "shapes")])
+                                      (5, 129, "white"), (130, 7, "gauss"), (24, 24, "shapes"),
+                                      (1023, 2, "white"), (1023, 3, "white")])      # walks of 1,024 and 1,025 steps
 def test_recovery_equals_algorithm1_on_the_flows(m, n, kind):
     import torch
     from paper_2408_00598_gb300 import hot
@@ -45,6 +46,27 @@ def test_recovery_equals_algorithm1_on_the_flows(m, n, kind):
     assert np.abs(P - Q).max() <= 1e-13
     assert abs(np.abs(Q.sum(1) - mu.ravel()).sum() - l1[0]) <= 1e-12
     assert abs(np.abs(Q.sum(0) - nu.ravel()).sum() - l1[1]) <= 1e-12
+
+
+def test_offsets_of_many_nodes():
+    """98,304 nodes, two steps of the scan per CTA: entries in node order without gaps."""
+    import torch
+    from paper_2408_00598_gb300 import hot
+    m, n = 512, 192
+    mu, nu = syn.make_pair("white", m, 5, n)
+    with hot.Context(precision="fp32") as ctx:
+        r = ctx.solve(mu, nu, tol=0.0, max_iter=30)
+        nnz, l1 = ctx.recover_plan(r, ())
+        o = (torch.full((nnz,), -1, dtype=torch.int32, device="cuda"), torch.full((nnz,), -1, dtype=torch.int32, device="cuda"),
+             torch.full((nnz,), -1.0, dtype=torch.float64, device="cuda"))
+        assert ctx.recover_plan(r, o)[0] == nnz
+        ctx.release(r)
+    src, dst, mass = o
+    node = torch.div(dst, n, rounding_mode="floor") * n + src % n
+    assert (mass > 0).all() and (src >= 0).all() and (node.diff() >= 0).all()
+    for idx, hist, want in ((src, mu, l1[0]), (dst, nu, l1[1])):
+        got = torch.bincount(idx, weights=mass, minlength=m * n).cpu().numpy()
+        assert abs(np.abs(got - hist.ravel()).sum() - want) <= 1e-12
 
 
 @pytest.mark.parametrize("nnz,D", [(1, 1), (7, 4), (255, 5), (257, 7), (2049, 8), (5000, 3)])
