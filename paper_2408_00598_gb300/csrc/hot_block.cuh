@@ -17,7 +17,7 @@ struct Sweep64Smem {
     double col[kThreads * 2];
     double xcol[kThreads * 2];
     double red[kNK * 32];
-    double3 a[kMaxTR64];                   // per row: h x^2 - alpha, -2 h x, dalpha
+    double3 a[kMaxTR64];                   // per row: alpha, scaled x, dalpha
 };
 
 // a > b for doubles, on the integer pipe (FP64 comparisons run at a 64th of the
@@ -36,13 +36,12 @@ __device__ __forceinline__ double neg64(double a) {
 
 // Steps 2-4 of Algorithm 2 on one tile (TR rows of a slab) in FP64, and the
 // tile's row and column sums.  ab, dab: the slab's pieces, rows then columns.
-// Bound: the FP64 pipe (2 lanes per clock and SM).  An element takes 8.5 FP64
-// instructions (about 13 before): the cost is separable, h (x_r - x_c)^2 - alpha -
-// beta = (h x_r^2 - alpha) + (h x_c^2 - beta) - 2 h x_r x_c with the first term per
-// row and the second per column (x taken from the middle bin, so that the
-// squares stay below the largest cost), and comparisons run on integers.
-// FP64 pipe 81 % busy.  One sweep: 128 x 128 125 -> 92 us, 256 x 256 947 -> 651 us;
-// on check iterations 224 -> 193 and 1,748 -> 1,424 us.
+// Bound: the FP64 pipe (2 lanes per clock and SM).  An element takes 9.5 FP64
+// instructions (about 13 before): the cost h (x_r - x_c)^2 enters the reduced
+// cost by one fma of the difference t, with x times 2^floor(e / 2), h = 2^e, and
+// for odd e one factor doubled in its exponent; comparisons run on integers.
+// (The separable form h x_r^2 - alpha + h x_c^2 - beta - 2 h x_r x_c takes 8.5, but its
+// error is relative to the largest cost instead of the element's.)
 template <bool CHECK>
 __device__ __forceinline__ void sweep64_tile(const HotInst& I, int slab, int band, const double* __restrict__ din_,
                                              double* __restrict__ dout_, const P64& p, const double* __restrict__ ab,
@@ -61,19 +60,18 @@ __device__ __forceinline__ void sweep64_tile(const HotInst& I, int slab, int ban
     const double* __restrict__ din = din_ + off;
     double* __restrict__ dout = dout_ + off;
     const double* __restrict__ X = I.X64 + g_xbase(I, slab);               // bin coordinates of this half
-    const double mid = X[S / 2], h = p.h;
-    if (tid < nr) {
-        const double x = X[r0 + tid] - mid;
-        s.a[tid] = make_double3(fma(h * x, x, -ab[r0 + tid]), -2.0 * h * x, dab[r0 + tid]);
-    }
+    const int he = (__double2hiint(p.h) >> 20) - 1023;                     // h = 2^he
+    const int odd = (he & 1) << 20;
+    const double sc = __hiloint2double(((he >> 1) + 1023) << 20, 0);       // h = sc^2, or 2 sc^2 for odd he
+    if (tid < nr) s.a[tid] = make_double3(ab[r0 + tid], X[r0 + tid] * sc, dab[r0 + tid]);
     const int c0 = cg * NV;
     const int nval = S - c0;                                               // columns inside the slab (pad after)
     double B[NV], db[NV], xc[NV], cacc[NV], xacc[NV];
 #pragma unroll
     for (int e = 0; e < NV; ++e) {
         const bool v = active && e < nval;
-        xc[e] = v ? X[c0 + e] - mid : 0.0;
-        B[e] = v ? fma(h * xc[e], xc[e], -ab[S + c0 + e]) : 0.0;
+        xc[e] = v ? X[c0 + e] * sc : 0.0;
+        B[e] = v ? ab[S + c0 + e] : 0.0;
         db[e] = v ? dab[S + c0 + e] : 0.0;
         cacc[e] = xacc[e] = 0.0;
     }
@@ -96,7 +94,9 @@ __device__ __forceinline__ void sweep64_tile(const HotInst& I, int slab, int ban
             double out[NV], xo[NV];
 #pragma unroll
             for (int e = 0; e < NV; ++e) {
-                const double g = fma(a.y, xc[e], a.x + B[e]);              // c - A^T y-bar
+                const double t = a.y - xc[e];
+                const double t2 = __hiloint2double(__double2hiint(t) + odd, __double2loint(t));
+                const double g = fma(t2, t, -a.x) - B[e];                  // c - A^T y-bar
                 const double D = a.z + db[e];                              // A^T (y-bar - y0)
                 const double sv = uu[e] + dd[e];
                 const double w = fma(nis, sv, -D);                         // g - v / sigma
