@@ -56,15 +56,13 @@ __device__ __forceinline__ DF df_mul(DF a, float b) {
     const float h = __fadd_rn(p, e);
     return DF{h, __fsub_rn(e, __fsub_rn(h, p))};
 }
-// a + x y with the product's rounding error kept: the compensated dot product
-// of Ogita, Rump and Oishi (2005), half the operations of adding the product as
-// a pair.  lo collects the errors and is renormalised by the next df_add.
+// a + x y, the product as an exact pair and the sum renormalised.  (The
+// compensated dot product of Ogita, Rump and Oishi (2005), which collects the
+// errors in lo unnormalised, takes half the operations, but its error over 64
+// squares is 2.5 times this one's on average.)
 __device__ __forceinline__ DF df_dot(DF a, float x, float y) {
-    const float p = __fmul_rn(x, y), pe = fmaf(x, y, -p);
-    const float s = __fadd_rn(a.hi, p);
-    const float bb = __fsub_rn(s, a.hi);
-    const float e = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, bb)), __fsub_rn(p, bb));
-    return DF{s, __fadd_rn(a.lo, __fadd_rn(e, pe))};
+    const float p = __fmul_rn(x, y);
+    return df_add(a, DF{p, fmaf(x, y, -p)});
 }
 __device__ __forceinline__ DF df_shfl_down(DF a, int o) {
     return DF{__shfl_down_sync(0xffffffffu, a.hi, o), __shfl_down_sync(0xffffffffu, a.lo, o)};

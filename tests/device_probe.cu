@@ -11,6 +11,16 @@ __global__ void __launch_bounds__(kThreads) k_sweep(HotInst I, P64 p, const doub
     sweep64_tile<false>(I, 0, 0, (const double*)I.d0, out, p, ab, dab, rs, cs, sm);
 }
 
+// one sum of products per thread
+__global__ void k_dot(const float* x, const float* y, int terms, int sums, float* hi, float* lo) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= sums) return;
+    DF a{0.f, 0.f};
+    for (int q = 0; q < terms; ++q) a = df_dot(a, x[t * terms + q], y[t * terms + q]);
+    hi[t] = a.hi;
+    lo[t] = a.lo;
+}
+
 }  // namespace
 
 // The reduced costs g = h (X_r - X_c)^2 - alpha_r - beta_c of one S x S tile as the FP64 sweep forms them:
@@ -41,6 +51,22 @@ extern "C" int probe_sweep64(int S, double h, const double* X, const double* ab,
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e == cudaSuccess) e = cudaMemcpy2D(out, S * 8, o, Sp * 8, S * 8, S, cudaMemcpyDeviceToHost);
+    cudaFree(d);
+    return (int)e;
+}
+
+// sums[t] = sum over q of x[t][q] y[t][q], as a pair
+extern "C" int probe_dot(const float* x, const float* y, int terms, int sums, float* hi, float* lo) {
+    const size_t N = (size_t)terms * sums;
+    float* d = nullptr;
+    if (cudaMalloc(&d, (2 * N + 2 * sums) * 4) != cudaSuccess) return 1;
+    float *dx = d, *dy = d + N, *dh = dy + N, *dl = dh + sums;
+    cudaMemcpy(dx, x, N * 4, cudaMemcpyHostToDevice);
+    cudaMemcpy(dy, y, N * 4, cudaMemcpyHostToDevice);
+    k_dot<<<(sums + 127) / 128, 128>>>(dx, dy, terms, sums, dh, dl);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpy(hi, dh, sums * 4, cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess) e = cudaMemcpy(lo, dl, sums * 4, cudaMemcpyDeviceToHost);
     cudaFree(d);
     return (int)e;
 }

@@ -51,3 +51,38 @@ def test_fp64_reduced_cost_error_is_relative_to_the_element(probe, S, span, size
             bound = u * (2 * cost + abs(cost - Fraction(ab[r])) + abs(g)) * (1 + 8 * u)
             assert abs(Fraction(out[r, c]) + g) <= bound, (r, c)
     assert seen >= S
+
+
+def _two_sum(a, b):
+    s = a + b
+    bb = s - a
+    return s, (a - (s - bb)) + (b - bb)
+
+
+def _pair_add(ah, al, b):
+    s, e = _two_sum(ah, b)
+    e = e + al
+    h = s + e
+    return h, e - (h - s)
+
+
+@pytest.mark.parametrize("terms", [1, 5, 64])
+@pytest.mark.parametrize("square", [True, False])
+def test_sums_of_products_are_sums_of_renormalised_pairs(probe, terms, square):
+    """df_dot against the pair sum restated in numpy FP32 (each exact product added as a pair), bit for bit."""
+    f4 = np.float32
+    rng = np.random.default_rng(terms)
+    sums = 4000
+    x = (rng.standard_normal((sums, terms)) * 10.0 ** rng.uniform(-3, 3, (sums, terms))).astype(f4)
+    y = x if square else rng.standard_normal((sums, terms)).astype(f4)
+    hi, lo = np.zeros(sums, f4), np.zeros(sums, f4)
+    assert probe.probe_dot(_ptr(x), _ptr(np.ascontiguousarray(y)), terms, sums, _ptr(hi), _ptr(lo)) == 0
+    h = np.zeros(sums, f4)
+    l = np.zeros(sums, f4)
+    for q in range(terms):
+        exact = x[:, q].astype(np.float64) * y[:, q]              # exact: 24 + 24 bits
+        p = exact.astype(f4)
+        pe = (exact - p).astype(f4)
+        h, l = _pair_add(*_pair_add(h, l, p), pe)
+    np.testing.assert_array_equal(hi, h)
+    np.testing.assert_array_equal(lo, l)
