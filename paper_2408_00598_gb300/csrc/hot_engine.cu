@@ -173,9 +173,10 @@ GroupPlan plan_groups(const std::vector<int>& inst, const std::vector<int>& tile
     double tau = wait + 1.0;
     while (!build(tau, false)) tau *= 1.08;
     build(tau, true);
-    P.start.assign(grid + 1, 0);
-    for (int c = 0; c < grid; ++c) {
-        if (c < (int)cta.size()) P.entries.insert(P.entries.end(), cta[c].begin(), cta[c].end());
+    P.used = (int)cta.size();
+    P.start.assign(P.used + 1, 0);
+    for (int c = 0; c < P.used; ++c) {
+        P.entries.insert(P.entries.end(), cta[c].begin(), cta[c].end());
         P.start[c + 1] = (int)P.entries.size();
     }
     return P;
@@ -601,7 +602,7 @@ int Batch::set_instances(const std::vector<Inst*>& v, cudaStream_t st, bool grou
     pt[0] = ps[0] = pv[0] = pk[0] = pa[0] = 0;
     int running = 0;
     size_t swept = 0;                 // bytes one sweep of the chain streams: u, d read, d written
-    n_group = n_chain = 0;
+    n_group = n_chain = gused = 0;
     pad = gpad = 0;
     // many tiles per CTA hide the chain's launches, and its sweep has more
     // CTAs per SM: beyond a few tiles per CTA the chain is the faster one
@@ -637,8 +638,8 @@ int Batch::set_instances(const std::vector<Inst*>& v, cudaStream_t st, bool grou
         pa[i + 1] = pa[i] + (g ? 0 : v[i]->desc.n_achunk);
         if (v[i]->ctl_host.status == ST_RUNNING) ++running;
     }
-    // the kernels of a block, and their variants, depend on the mix: a change needs new graphs
-    if (captured >= 0 && captured != shape()) drop_graphs();
+    // the chain's kernels, and their variants, depend on its instances: a change needs new graphs
+    if (n_chain > 0 && captured >= 0 && captured != shape()) drop_graphs();
     // a state larger than L2: alternate the sweep's tile order, so that each
     // sweep starts on the tiles the previous one touched last (still in L2);
     // a state that fits gains nothing from it
@@ -672,6 +673,7 @@ int Batch::set_instances(const std::vector<Inst*>& v, cudaStream_t st, bool grou
     h_running[1] = 0;
     if (n_group > 0) {
         const GroupPlan gp = plan_groups(gi, gt, ge, ggrid, fp64);
+        gused = gp.used;
         std::copy(gp.start.begin(), gp.start.end(), h_gstart);
         std::copy(gp.entries.begin(), gp.entries.end(), h_gent);
         HOT_CK(cudaMemcpyAsync(d_gstart, h_gstart, sizeof(int) * gp.start.size(), cudaMemcpyHostToDevice, st));
@@ -692,30 +694,21 @@ int Batch::set_instances(const std::vector<Inst*>& v, cudaStream_t st, bool grou
 }
 
 int Batch::launches() const {
-    return (n_group > 0 ? 1 : 0) + (n_chain > 0 ? launches_per_block(fp64, K, n_chain == 1) + kLaunchesBlockEnd : 0);
+    return (gused > 0 ? 1 : 0) + (n_chain > 0 ? launches_per_block(fp64, K, n_chain == 1) + kLaunchesBlockEnd : 0);
 }
 
-// The K iterations of a block: k_group32 for the grouped instances, the chain
-// of kernels for the others; with ev, an event pair around the sweep of
-// iteration timed_iter().
-void Batch::launch_iterations(cudaStream_t st, cudaEvent_t* ev) const {
-    if (n_group > 0) launch_group(d_work, ggrid, fp64, K, group_blocks(), a1, a2, a3, gpad != 0, st);
-    if (n_chain == 0) return;
-    for (int j = 0; j < K; ++j) {
-        launch_solve_kernels(d_work, ld, fp64, j, j == K - 1, n_chain == 1, st);
-        const bool t = ev && j == timed_iter() && j < K - 1;
-        if (t) cudaEventRecordWithFlags(ev[0], st, cudaEventRecordExternal);
-        launch_sweep(d_work, ld, fp64, j, j == K - 1, pad != 0, st);
-        if (t) cudaEventRecordWithFlags(ev[1], st, cudaEventRecordExternal);
-    }
-}
-
-// One check block (K iterations plus the block end) captured into *out; with
-// ev, an event pair recorded around the sweep of iteration timed_iter().
+// One check block of the chain (K iterations plus the block end) captured into
+// *out; with ev, an event pair recorded around the sweep of iteration timed_iter().
 int Batch::capture(cudaGraphExec_t* out, cudaEvent_t* ev) {
     HOT_CK(cudaStreamBeginCapture(cap_stream, cudaStreamCaptureModeThreadLocal));
-    launch_iterations(cap_stream, ev);
-    if (n_chain > 0) launch_block_end(d_work, ld, fp64, K, a1, a2, a3, cap_stream);
+    for (int j = 0; j < K; ++j) {
+        launch_solve_kernels(d_work, ld, fp64, j, j == K - 1, n_chain == 1, cap_stream);
+        const bool t = ev && j == timed_iter() && j < K - 1;
+        if (t) cudaEventRecordWithFlags(ev[0], cap_stream, cudaEventRecordExternal);
+        launch_sweep(d_work, ld, fp64, j, j == K - 1, pad != 0, cap_stream);
+        if (t) cudaEventRecordWithFlags(ev[1], cap_stream, cudaEventRecordExternal);
+    }
+    launch_block_end(d_work, ld, fp64, K, a1, a2, a3, cap_stream);
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamEndCapture(cap_stream, &g);
     if (e != cudaSuccess) {
@@ -734,6 +727,7 @@ int Batch::capture(cudaGraphExec_t* out, cudaEvent_t* ev) {
 
 int Batch::ensure_graph(int want_timing) {
     timing = want_timing && K >= 2 ? 1 : 0;
+    if (n_chain == 0) return HOT_OK;                 // the group kernels are launched as they are
     if (timing ? (tgraph[0] && tgraph[1]) : graph != nullptr) return HOT_OK;
     if (!cap_stream) HOT_CK(cudaStreamCreateWithFlags(&cap_stream, cudaStreamNonBlocking));
     ld = make_launch_dims(device, fp64);
@@ -751,7 +745,8 @@ int Batch::ensure_graph(int want_timing) {
 }
 
 int Batch::launch_block(cudaStream_t st, long long block) const {
-    HOT_CK(cudaGraphLaunch(timing ? tgraph[block & 1] : graph, st));
+    if (gused > 0) HOT_CK(launch_group(d_work, gused, fp64, K, group_blocks(), a1, a2, a3, gpad != 0, st));
+    if (n_chain > 0) HOT_CK(cudaGraphLaunch(timing ? tgraph[block & 1] : graph, st));
     return HOT_OK;
 }
 

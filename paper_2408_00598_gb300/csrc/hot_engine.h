@@ -70,13 +70,14 @@ int inst_create(const PairHost& p, int fp64, const hot_config& cfg, double tol, 
                 cudaStream_t st, Inst** out);
 void inst_destroy(Inst* I, cudaStream_t st);
 
-// Device work tables plus the instantiated block graph that reads them.
+// Device work tables plus the instantiated block graph of the chain that reads them.
 // Prefix tables (cap + 1 ints each): tiles, slabs, k_vec items, k_kkt1 chunks, k_alpha32 chunks.
 constexpr int kPreTables = 5;
 // CTAs of k_group32 for the grouped instances of a batch, by a cost model of
 // one iteration: entries (instance, rank, group size) per CTA.
 struct GroupPlan {
-    std::vector<int> start;      // [grid + 1]
+    int used = 0;                // CTAs with entries: the grid of the launch
+    std::vector<int> start;      // [used + 1]
     std::vector<int4> entries;
 };
 GroupPlan plan_groups(const std::vector<int>& inst, const std::vector<int>& tiles, const std::vector<int>& elems, int grid,
@@ -97,7 +98,8 @@ struct Batch {
     int4* d_gent = nullptr;         // [ggrid + cap]
     int* h_gstart = nullptr;        // pinned
     int4* h_gent = nullptr;         // pinned
-    int ggrid = 0;                  // grid of k_group32 on this device
+    int ggrid = 0;                  // CTAs of k_group32 resident at once on this device
+    int gused = 0;                  // grid of its launch (0: nothing to launch)
     // k_group32 takes part while the instances it may run have at most this many
     // tiles: a batch of 20 with sides 32 to 128 (4,500 tiles) took 0.91 of the chain's speed with it
     long long group_tiles() const { return 4LL * ggrid; }
@@ -126,9 +128,7 @@ struct Batch {
     int max_group_blocks = 4;       // check blocks per launch of k_group32 when it runs alone (the host looks in between)
     int group_blocks() const { return n_chain > 0 ? 1 : max_group_blocks; }
     int pad = 0, gpad = 0;
-    int shape() const {             // what a captured graph depends on
-        return (n_group > 0) | (n_chain > 0) << 1 | (n_chain == 1) << 2 | (pad != 0) << 3 | (gpad != 0) << 4;
-    }
+    int shape() const { return (n_chain == 1) | (pad != 0) << 1; }   // what a captured graph depends on
     int captured = -1;              // shape() of the captured graphs (-1: none)
     int launches() const;           // kernels of one block
     const int* running(long long block) const { return h_running + 2 + 2 * (block & 1); }
@@ -137,7 +137,6 @@ struct Batch {
     int reserve(int n);
     // async H2D; group: k_group32 takes the instances it may take
     int set_instances(const std::vector<Inst*>& v, cudaStream_t st, bool group = true);
-    void launch_iterations(cudaStream_t st, cudaEvent_t* ev) const;
     int ensure_graph(int timing = 0);
     int launch_block(cudaStream_t st, long long block = 0) const;
     int timed_iter() const { return (K - 1) / 2; }   // a non-check iteration when K >= 2

@@ -27,8 +27,10 @@
 // 24.9 -> 11.3, 64 x 64 25.9 -> 13.2, 128 x 128 34.5 -> 23.1, 192 x 192 64.7 -> 59.8.
 //
 // The groups of one launch are independent.  The grid is launched
-// cooperatively, so that the CTAs of a group are resident together; every
-// wait is bounded and sets W->err when it runs out.
+// cooperatively, so that the CTAs of a group are resident together; it has the
+// CTAs that plan_groups gave work, so that a small instance leaves the rest of
+// the device to other contexts and to the caller's kernels.  Every wait is
+// bounded and sets W->err when it runs out.
 
 #include <atomic>
 
@@ -906,8 +908,8 @@ int group_grid(int fp64) {
     return c.load();
 }
 
-void launch_group(const WorkDev* w, int grid, int fp64, int K, int blocks, double a1, double a2, double a3, bool pad,
-                  cudaStream_t st) {
+cudaError_t launch_group(const WorkDev* w, int grid, int fp64, int K, int blocks, double a1, double a2, double a3, bool pad,
+                         cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(kThreads);
@@ -919,7 +921,7 @@ void launch_group(const WorkDev* w, int grid, int fp64, int K, int blocks, doubl
     cfg.attrs = at;
     cfg.numAttrs = 1;
     const BlockRule rule{K, a1, a2, a3};
-    cudaLaunchKernelEx(&cfg, fp64 ? k_group64 : pad ? k_group32<true> : k_group32<false>, w, blocks, rule);
+    return cudaLaunchKernelEx(&cfg, fp64 ? k_group64 : pad ? k_group32<true> : k_group32<false>, w, blocks, rule);
 }
 
 }  // namespace hot

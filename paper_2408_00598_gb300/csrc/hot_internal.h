@@ -310,8 +310,8 @@ void launch_sweep(const WorkDev* w, const LaunchDims& ld, int fp64, int j, bool 
 void launch_block_end(const WorkDev* w, const LaunchDims& ld, int fp64, int K, double a1, double a2, double a3,
                       cudaStream_t st);
 // k_group32, k_group64 (hot_group.cu): up to `blocks` check blocks of every grouped instance in one cooperative launch
-void launch_group(const WorkDev* w, int grid, int fp64, int K, int blocks, double a1, double a2, double a3, bool pad,
-                  cudaStream_t st);
+cudaError_t launch_group(const WorkDev* w, int grid, int fp64, int K, int blocks, double a1, double a2, double a3, bool pad,
+                         cudaStream_t st);
 int group_grid(int fp64);                  // CTAs resident at once on the current device (0: not available)
 cudaError_t group_init();
 LaunchDims make_launch_dims(int device, int fp64);

@@ -106,3 +106,27 @@ def test_contexts_of_several_threads_share_the_device(sizes):
         t.join(120)
     for got in out:
         assert len(got) == 5 and all(g == got[0] for g in got)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_a_small_solve_runs_beside_a_kernel_of_the_caller(precision):
+    """A kernel of one thread on another stream (about a second) takes one SM's place for a CTA; a small pair's
+    group kernels need some of the others and do not wait for it."""
+    import torch
+    from paper_2408_00598_gb300 import hot
+    mu, nu = syn.make_pair("white", 16, 1)
+    with hot.Context(precision=precision) as ctx:
+        ctx.release(ctx.solve(mu, nu, tol=0.0, max_iter=40))         # tables, pools, modules
+        side, ended = torch.cuda.Stream(), torch.cuda.Event()
+        with torch.cuda.stream(side):
+            torch.cuda._sleep(1)
+        torch.cuda.synchronize()
+        with torch.cuda.stream(side):
+            torch.cuda._sleep(2 * 10 ** 9)
+            ended.record()
+        r = ctx.solve(mu, nu, tol=0.0, max_iter=40)
+        beside = not ended.query()
+        ctx.release(r)
+        torch.cuda.synchronize()
+    assert r["iters"] == 40
+    assert beside
