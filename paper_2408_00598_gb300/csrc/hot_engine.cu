@@ -504,6 +504,15 @@ void inst_destroy(Inst* I, cudaStream_t st) {
 
 // ------------------------------------------------------------------- batch --
 
+static std::atomic<int> g_at_work[64];               // per device ordinal
+AtWork::AtWork(int device) : n(device >= 0 && device < 64 ? &g_at_work[device] : nullptr) {
+    if (n) n->fetch_add(1);
+}
+AtWork::~AtWork() {
+    if (n) n->fetch_sub(1);
+}
+int AtWork::count(int device) { return device >= 0 && device < 64 ? std::max(1, g_at_work[device].load()) : 1; }
+
 Batch::~Batch() {
     if (graph) cudaGraphExecDestroy(graph);
     for (int p = 0; p < 2; ++p) {
@@ -609,11 +618,12 @@ int Batch::set_instances(const std::vector<Inst*>& v, cudaStream_t st, bool grou
     long long gtiles = 0;
     for (const Inst* I : v)
         if (I->group_ok && I->ctl_host.status == ST_RUNNING) gtiles += (long long)I->n * I->nb1 + (long long)I->m * I->nb2;
-    if (gtiles > group_tiles()) group = false;
+    const Room have = room();         // one look: others come and go
+    if (gtiles > have.tiles) group = false;
     std::vector<int> gi, gt, ge;      // grouped instances: index, tiles, elements of a tile
     for (int i = 0; i < n; ++i) {
         h_inst[i] = v[i]->desc;
-        const int g = group && ggrid > 0 && v[i]->group_ok ? 1 : 0;
+        const int g = group && have.ctas > 0 && v[i]->group_ok ? 1 : 0;
         h_inst[i].grp = g;
         const int m = v[i]->m, nn = v[i]->n;
         const int tiles = nn * v[i]->nb1 + m * v[i]->nb2;
@@ -672,7 +682,7 @@ int Batch::set_instances(const std::vector<Inst*>& v, cudaStream_t st, bool grou
     h_running[0] = running;
     h_running[1] = 0;
     if (n_group > 0) {
-        const GroupPlan gp = plan_groups(gi, gt, ge, ggrid, fp64);
+        const GroupPlan gp = plan_groups(gi, gt, ge, have.ctas, fp64);
         gused = gp.used;
         std::copy(gp.start.begin(), gp.start.end(), h_gstart);
         std::copy(gp.entries.begin(), gp.entries.end(), h_gent);
@@ -783,6 +793,7 @@ void fill_result(const Inst* I, hot_result* r) {
 
 int run_solve(Ctx* ctx, const std::vector<PairHost>& pairs, double tol, long long max_iter, bool keep,
               hot_result* out, hot_kernel_times* kt) {
+    const AtWork at_work(ctx->device);
     cudaStream_t st = ctx->stream;
     const int fp64 = ctx->cfg.precision == HOT_FP64 ? 1 : 0;
     if (!ctx->batch || ctx->batch->fp64 != fp64) {
@@ -892,7 +903,7 @@ int run_solve(Ctx* ctx, const std::vector<PairHost>& pairs, double tol, long lon
                         any = true;
                         tiles += (long long)I->n * I->nb1 + (long long)I->m * I->nb2;
                     }
-                    rebuild = any && tiles <= B.group_tiles();
+                    rebuild = any && tiles <= B.room().tiles;
                 }
                 if (rebuild) {
                     cudaEventSynchronize(ev[nb & 1]);            // block nb and its status copy

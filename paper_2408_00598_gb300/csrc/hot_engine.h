@@ -70,6 +70,21 @@ int inst_create(const PairHost& p, int fp64, const hot_config& cfg, double tol, 
                 cudaStream_t st, Inst** out);
 void inst_destroy(Inst* I, cudaStream_t st);
 
+// A solve, or a serve loop with requests, at work on a device.  The group kernels
+// of one hold their CTAs' places from launch to end, so two that want the whole
+// device take turns; each new set of work tables therefore plans its groups for
+// an equal share of the device (Batch::room).  Results do not depend on it.
+// 128 x 128 FP32 solves in 1 / 2 / 4 / 8 contexts: 110 / 112 / 113 / 113 -> 110 / 141 / 159 / 170 a second.
+struct AtWork {
+    explicit AtWork(int device);
+    ~AtWork();
+    AtWork(const AtWork&) = delete;
+    AtWork& operator=(const AtWork&) = delete;
+    static int count(int device);          // at least 1
+private:
+    std::atomic<int>* n;
+};
+
 // Device work tables plus the instantiated block graph of the chain that reads them.
 // Prefix tables (cap + 1 ints each): tiles, slabs, k_vec items, k_kkt1 chunks, k_alpha32 chunks.
 constexpr int kPreTables = 5;
@@ -102,7 +117,16 @@ struct Batch {
     int gused = 0;                  // grid of its launch (0: nothing to launch)
     // k_group32 takes part while the instances it may run have at most this many
     // tiles: a batch of 20 with sides 32 to 128 (4,500 tiles) took 0.91 of the chain's speed with it
-    long long group_tiles() const { return 4LL * ggrid; }
+    // (beside other solves FP64 ones, whose pipe their CTAs share, gain only with a CTA per tile:
+    // 64 x 64 in four contexts 105 solves/s with more, 129 with the chain)
+    struct Room {
+        int ctas;
+        long long tiles;
+    };
+    Room room() const {
+        const int at_work = AtWork::count(device), ctas = ggrid / at_work;
+        return Room{ctas, (fp64 && at_work > 1 ? 1LL : 4LL) * ctas};
+    }
     int* d_st = nullptr;            // [cap] per-instance status after each check
     int* h_st = nullptr;            // pinned mirror
     int* h_stb = nullptr;           // pinned, [2][cap]: statuses after the last two blocks (finish times)

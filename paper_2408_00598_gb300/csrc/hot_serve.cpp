@@ -105,6 +105,7 @@ static void serve_loop(Ctx* ctx) {
     const int fp64 = ctx->cfg.precision == HOT_FP64 ? 1 : 0;
     const int max_batch = ctx->cfg.max_batch > 0 ? ctx->cfg.max_batch : 1024;
     bool changed = false;
+    std::unique_ptr<AtWork> at_work;                 // while requests run
     for (;;) {
         std::vector<Req*> admit;
         {
@@ -136,11 +137,13 @@ static void serve_loop(Ctx* ctx) {
                 admit.push_back(r);
             }
             if (admit.empty() && s->active.empty()) {
+                at_work.reset();
                 s->cv_done.notify_all();
                 s->cv_work.wait_for(lk, std::chrono::milliseconds(20));
                 continue;
             }
         }
+        if (!at_work) at_work.reset(new AtWork(ctx->device));
         for (Req* r : admit) {
             Inst* I = nullptr;
             r->t_admit = Clock::now();

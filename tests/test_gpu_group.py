@@ -130,3 +130,33 @@ def test_a_small_solve_runs_beside_a_kernel_of_the_caller(precision):
         torch.cuda.synchronize()
     assert r["iters"] == 40
     assert beside
+
+
+@pytest.mark.parametrize("precision,S", [("fp32", 128), ("fp64", 64)])
+def test_solves_of_two_contexts_overlap(precision, S):
+    """Two threads with a context each against one thread with the same number of solves: the groups of each plan
+    for a share of the device, so the two run side by side (taking turns, the times are equal)."""
+    import threading
+    import time
+    from paper_2408_00598_gb300 import hot
+    mu, nu = syn.make_pair("white", S, 1)
+
+    def run(ctx, times):
+        for _ in range(times):
+            ctx.release(ctx.solve(mu, nu, tol=0.0, max_iter=400))
+
+    with hot.Context(precision=precision) as a, hot.Context(precision=precision) as b:
+        run(a, 1)
+        run(b, 1)
+        best = [1e9, 1e9]
+        for _ in range(3):
+            t0 = time.perf_counter()
+            run(a, 12)
+            t1 = time.perf_counter()
+            threads = [threading.Thread(target=run, args=(ctx, 6)) for ctx in (a, b)]
+            for t in threads:
+                t.start()
+            for t in threads:
+                t.join()
+            best = [min(best[0], t1 - t0), min(best[1], time.perf_counter() - t1)]
+    assert best[1] < 0.9 * best[0], best
