@@ -236,6 +236,14 @@ HOT_API int hot_solve_profiled(hot_ctx *ctx, const double *mu, const double *nu,
  * hot_solve_profiled are never timed this way. */
 HOT_API int hot_sweep_timing(hot_ctx *ctx, int enable, double *total_ms, long long *launches, double *bytes);
 
+/* Diagnostics: the bound of the device-side waits (small instances run whole
+ * check blocks in one kernel whose thread blocks wait for one another), in
+ * polls of about a microsecond each; 0: the default, a few seconds.  It takes
+ * effect with the next call, in the serve loop with the next admission.  A
+ * wait that runs out ends the call (serve loop: the requests running) with
+ * HOT_ECUDA; the context and the device stay usable.  No CUDA error is raised. */
+HOT_API int hot_wait_limit(hot_ctx *ctx, int polls);
+
 /* Algorithm 1 without any device allocation (the paper has no counterpart;
  * this exists for callers that cannot let a library allocate device memory at
  * call time: code with a fixed, pre-accounted device-memory footprint, or a

@@ -250,6 +250,17 @@ int hot_sweep_timing(hot_ctx* ctx, int enable, double* total_ms, long long* laun
     HOT_GUARD_END
 }
 
+int hot_wait_limit(hot_ctx* ctx, int polls) {
+    HOT_GUARD_BEGIN
+    if (!ctx || polls < 0) {
+        set_error(ctx ? "polls must be >= 0" : "ctx is NULL");
+        return HOT_EINVAL;
+    }
+    ctx->impl.polls = polls;
+    return HOT_OK;
+    HOT_GUARD_END
+}
+
 int hot_solve_batch(hot_ctx* ctx, int count, const double* const* mus, const double* const* nus, const int* ms,
                     const int* ns, int space, double tol, long long max_iter, hot_result* out) {
     HOT_GUARD_BEGIN

@@ -677,6 +677,7 @@ int Batch::set_instances(const std::vector<Inst*>& v, cudaStream_t st, bool grou
     h_work->gent = d_gent;
     h_work->n_running = d_running;
     h_work->err = d_running + 1;
+    h_work->polls = polls > 0 ? polls : kPollLimit;
     h_work->st_out = d_st;
     for (int i = 0; i < n; ++i) h_st[i] = v[i]->ctl_host.status;
     h_running[0] = running;
@@ -807,6 +808,7 @@ int run_solve(Ctx* ctx, const std::vector<PairHost>& pairs, double tol, long lon
         b.a3 = ctx->cfg.restart_long;
     }
     Batch& B = *ctx->batch;
+    B.polls = ctx->polls;
     std::vector<Inst*> insts;
     insts.reserve(pairs.size());
     auto cleanup = [&]() {
@@ -841,6 +843,7 @@ int run_solve(Ctx* ctx, const std::vector<PairHost>& pairs, double tol, long lon
     const long long max_blocks = (max_iter + K - 1) / K + 2;
     long long nb = 0;
     int err = HOT_OK;
+    const char* why = nullptr;
     // profiled mode: direct launches with an event pair around each kernel family
     std::vector<cudaEvent_t> pev;
     if (kt) {
@@ -888,6 +891,7 @@ int run_solve(Ctx* ctx, const std::vector<PairHost>& pairs, double tol, long lon
                 const int run_prev = B.running(nb - 1)[0];
                 if (B.running(nb - 1)[1]) {                      // a bounded wait ran out on the device
                     err = HOT_ECUDA;
+                    why = "a wait between the CTAs of a group ran out";
                     ++nb;
                     break;
                 }
@@ -1006,7 +1010,8 @@ int run_solve(Ctx* ctx, const std::vector<PairHost>& pairs, double tol, long lon
         kt->sweep_bytes = vb;
     }
     if (e != cudaSuccess || err != HOT_OK) {
-        set_error(std::string("solve failed on the device: ") + cudaGetErrorString(e != cudaSuccess ? e : cudaGetLastError()));
+        set_error(std::string("solve failed on the device: ") +
+                  (e == cudaSuccess && why ? why : cudaGetErrorString(e != cudaSuccess ? e : cudaGetLastError())));
         cleanup();
         return HOT_ECUDA;
     }

@@ -149,6 +149,7 @@ struct Batch {
     // some instance of that kind needs the general sweep: a side that is not
     // a multiple of 4, or (FP32) real-valued bin coordinates
     int n_group = 0, n_chain = 0;
+    int polls = 0;                  // of a wait in the group kernels (0: kPollLimit)
     int max_group_blocks = 4;       // check blocks per launch of k_group32 when it runs alone (the host looks in between)
     int group_blocks() const { return n_chain > 0 ? 1 : max_group_blocks; }
     int pad = 0, gpad = 0;
@@ -183,6 +184,7 @@ struct Ctx {
     std::map<unsigned long long, Solution> solutions;
     std::atomic<unsigned long long> next_id{1};
     std::unique_ptr<ServeState> serve;
+    std::atomic<int> polls{0};             // hot_wait_limit
     int tile_override = 0;                 // force TR (0 = tuned or default); the autotuner sets it
     std::mutex tune_mu;                    // guards tuned (the serve thread reads it)
     std::map<int, std::pair<int, double>> tuned[2];   // [fp64][S] -> (TR, us per iteration)

@@ -44,7 +44,6 @@ constexpr int kW = kThreads / 32;
 constexpr int kRowN = kRowSmemBytes / sizeof(float) + 256;
 constexpr int kTileTable = 32;            // tiles of a CTA whose geometry is kept
 constexpr int kRing = 4;                  // passes of state in flight (one float4 of u and of d per thread each)
-constexpr int kPollLimit = 1 << 22;       // polls of a wait before it gives up (a few seconds)
 
 // Geometry of a tile; offsets fit 32 bits (sides up to kMaxGroupSide).
 struct GTile {
@@ -86,7 +85,8 @@ struct GroupSmem {
     DF F[2];                              // half totals
     DF sm1, sm2;                          // the marginals' sums
     P32 p[64];                            // of every iteration of the block (check_every <= 64)
-    int dead;
+    int dead;                             // a wait of this CTA ran out
+    int polls;                            // polls of a wait before it gives up (WorkDev::polls)
     // buffers of the block end
     __device__ double* rows() { return reinterpret_cast<double*>(row); }      // row and xrow
     __device__ double* cols() { return reinterpret_cast<double*>(col); }      // col and xcol
@@ -111,7 +111,7 @@ __device__ __forceinline__ bool group_wait(S& s, int G, unsigned epoch, int* err
         unsigned* count = s.I.gcount;
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;\n" ::"l"(count) : "memory");
         unsigned v;
-        int left = kPollLimit;
+        int left = s.polls;
         do {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(v) : "l"(count) : "memory");
         } while (v < epoch * (unsigned)G && --left > 0);
@@ -729,11 +729,15 @@ template <typename S, typename F>
 __device__ __forceinline__ void group_entries(S& s, const WorkDev* __restrict__ W, F run) {
     const int tid = threadIdx.x;
     const int e0 = W->gstart[blockIdx.x], e1 = W->gstart[blockIdx.x + 1];
-    if (tid == 0) s.dead = 0;
+    if (tid == 0) {
+        s.dead = __ldcg(W->err);                       // set in an earlier launch: nothing more is done
+        s.polls = W->polls;
+    }
 #pragma unroll 1
     for (int e = e0; e < e1; ++e) {
         const int4 ge = W->gent[e];                    // instance, rank, group size
         __syncthreads();
+        if (s.dead) return;                            // its state is lost; no later entry would be waited for
         const HotInst* src = W->inst + ge.x;
 #pragma unroll 1
         for (int q = tid; q < (int)(sizeof(HotInst) / 8); q += kThreads)
@@ -777,7 +781,7 @@ struct Group64Smem {
     HotInst I;
     Recip64 R;
     P64 p[64];
-    int dead;
+    int dead, polls;
     __device__ double* rows() { return sw.row; }             // row and xrow
     __device__ double* cols() { return sw.col; }             // col and xcol
     __device__ double* reds() { return red; }

@@ -43,6 +43,7 @@ constexpr int kMaxTileElems = 16384;   // FP32 tiles: TR * (longer row pitch) <=
 constexpr int kMaxGroupSide = 256;     // k_group32: longest side (one column per thread)
 constexpr int kMaxGroupSide64 = 128;   // k_group64: longest side
 constexpr int kMaxGroup = 512;         // k_group32: most CTAs of one instance
+constexpr int kPollLimit = 1 << 22;    // polls of a wait between CTAs before it gives up (a few seconds)
 
 enum : int {
     ST_RUNNING = 0,
@@ -265,6 +266,7 @@ struct WorkDev {
     int4* gent;            // instance, rank in its group, group size
     int* n_running;        // instances still running
     int* err;              // set when a bounded wait ran out
+    int polls;             // polls of such a wait before it gives up
     int* st_out;           // [ninst] status of each instance after its last check
 };
 

@@ -174,6 +174,7 @@ static void serve_loop(Ctx* ctx) {
                 }
         }
         if (changed) {
+            s->batch->polls = ctx->polls;
             if (s->batch->set_instances(insts, s->st) != HOT_OK || s->batch->ensure_graph() != HOT_OK) {
                 std::lock_guard<std::mutex> g(s->mu);
                 for (Req* r : s->active) finish_req(ctx, s, r, HOT_ECUDA);

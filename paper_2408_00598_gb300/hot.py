@@ -136,6 +136,7 @@ def load_library(path=None):
         "hot_solve_coords": (i, [vp, vp, vp, i, i, i, vp, vp, d, ll, P(hot_result)]),
         "hot_solve_profiled": (i, [vp, vp, vp, i, i, i, d, ll, P(hot_result), P(hot_kernel_times)]),
         "hot_sweep_timing": (i, [vp, i, P(d), P(ll), P(d)]),
+        "hot_wait_limit": (i, [vp, i]),
         "hot_get_flows": (i, [vp, ull, vp, i]),
         "hot_recover_plan": (i, [vp, ull, vp, vp, vp, i, sz, P(sz), P(d)]),
         "hot_release": (i, [vp, ull]),
@@ -305,6 +306,14 @@ def hot_sweep_timing(ctx, enable):
     if rc != HOT_OK:
         raise _err(lib, ctx, rc)
     return {"ms": ms.value, "launches": n.value, "bytes": b.value}
+
+
+def hot_wait_limit(ctx, polls):
+    """Bound of the device-side waits, in polls (0: the default of a few seconds)."""
+    lib = load_library()
+    rc = lib.hot_wait_limit(ctx, int(polls))
+    if rc != HOT_OK:
+        raise _err(lib, ctx, rc)
 
 
 def hot_solve_batch(ctx, mus, nus, tol=1e-6, max_iter=100000):
@@ -509,6 +518,9 @@ class Context:
 
     def sweep_timing(self, enable=-1):
         return hot_sweep_timing(self.ctx, enable)
+
+    def wait_limit(self, polls=0):
+        hot_wait_limit(self.ctx, polls)
 
     def flows(self, res, out=None):
         return hot_get_flows(self.ctx, res["solution_id"], res["m"], res["n"], out)

@@ -160,3 +160,32 @@ def test_solves_of_two_contexts_overlap(precision, S):
                 t.join()
             best = [min(best[0], t1 - t0), min(best[1], time.perf_counter() - t1)]
     assert best[1] < 0.9 * best[0], best
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_a_wait_that_runs_out_ends_the_call_with_an_error(precision):
+    """With one poll per wait, the CTAs that arrive before the last one of their group give up at the first wait.
+    The call says so, nothing is left behind, and the context solves again; so does the serve loop."""
+    from paper_2408_00598_gb300 import hot
+    mu, nu = syn.make_pair("white", 32, 1)
+    with hot.Context(precision=precision) as ctx:
+        a = ctx.solve(mu, nu, tol=1e-6, max_iter=200)
+        ctx.release(a)
+        ctx.wait_limit(1)
+        for _ in range(2):
+            with pytest.raises(hot.HotError, match="a wait between the CTAs of a group ran out") as e:
+                ctx.solve(mu, nu, tol=1e-6, max_iter=200)
+            assert e.value.status == hot.HOT_ECUDA
+        with pytest.raises(hot.HotError, match="ran out"):
+            ctx.solve_batch([mu] * 3, [nu] * 3, tol=1e-6, max_iter=200)
+        t = ctx.submit(mu, nu, tol=1e-6, max_iter=200)
+        assert ctx.wait(t)[0] == hot.HOT_ECUDA
+        ctx.wait_limit(0)
+        b = ctx.solve(mu, nu, tol=1e-6, max_iter=200)
+        ctx.release(b)
+        t = ctx.submit(mu, nu, tol=1e-6, max_iter=200)
+        status, c = ctx.wait(t)
+        ctx.forget(t)
+    for r in (b, c):
+        assert (r["ot_value"], r["iters"], r["status"]) == (a["ot_value"], a["iters"], a["status"])
+    assert status == a["status"]
