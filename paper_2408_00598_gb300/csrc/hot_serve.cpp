@@ -185,13 +185,14 @@ static void serve_loop(Ctx* ctx) {
             changed = false;
         }
         // two blocks back to back, then look at the statuses
-        s->batch->launch_block(s->st);
-        s->batch->launch_block(s->st);
+        bool launched = true;
+        for (int b = 0; b < 2; ++b) launched = s->batch->launch_block(s->st) == HOT_OK && launched;
         const int n = (int)insts.size();
         cudaMemcpyAsync(s->batch->h_st, s->batch->d_st, sizeof(int) * n, cudaMemcpyDeviceToHost, s->st);
         cudaMemcpyAsync((void*)s->batch->running(0), s->batch->d_running, 2 * sizeof(int), cudaMemcpyDeviceToHost, s->st);
         cudaError_t e = cudaStreamSynchronize(s->st);
-        if (e == cudaSuccess && s->batch->running(0)[1]) e = cudaErrorUnknown;   // a bounded wait ran out on the device
+        // a launch that failed would leave its requests running for good; a bounded wait ran out on the device
+        if (e == cudaSuccess && (!launched || s->batch->running(0)[1])) e = cudaErrorUnknown;
         std::lock_guard<std::mutex> g(s->mu);
         s->blocks += 2;
         std::vector<Req*> still;
