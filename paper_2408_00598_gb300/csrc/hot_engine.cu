@@ -859,7 +859,8 @@ int run_solve(Ctx* ctx, const std::vector<PairHost>& pairs, double tol, long lon
     // finished pairs from the tables as they go, see below)
     std::vector<int> live(insts.size());
     for (size_t q = 0; q < insts.size(); ++q) live[q] = (int)q;
-    long long launches = 0, blocks = 0;
+    long long launches = 0;
+    int ahead = 0;                 // the last launch was one too many: every instance had ended before it
     const auto th0 = std::chrono::steady_clock::now();
     auto note_finished = [&](const int* sts) {
         const double now = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - th0).count();
@@ -874,7 +875,6 @@ int run_solve(Ctx* ctx, const std::vector<PairHost>& pairs, double tol, long lon
                 break;
             }
             launches += B.launches();
-            blocks += B.group_blocks();
             cudaMemcpyAsync((void*)B.running(nb), B.d_running, 2 * sizeof(int), cudaMemcpyDeviceToHost, st);
             if (track)
                 cudaMemcpyAsync(B.h_stb + (size_t)(nb & 1) * B.cap, B.d_st, sizeof(int) * live.size(),
@@ -950,6 +950,7 @@ int run_solve(Ctx* ctx, const std::vector<PairHost>& pairs, double tol, long lon
                     }
                 }
                 if (run_prev <= 0) {
+                    ahead = 1;
                     ++nb;
                     break;
                 }
@@ -1015,13 +1016,16 @@ int run_solve(Ctx* ctx, const std::vector<PairHost>& pairs, double tol, long lon
         cleanup();
         return HOT_ECUDA;
     }
-    if (kt) {
-        launches = nb * B.launches();
-        blocks = nb;
+    if (kt) launches = nb * B.launches();
+    // a launch of the group kernels runs several blocks, or fewer when its
+    // instances end: the blocks are counted by the iterations
+    long long blocks = 0;
+    for (Inst* I : insts) {
+        cudaMemcpy(&I->ctl_host, I->desc.ctl, sizeof(HotCtl), cudaMemcpyDeviceToHost);
+        blocks = std::max(blocks, I->ctl_host.total / K + ahead);
     }
     for (size_t q = 0; q < insts.size(); ++q) {
         Inst* I = insts[q];
-        cudaMemcpy(&I->ctl_host, I->desc.ctl, sizeof(HotCtl), cudaMemcpyDeviceToHost);
         fill_result(I, &out[q]);
         // a batch reports each instance's own completion (host-observed, from
         // the start of the batch); a single solve the device time of the solve

@@ -189,3 +189,19 @@ def test_a_wait_that_runs_out_ends_the_call_with_an_error(precision):
     for r in (b, c):
         assert (r["ot_value"], r["iters"], r["status"]) == (a["ot_value"], a["iters"], a["status"])
     assert status == a["status"]
+
+
+@pytest.mark.parametrize("S,max_iter", [(16, 10), (16, 50), (64, 3000)])
+def test_blocks_of_a_solve_do_not_depend_on_the_form(S, max_iter):
+    """hot_result.blocks: the check blocks that ran and the one launched ahead, though a group launch runs several."""
+    from paper_2408_00598_gb300 import hot
+    mu, nu = syn.make_pair("shapes", S, 1)
+    with hot.Context(precision="fp32") as ctx:
+        got = []
+        for chain in (0, 1):
+            ctx.sweep_timing(chain)
+            r = ctx.solve(mu, nu, tol=1e-6, max_iter=max_iter)
+            ctx.release(r)
+            got.append(r["blocks"])
+        ctx.sweep_timing(0)
+    assert got == [r["iters"] // 10 + 1] * 2
