@@ -758,6 +758,7 @@ __device__ __forceinline__ void check_instance(const HotInst& I, const WorkDev* 
             else C->k = C->k + K;
         }
         if (fin) {
+            C->t_end = clock_ns();
             C->just_finished = 1;
             atomicSub(W->n_running, 1);
         }

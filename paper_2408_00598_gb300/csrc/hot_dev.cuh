@@ -15,6 +15,13 @@ namespace hot {
 
 // ---------------------------------------------------------------- helpers --
 
+// the device's clock in nanoseconds
+__device__ __forceinline__ unsigned long long clock_ns() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %globaltimer;\n" : "=l"(t));
+    return t;
+}
+
 __device__ __forceinline__ int find_inst(const int* __restrict__ pre, int n, int t) {
     int lo = 0, hi = n - 1;
     while (lo < hi) {

@@ -851,8 +851,9 @@ int run_solve(Ctx* ctx, const std::vector<PairHost>& pairs, double tol, long lon
         pev.resize(3 * K + 2);
         for (auto& e : pev) cudaEventCreate(&e);
     }
-    // batches: the host time at which the block holding each instance's last
-    // check was seen complete (its status copied back after every block)
+    // batches: the host time at which the launch holding each instance's last
+    // check was seen complete (its status copied back after every launch); the
+    // group kernels, which run several blocks per launch, leave device times
     const bool track = insts.size() > 1 && !kt;
     std::vector<double> fin_ms(insts.size(), -1.0);
     // live[q]: the pair at position q of the work tables (batches drop their
@@ -1020,16 +1021,21 @@ int run_solve(Ctx* ctx, const std::vector<PairHost>& pairs, double tol, long lon
     // a launch of the group kernels runs several blocks, or fewer when its
     // instances end: the blocks are counted by the iterations
     long long blocks = 0;
+    unsigned long long start = 0;              // of the first group launch, if the batch began with one
     for (Inst* I : insts) {
         cudaMemcpy(&I->ctl_host, I->desc.ctl, sizeof(HotCtl), cudaMemcpyDeviceToHost);
         blocks = std::max(blocks, I->ctl_host.total / K + ahead);
+        const unsigned long long t = I->ctl_host.t_start;
+        if (t && (!start || t < start)) start = t;
     }
     for (size_t q = 0; q < insts.size(); ++q) {
         Inst* I = insts[q];
         fill_result(I, &out[q]);
-        // a batch reports each instance's own completion (host-observed, from
-        // the start of the batch); a single solve the device time of the solve
-        out[q].solve_ms = track ? (fin_ms[q] >= 0.0 ? fin_ms[q] : (double)ms) : ms;
+        // a batch reports each instance's own completion from the start of the
+        // batch; a single solve the device time of the solve
+        out[q].solve_ms = ms;
+        if (track && start && I->ctl_host.t_end > start) out[q].solve_ms = 1e-6 * (double)(I->ctl_host.t_end - start);
+        else if (track && fin_ms[q] >= 0.0) out[q].solve_ms = fin_ms[q];
         out[q].kernel_launches = launches;
         out[q].blocks = blocks;
         if (keep) {

@@ -744,6 +744,7 @@ __device__ __forceinline__ void group_entries(S& s, const WorkDev* __restrict__ 
             reinterpret_cast<double*>(&s.I)[q] = reinterpret_cast<const double*>(src)[q];
         __syncthreads();
         if (s.I.ctl->status != ST_RUNNING) continue;   // the same for the whole group
+        if (ge.y == 0 && tid == 0 && s.I.ctl->total == 0) s.I.ctl->t_start = clock_ns();
         run(ge);
         asm volatile("cp.async.wait_group 0;\n" ::: "memory");
         if (ge.z > 1 && tid == 0 && s.dead == 0) {

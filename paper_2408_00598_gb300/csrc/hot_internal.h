@@ -65,6 +65,7 @@ struct HotCtl {
     double dx2, dz2;       // ||x-bar - x_r||^2, ||z-bar - z_r||^2 at the last restart
     double sigma_old;      // sigma of the check iteration that triggered the last restart
     double res_norm;       // ||w - w-bar||_M at the last check
+    unsigned long long t_start, t_end;   // device clock (ns): the group kernel's first block of the instance, its last check; 0: not yet
     long long total;       // iterations completed before the current block
     long long max_iter;
     int k;                 // Halpern counter at the start of the block

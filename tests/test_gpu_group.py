@@ -205,3 +205,21 @@ def test_blocks_of_a_solve_do_not_depend_on_the_form(S, max_iter):
             got.append(r["blocks"])
         ctx.sweep_timing(0)
     assert got == [r["iters"] // 10 + 1] * 2
+
+
+def test_pairs_of_a_batch_report_their_own_completion():
+    """25 pairs of one size and several classes, some of which end in different blocks of the same launch of the group
+    kernel (four blocks): another number of iterations is another solve_ms, and 20 more of them a larger one."""
+    from paper_2408_00598_gb300 import hot
+    kinds = ("white", "gauss", "cauchy", "shapes", "translate")
+    pairs = [syn.make_pair(kinds[q % 5], 16, q) for q in range(25)]
+    with hot.Context(precision="fp32") as ctx:
+        for _ in range(2):
+            out = ctx.solve_batch([p[0] for p in pairs], [p[1] for p in pairs], tol=4e-3, max_iter=3000)
+    got = [(r["iters"], r["solve_ms"]) for r in out]
+    assert len({i for i, _ in got}) >= 3, got
+    for ia, ta in got:
+        assert ta > 0.0
+        for ib, tb in got:
+            assert ia == ib or ta != tb, got
+            assert ib < ia + 20 or ta < tb, got
