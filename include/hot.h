@@ -223,7 +223,10 @@ HOT_API int hot_solve_profiled(hot_ctx *ctx, const double *mu, const double *nu,
 
 /* Live timing of the dominant kernel, the fused Steps 2-4 sweep of a
  * non-check iteration (the paper has no counterpart; it measures the kernel
- * inside the production path, not in a separate profiled run).  enable = 1:
+ * inside the block graphs that solves run, not in a separate profiled run).
+ * While it is on, pairs of every size run the chain of kernels: small pairs,
+ * which otherwise run whole blocks in one kernel without a sweep launch, take
+ * up to twice as long (the results are the same).  enable = 1:
  * later single-instance hot_solve calls on this context launch block graphs
  * that carry a CUDA event pair around one non-check sweep per block of
  * check_every iterations (check_every >= 2), and add each measured duration

@@ -29,3 +29,18 @@ def test_recorded_traffic_only_for_the_source_it_was_taken_on(monkeypatch):
     assert bench.recorded_traffic(256, "fp64") is None
     monkeypatch.setattr(bench, "kernels_sha", lambda: "0" * 64)     # the kernels changed since
     assert bench.recorded_traffic(256, "fp32") is None
+
+
+def test_sweep_timing_inside_the_timed_region_only_where_it_keeps_the_kernels():
+    class Ctx:
+        def __init__(self, group):
+            self.group, self.on = group, 0
+
+        def sweep_timing(self, enable):
+            self.on = enable
+
+    for group in (False, True):
+        ctx = Ctx(group)
+        solve = lambda: {"kernel_launches": 26 if ctx.group and not ctx.on else 798}
+        assert bench.timing_keeps_the_path(ctx, solve) is (not group)
+        assert ctx.on == 0
