@@ -258,7 +258,7 @@ def oracle_baseline(mu1, mu2, kind, seed, tol, gpu_iters, n_iter=50, stop="relat
 
 # ------------------------------------------------------------------ modes --
 
-RECOVERY_KERNELS = 5    # of one plan recovery: count, scan, 2 x L1, write
+RECOVERY_KERNELS = 4    # of one plan recovery: count, scan, L1, fill
 
 
 def timing_keeps_the_path(ctx, solve):
