@@ -129,59 +129,6 @@ static int group_rule(const Inst& I) {
     return std::max(I.m, I.n) <= kMaxGroupSide && I.big_bytes / 5 * 2 <= kGroupStateBytes ? 1 : 0;
 }
 
-// Groups of CTAs for one launch of k_group32.  An iteration of an instance
-// costs its CTAs two waits plus their tiles one after the other; the plan
-// takes the smallest time in which every instance fits into the grid: large
-// ones get as many CTAs as they need, small ones share a CTA (group size 1).
-GroupPlan plan_groups(const std::vector<int>& inst, const std::vector<int>& tiles, const std::vector<int>& elems,
-                      int grid, int fp64) {
-    GroupPlan P;
-    const int n = (int)inst.size();
-    const double wait = 4.0, self = 1.5;                      // microseconds: two waits and the stage; the stage alone
-    auto tile_us = [&](int q) { return 0.9 + elems[q] * (fp64 ? 0.003 : 0.00015); };
-    std::vector<int> order(n);
-    for (int q = 0; q < n; ++q) order[q] = q;
-    std::stable_sort(order.begin(), order.end(),
-                     [&](int a, int b) { return tiles[a] * tile_us(a) > tiles[b] * tile_us(b); });
-    std::vector<std::vector<int4>> cta;
-    auto build = [&](double tau, bool write) {
-        int used = 0;
-        double room = -1.0;                                   // of the shared CTA being filled
-        for (int q : order) {
-            const double alone = self + tiles[q] * tile_us(q);
-            if (alone > tau) {
-                const int per = std::max(1, (int)((tau - wait) / tile_us(q)));
-                int G = (tiles[q] + per - 1) / per;
-                G = std::min(G, std::min(kMaxGroup, grid));
-                if (write)
-                    for (int r = 0; r < G; ++r) cta.push_back({make_int4(inst[q], r, G, 0)});
-                used += G;
-            } else {
-                if (room < alone) {
-                    ++used;
-                    room = tau;
-                    if (write) cta.emplace_back();
-                }
-                room -= alone;
-                if (write) cta.back().push_back(make_int4(inst[q], 0, 1, 0));
-            }
-            if (used > grid) return false;
-        }
-        return true;
-    };
-    // shared CTAs come after the large ones in `order`, so the last one is open
-    double tau = wait + 1.0;
-    while (!build(tau, false)) tau *= 1.08;
-    build(tau, true);
-    P.used = (int)cta.size();
-    P.start.assign(P.used + 1, 0);
-    for (int c = 0; c < P.used; ++c) {
-        P.entries.insert(P.entries.end(), cta[c].begin(), cta[c].end());
-        P.start[c + 1] = (int)P.entries.size();
-    }
-    return P;
-}
-
 // --------------------------------------------------------------- instances --
 
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -620,10 +567,22 @@ int Batch::set_instances(const std::vector<Inst*>& v, cudaStream_t st, bool grou
         if (I->group_ok && I->ctl_host.status == ST_RUNNING) gtiles += (long long)I->n * I->nb1 + (long long)I->m * I->nb2;
     const Room have = room();         // one look: others come and go
     if (gtiles > have.tiles) group = false;
-    std::vector<int> gi, gt, ge;      // grouped instances: index, tiles, elements of a tile
+    if (have.ctas < 1) group = false;
+    GroupPlan gp;
+    if (group) {
+        std::vector<int> gi, gt, ge;  // grouped instances: index, tiles, elements of a tile
+        for (int i = 0; i < n; ++i) {
+            if (!v[i]->group_ok || v[i]->ctl_host.status != ST_RUNNING) continue;
+            gi.push_back(i);
+            gt.push_back(v[i]->n * v[i]->nb1 + v[i]->m * v[i]->nb2);
+            ge.push_back((int)(v[i]->big_bytes / (fp64 ? 40 : 20) / gt.back()));
+        }
+        gp = plan_groups(gi, gt, ge, have.ctas, fp64);
+        if (!fp64 && gp.most > kTileTable) group = false;      // k_group32 keeps the geometry of that many
+    }
     for (int i = 0; i < n; ++i) {
         h_inst[i] = v[i]->desc;
-        const int g = group && have.ctas > 0 && v[i]->group_ok ? 1 : 0;
+        const int g = group && v[i]->group_ok ? 1 : 0;
         h_inst[i].grp = g;
         const int m = v[i]->m, nn = v[i]->n;
         const int tiles = nn * v[i]->nb1 + m * v[i]->nb2;
@@ -631,11 +590,6 @@ int Batch::set_instances(const std::vector<Inst*>& v, cudaStream_t st, bool grou
         if (g) {
             ++n_group;
             gpad |= odd;
-            if (v[i]->ctl_host.status == ST_RUNNING) {
-                gi.push_back(i);
-                gt.push_back(tiles);
-                ge.push_back((int)(v[i]->big_bytes / (fp64 ? 40 : 20) / tiles));
-            }
         } else {
             ++n_chain;
             pad |= odd;
@@ -683,9 +637,9 @@ int Batch::set_instances(const std::vector<Inst*>& v, cudaStream_t st, bool grou
     h_running[0] = running;
     h_running[1] = 0;
     if (n_group > 0) {
-        const GroupPlan gp = plan_groups(gi, gt, ge, have.ctas, fp64);
         gused = gp.used;
         std::copy(gp.start.begin(), gp.start.end(), h_gstart);
+        static_assert(sizeof(GroupEntry) == sizeof(int4), "the device reads the entries as int4");
         std::copy(gp.entries.begin(), gp.entries.end(), h_gent);
         HOT_CK(cudaMemcpyAsync(d_gstart, h_gstart, sizeof(int) * gp.start.size(), cudaMemcpyHostToDevice, st));
         if (!gp.entries.empty())

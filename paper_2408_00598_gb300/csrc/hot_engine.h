@@ -88,15 +88,6 @@ private:
 // Device work tables plus the instantiated block graph of the chain that reads them.
 // Prefix tables (cap + 1 ints each): tiles, slabs, k_vec items, k_kkt1 chunks, k_alpha32 chunks.
 constexpr int kPreTables = 5;
-// CTAs of k_group32 for the grouped instances of a batch, by a cost model of
-// one iteration: entries (instance, rank, group size) per CTA.
-struct GroupPlan {
-    int used = 0;                // CTAs with entries: the grid of the launch
-    std::vector<int> start;      // [used + 1]
-    std::vector<int4> entries;
-};
-GroupPlan plan_groups(const std::vector<int>& inst, const std::vector<int>& tiles, const std::vector<int>& elems, int grid,
-                      int fp64);
 struct Batch {
     int device = 0;
     int cap = 0;
@@ -112,7 +103,7 @@ struct Batch {
     int* d_gstart = nullptr;        // [ggrid + 1]
     int4* d_gent = nullptr;         // [ggrid + cap]
     int* h_gstart = nullptr;        // pinned
-    int4* h_gent = nullptr;         // pinned
+    GroupEntry* h_gent = nullptr;   // pinned
     int ggrid = 0;                  // CTAs of k_group32 resident at once on this device
     int gused = 0;                  // grid of its launch (0: nothing to launch)
     // k_group32 takes part while the instances it may run have at most this many

@@ -42,7 +42,6 @@ namespace {
 
 constexpr int kW = kThreads / 32;
 constexpr int kRowN = kRowSmemBytes / sizeof(float) + 256;
-constexpr int kTileTable = 32;            // tiles of a CTA whose geometry is kept
 constexpr int kRing = 4;                  // passes of state in flight (one float4 of u and of d per thread each)
 
 // Geometry of a tile; offsets fit 32 bits (sides up to kMaxGroupSide).
@@ -617,7 +616,7 @@ __device__ __forceinline__ void group_instance(GroupSmem& s, const WorkDev* __re
     int* err = W->err;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int ns = I.m + I.n, nt = g_ntiles(I);
-    const int nq = (nt - rank + G - 1) / G;            // tiles of this CTA: rank, rank + G, ...
+    const int nq = (nt - rank + G - 1) / G;            // tiles of this CTA: rank, rank + G, ... (at most kTileTable)
     const float* u = (const float*)I.u;
     float* d0 = (float*)I.d0;
     float* d1 = (float*)I.d1;
@@ -633,7 +632,7 @@ __device__ __forceinline__ void group_instance(GroupSmem& s, const WorkDev* __re
   for (int blk = 0; blk < blocks; ++blk) {
     const bool dz = __ldcg(&I.ctl->dzero) != 0;
     if (tid < K) s.p[tid] = make_p32(__ldcg(&I.ctl->sigma), __ldcg(&I.ctl->k) + tid, I.h, I.gadmm, I.relax);
-    if (tid >= 128 && tid - 128 < min(nq, kTileTable)) s.tile[tid - 128] = gtile(I, rank + (tid - 128) * G);
+    if (tid >= 128 && tid - 128 < nq) s.tile[tid - 128] = gtile(I, rank + (tid - 128) * G);
 #pragma unroll 1
     for (int q = tid; q < (int)(sizeof(CycleK) / 8); q += kThreads)
         reinterpret_cast<double*>(&s.C)[q] = __ldcg(reinterpret_cast<const double*>(I.cyc) + q);
@@ -654,7 +653,7 @@ __device__ __forceinline__ void group_instance(GroupSmem& s, const WorkDev* __re
         if (it > 0 && !group_wait(s, G, ++epoch, err)) return;
 #pragma unroll 1
         for (int q = 0; q < nq; ++q) {
-            const GTile& g = s.tile[q & (kTileTable - 1)];
+            const GTile& g = s.tile[q];
             const Half& hf = g.slab < I.n ? h1 : h2;
             if (q == 0) {
                 copy_tile(s, g, hf, u, din);                  // arrives under the sums and the second wait
@@ -693,8 +692,8 @@ __device__ __forceinline__ void group_instance(GroupSmem& s, const WorkDev* __re
             __syncthreads();
             auto between = [&]() {
                 const int qn = q + 1;
-                if (qn == nq || (qn & (kTileTable - 1)) == 0) return;     // the table's end: below
-                const GTile& gn = s.tile[qn & (kTileTable - 1)];
+                if (qn == nq) return;
+                const GTile& gn = s.tile[qn];
                 const Half& hn = gn.slab < I.n ? h1 : h2;
                 copy_tile(s, gn, hn, u, din);
                 if (tid < gn.nr + hn.S) pl = piece_load(I, gn, hn.S, tid, rs, cs);
@@ -703,19 +702,6 @@ __device__ __forceinline__ void group_instance(GroupSmem& s, const WorkDev* __re
                 group_sweep<true, PAD>(s, g, hf, s.p[it], u, din, dout, rs_out, cs_out, between);
             else
                 group_sweep<false, PAD>(s, g, hf, s.p[it], u, din, dout, rs_out, cs_out, between);
-            if (nq > kTileTable && (((q + 1) & (kTileTable - 1)) == 0 || q + 1 == nq)) {
-                // the next tiles' geometry (the first ones' after the last)
-                const int qn = q + 1 == nq ? 0 : q + 1;
-                __syncthreads();
-                if (tid < min(nq - qn, kTileTable)) s.tile[tid] = gtile(I, rank + (qn + tid) * G);
-                __syncthreads();
-                if (qn > 0) {
-                    const GTile& gn = s.tile[0];
-                    const Half& hn = gn.slab < I.n ? h1 : h2;
-                    copy_tile(s, gn, hn, u, din);
-                    if (tid < gn.nr + hn.S) pl = piece_load(I, gn, hn.S, tid, rs, cs);
-                }
-            }
         }
     }
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");

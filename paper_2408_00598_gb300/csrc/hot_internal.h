@@ -30,6 +30,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "hot_plan.h"
+
 namespace hot {
 
 constexpr int kThreads = 256;          // block size of the tile kernels
@@ -42,7 +44,6 @@ constexpr int kMaxTR = 128;            // FP32 tiles: TR * max(m, n) <= kRowSmem
 constexpr int kMaxTileElems = 16384;   // FP32 tiles: TR * (longer row pitch) <= this
 constexpr int kMaxGroupSide = 256;     // k_group32: longest side (one column per thread)
 constexpr int kMaxGroupSide64 = 128;   // k_group64: longest side
-constexpr int kMaxGroup = 512;         // k_group32: most CTAs of one instance
 constexpr int kPollLimit = 1 << 22;    // polls of a wait between CTAs before it gives up (a few seconds)
 
 enum : int {
