@@ -223,3 +223,33 @@ def test_pairs_of_a_batch_report_their_own_completion():
         for ib, tb in got:
             assert ia == ib or ta != tb, got
             assert ib < ia + 20 or ta < tb, got
+
+
+@pytest.mark.parametrize("precision,m,n,tiny", [("fp32", 256, 60, 150), ("fp64", 64, 64, 200)])
+def test_tiny_pairs_that_share_a_cta_equal_single_solves(precision, m, n, tiny):
+    """A CTA takes several instances one after the other (test_group_plan_host.py looks at this batch's plan), in one
+    launch with an instance that many CTAs take."""
+    from paper_2408_00598_gb300 import hot
+    pairs = [syn.make_pair("white", m, 1, n)] + [syn.make_pair("white", 2, q, 2 + q % 2) for q in range(tiny)]
+    with hot.Context(precision=precision) as ctx:
+        out = ctx.solve_batch([p[0] for p in pairs], [p[1] for p in pairs], tol=1e-6, max_iter=80)
+        # one kernel per four check blocks: the chain launches 30 or more per block
+        assert out[0]["iters"] == 80 and out[0]["kernel_launches"] <= 4
+        for (mu, nu), b in zip(pairs, out):
+            a = ctx.solve(mu, nu, tol=1e-6, max_iter=80)
+            ctx.release(a)
+            for key in ("ot_value", "dual_value", "rel_kkt", "sigma", "iters", "restarts", "status"):
+                assert a[key] == b[key], (key, a[key], b[key])
+
+
+def test_fp64_groups_of_a_batch_equal_single_solves():
+    """Groups of several sizes in one launch of k_group64."""
+    from paper_2408_00598_gb300 import hot
+    pairs = [syn.make_pair("white", 4 + (7 * q) % 23, q) for q in range(30)]
+    with hot.Context(precision="fp64") as ctx:
+        out = ctx.solve_batch([p[0] for p in pairs], [p[1] for p in pairs], tol=1e-6, max_iter=300)
+        assert max(r["kernel_launches"] for r in out) <= 300 // 40 + 3
+        for (mu, nu), b in zip(pairs, out):
+            a = ctx.solve(mu, nu, tol=1e-6, max_iter=300)
+            ctx.release(a)
+            assert (a["ot_value"], a["dual_value"], a["iters"]) == (b["ot_value"], b["dual_value"], b["iters"])
