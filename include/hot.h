@@ -299,7 +299,10 @@ HOT_API int hot_barycentric_map(const int32_t *src, const int32_t *dst, const do
  * rows; this times each candidate TR on a synthetic S x S instance on the
  * context's device (a fixed number of iterations, no early stop) and keeps
  * the fastest for every later instance of that size on this context,
- * including the serve loop.  With cfg.autotune_cache set, hot_create loads
+ * including the serve loop.  Sizes that single solves run in one kernel per
+ * block are timed there and in the chain of kernels, which batches of many
+ * run, and the smallest product of the two is kept (us_per_iter: of a single
+ * solve).  With cfg.autotune_cache set, hot_create loads
  * the entries for this device from that file and hot_autotune appends its
  * result (text, one entry per line: device name, fp32|fp64, S, TR,
  * microseconds per iteration; the last entry for a key wins).

@@ -3,8 +3,9 @@
 // the per-tile set-up and reductions fewer times; shorter ones spread a small
 // slab set over more CTAs.  Which wins depends on S and the device, so the
 // context can measure it: every candidate TR runs the same synthetic
-// instance for a fixed number of iterations (tol = 0, so no early stop) and
-// the fastest per-iteration time is kept for that (precision, S).  The table
+// instance for a fixed number of iterations (tol = 0, so no early stop), in the
+// chain of kernels and, where the instance is small enough, in the group kernel,
+// and one height is kept for that (precision, S) by pick_height.  The table
 // lives in the context and, when hot_config.autotune_cache names a file, in
 // that file (one line per entry: device, precision, S, TR, microseconds per
 // iteration), so later processes start tuned.  The table covers square S x S
@@ -118,26 +119,32 @@ int autotune(Ctx* ctx, int S, int* tr_out, double* us_out) {
     tune_pair(S, p);
     const std::vector<int> cand = tile_candidates(S, fp64);
     const long long iters = (long long)ctx->cfg.check_every * (S >= 512 ? 2 : 4);
-    int best = 0;
-    double best_us = 1e300;
+    std::vector<HeightTime> times;
     const int saved = ctx->tile_override;
     for (int tr : cand) {
         ctx->tile_override = tr;
         std::vector<PairHost> one(1, p);
-        hot_result r{};
-        int rc = run_solve(ctx, one, 0.0, ctx->cfg.check_every, false, &r);   // warm-up: graph, pools
-        if (rc == HOT_OK || rc == HOT_NOT_CONVERGED) rc = run_solve(ctx, one, 0.0, iters, false, &r);
-        if (rc != HOT_OK && rc != HOT_NOT_CONVERGED) {
-            ctx->tile_override = saved;
-            return rc;
+        HeightTime t{tr, 0.0, 0.0};
+        for (int chain = 0; chain < 2; ++chain) {
+            hot_result r{};
+            int rc = run_solve(ctx, one, 0.0, ctx->cfg.check_every, false, &r, nullptr, chain);   // warm-up: graph, pools
+            if (rc == HOT_OK || rc == HOT_NOT_CONVERGED) rc = run_solve(ctx, one, 0.0, iters, false, &r, nullptr, chain);
+            if (rc != HOT_OK && rc != HOT_NOT_CONVERGED) {
+                ctx->tile_override = saved;
+                return rc;
+            }
+            const double us = 1000.0 * r.solve_ms / (double)std::max(1LL, r.iters);
+            if (!chain) t.single_us = us;
+            t.chain_us = us;
+            if (ctx->batch->n_group == 0) break;       // it was the chain already
         }
-        const double us = 1000.0 * r.solve_ms / (double)std::max(1LL, r.iters);
-        if (us < best_us) {
-            best_us = us;
-            best = tr;
-        }
+        times.push_back(t);
     }
     ctx->tile_override = saved;
+    const int best = pick_height(times);
+    double best_us = 0.0;                      // as a single instance runs it
+    for (const HeightTime& t : times)
+        if (t.rows == best) best_us = t.single_us;
     {
         std::lock_guard<std::mutex> g(ctx->tune_mu);
         ctx->tuned[fp64][S] = {best, best_us};

@@ -747,7 +747,7 @@ void fill_result(const Inst* I, hot_result* r) {
 }
 
 int run_solve(Ctx* ctx, const std::vector<PairHost>& pairs, double tol, long long max_iter, bool keep,
-              hot_result* out, hot_kernel_times* kt) {
+              hot_result* out, hot_kernel_times* kt, bool chain) {
     const AtWork at_work(ctx->device);
     cudaStream_t st = ctx->stream;
     const int fp64 = ctx->cfg.precision == HOT_FP64 ? 1 : 0;
@@ -782,7 +782,7 @@ int run_solve(Ctx* ctx, const std::vector<PairHost>& pairs, double tol, long lon
     // timed launch are then those of the one instance).  It and the profiled
     // solve time the chain's kernels, so they run the chain at every size.
     const int timing = ctx->sweep_timing && insts.size() == 1 && !kt ? 1 : 0;
-    int rc = B.set_instances(insts, st, !timing && !kt);
+    int rc = B.set_instances(insts, st, !timing && !kt && !chain);
     if (rc == HOT_OK) rc = B.ensure_graph(timing);   // also fixes the launch dimensions
     if (rc != HOT_OK) {
         cleanup();

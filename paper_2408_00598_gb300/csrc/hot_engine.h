@@ -189,7 +189,7 @@ struct Ctx {
 };
 
 int run_solve(Ctx* ctx, const std::vector<PairHost>& pairs, double tol, long long max_iter, bool keep,
-              hot_result* out, hot_kernel_times* kt = nullptr);
+              hot_result* out, hot_kernel_times* kt = nullptr, bool chain = false);   // chain: no group kernels
 void fill_result(const Inst* I, hot_result* r);
 int recover_plan(Ctx* ctx, Inst* I, int32_t* src, int32_t* dst, double* mass, int space, size_t cap, size_t* nnz,
                  double* marg_l1, cudaStream_t st);

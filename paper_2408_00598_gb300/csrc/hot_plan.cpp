@@ -61,4 +61,15 @@ GroupPlan plan_groups(const std::vector<int>& inst, const std::vector<int>& tile
     return P;
 }
 
+int pick_height(const std::vector<HeightTime>& t) {
+    int best = 0;
+    double least = 0.0;
+    for (const HeightTime& h : t)
+        if (!best || h.single_us * h.chain_us < least) {
+            best = h.rows;
+            least = h.single_us * h.chain_us;
+        }
+    return best;
+}
+
 }  // namespace hot

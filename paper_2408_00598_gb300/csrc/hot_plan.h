@@ -22,4 +22,15 @@ struct GroupPlan {
 GroupPlan plan_groups(const std::vector<int>& inst, const std::vector<int>& tiles, const std::vector<int>& elems, int grid,
                       int fp64);
 
+// One tile height the autotuner measured: microseconds per iteration of a single
+// instance, as single solves run it (group kernel or chain) and in the chain.
+struct HeightTime {
+    int rows;
+    double single_us, chain_us;
+};
+// The height to keep.  It serves both forms (an instance's results depend on the
+// height, not on the form): single small instances run the group kernels, batches
+// and the serve loop of many of them the chain, so the smallest product wins.
+int pick_height(const std::vector<HeightTime>& t);
+
 }  // namespace hot

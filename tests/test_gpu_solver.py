@@ -388,6 +388,23 @@ def test_results_do_not_depend_on_the_sweeps_tile_order(lib, ctx32):
         assert rb["ot_value"] == rs["ot_value"] and rb["dual_value"] == rs["dual_value"]
 
 
+def test_results_do_not_depend_on_the_tile_order_of_the_chain(lib, ctx32):
+    """The same for a pair that the chain of kernels runs both times (a side above 256): a 300 x 40 pair alone (its
+    state fits in L2: one order) against the same pair batched with a 256 x 256 one (alternating order)."""
+    thin = syn.make_pair("gauss", 300, 7, 40)
+    big = syn.make_pair("white", 256, 1000)
+    alone = []
+    for a, b in (thin, big):
+        r = ctx32.solve(a, b, tol=1e-6, max_iter=300)
+        ctx32.release(r)
+        assert r["kernel_launches"] >= 10 * r["blocks"]          # the chain, not one kernel for several blocks
+        alone.append(r)
+    out = ctx32.solve_batch([thin[0], big[0]], [thin[1], big[1]], tol=1e-6, max_iter=300)
+    for rb, rs in zip(out, alone):
+        for key in ("ot_value", "dual_value", "rel_kkt", "sigma", "iters", "restarts", "status"):
+            assert rb[key] == rs[key], (key, rb[key], rs[key])
+
+
 # ------------------------------------------------------- live sweep timing --
 
 def test_live_sweep_timing_leaves_the_solve_unchanged(lib):

@@ -25,6 +25,11 @@ extern "C" int plan(int n, const int* tiles, const int* elems, int grid, int fp6
     *most = p.most;
     return p.used;
 }
+extern "C" int pick(int n, const int* rows, const double* single, const double* chain) {
+    std::vector<HeightTime> t(n);
+    for (int q = 0; q < n; ++q) t[q] = HeightTime{rows[q], single[q], chain[q]};
+    return pick_height(t);
+}
 """
 
 
@@ -109,3 +114,19 @@ def test_tiny_pairs_beside_a_larger_one_share_ctas(rules, fp64, m, n, tiny):
     ctas, _ = _check(rules, [t for t, _ in work], [e for _, e in work], 304, fp64)
     assert sum(t for t, _ in work) <= 4 * 304
     assert sum(1 for e in ctas if len(e) >= 2) >= 10
+
+
+@pytest.mark.parametrize("times,want", [
+    ([(64, 13.2, 26.1), (32, 12.7, 25.6), (16, 16.5, 28.0)], 32),
+    # the chain loses more at the height that the group kernel likes best
+    ([(48, 12.0, 25.0), (24, 11.8, 30.0)], 48),
+    ([(128, 20.0, 35.0), (64, 22.7, 33.8)], 128),
+    # heights at which a single solve runs the chain too
+    ([(64, 111.5, 111.5), (32, 126.5, 126.5)], 64),
+    ([(96, 18.3, 30.3), (48, 22.0, 30.2), (12, 41.5, 41.5)], 96),
+    ([(16, 12.6, 25.2)], 16),
+])
+def test_tile_height_serves_both_forms(rules, times, want):
+    n = len(times)
+    col = lambda k, t: (t * n)(*[r[k] for r in times])
+    assert rules.pick(n, col(0, ctypes.c_int), col(1, ctypes.c_double), col(2, ctypes.c_double)) == want
