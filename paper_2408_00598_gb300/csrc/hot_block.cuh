@@ -21,7 +21,10 @@ struct Sweep64Smem {
 };
 
 // a > b for doubles, on the integer pipe (FP64 comparisons run at a 64th of the
-// FP32 rate, like all FP64 instructions here); a NaN compares as larger.
+// FP32 rate, like all FP64 instructions here).  A NaN sorts by its sign bit, beyond
+// the infinities: which of z-bar - g's two values stays is then arbitrary, but a
+// NaN among the pieces or the state is also in x-bar = u + d + sigma D, whose
+// objective the check tests (HOT_NUMERIC).
 __device__ __forceinline__ bool gt64(double a, double b) {
     long long x = __double_as_longlong(a), y = __double_as_longlong(b);
     x ^= (x >> 63) & 0x7fffffffffffffffLL;

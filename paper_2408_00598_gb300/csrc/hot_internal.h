@@ -242,8 +242,6 @@ struct alignas(128) SweepTile {
     int row;          // g_row: first row entry of the slab
     int tile;         // g_tile: index of the tile within its instance
     int colp;         // g_colp: first column-partial entry of (slab, band)
-    int dz;           // set by the sweep: the delta read is zero (first iteration after an FP32 restart): no loads
-    int pad;
     long long elem;   // g_elem: first flow variable of the slab
     const HotCtl* ctl;
     const float *u, *d0, *d1;     // of the tile's first row

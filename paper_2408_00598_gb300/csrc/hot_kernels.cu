@@ -459,7 +459,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_sweep64(const WorkDev* __restri
 // drained between tiles, so the next tile's loads are in flight while the
 // current tile's row and column sums are reduced.  The rows' alpha pieces
 // travel in the group of each tile's first pass into a ring of their own, and
-// thread 0 leaves each tile's descriptor in a third ring for the compute side.
+// the first threads leave each tile's descriptor (128 bytes) in a third ring for the
+// compute side.
 //
 // The scaled cost is separable, h (x_r - x_c)^2 = h x_r^2 + h x_c^2 - 2 h x_r x_c
 // (x the bin coordinates of the slab's half, integers in FP32 mode), so the
@@ -622,7 +623,7 @@ __global__ void __launch_bounds__(kThreads, CHECK ? 2 : 3) k_sweep32(const WorkD
     int n = 0;                                   // global index of the next pass to compute
     for (int ck = 0;; ++ck) {
         // the tile's alpha pieces and its descriptor: group n (its first pass)
-        // and thread 0's store, both complete before this barrier
+        // and the first threads' store, both complete before this barrier
         cp_async_wait<kStages - 2>();
         __syncthreads();
         // the issue side has started every tile this CTA still has (it runs ahead)
@@ -722,7 +723,7 @@ __global__ void __launch_bounds__(kThreads, CHECK ? 2 : 3) k_sweep32(const WorkD
                 *reinterpret_cast<float4*>(&s_xcol[ro * Sp + c0]) = make_float4(xacc[0], xacc[1], xacc[2], xacc[3]);
         }
         __syncthreads();
-        // the next tile's column values (thread 0 stored its descriptor while
+        // the next tile's column values (the first threads stored its descriptor while
         // issuing its first pass, before this barrier); the loads complete
         // under the reductions below
         have = !(c.it >= ntiles && ck + 1 >= c.ik);
