@@ -34,6 +34,7 @@
 #include "hot_block.cuh"
 
 #include <algorithm>
+#include <atomic>
 #include <cstdint>
 #include <type_traits>
 
@@ -1042,13 +1043,13 @@ LaunchDims make_launch_dims(int device, int fp64) {
 }
 
 int sweep_grid(int fp64) {
-    static int cache[2][64];                 // per precision and device ordinal; 0 = not yet queried
+    static std::atomic<int> cache[2][64];    // per precision and device ordinal; 0 = not yet queried
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) return 0;
-    int& c = cache[fp64 ? 1 : 0][dev];
-    if (c == 0) c = make_launch_dims(dev, fp64).grid_tile;
-    return c;
+    std::atomic<int>& c = cache[fp64 ? 1 : 0][dev];
+    if (c.load() == 0) c.store(make_launch_dims(dev, fp64).grid_tile);
+    return c.load();
 }
 
 void launch_tile_table(const WorkDev* w, int ntiles, cudaStream_t st) {
