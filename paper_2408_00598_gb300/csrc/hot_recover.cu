@@ -565,13 +565,16 @@ __global__ void __launch_bounds__(256) k_export(const T* __restrict__ x, int m, 
 int export_flows(Inst* I, double* x, int space, cudaStream_t st) {
     const int m = I->m, n = I->n;
     const size_t V = (size_t)m * n * (m + n);
+    int dev = 0, sms = 0;
+    HOT_CK(cudaGetDevice(&dev));
+    HOT_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     double* dst = x;
     double* tmp = nullptr;
     if (space == HOT_SPACE_HOST) {
         HOT_CK(cudaMallocAsync(&tmp, V * 8, st));
         dst = tmp;
     }
-    const int grid = 152 * 8;
+    const int grid = sms * 8;
     if (I->fp64) k_export<double><<<grid, 256, 0, st>>>((const double*)I->desc.xr, m, n, dst);
     else k_export<float><<<grid, 256, 0, st>>>((const float*)I->desc.xr, m, n, dst);
     HOT_CK(cudaGetLastError());
