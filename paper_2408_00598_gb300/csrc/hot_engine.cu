@@ -503,27 +503,31 @@ int Batch::reserve(int n) {
     if (n <= cap && d_work) return HOT_OK;
     int ncap = std::max(n, std::max(16, cap * 2));
     drop_graphs();   // the graphs captured the old table pointers
-    cudaFree(d_work);
-    cudaFree(d_inst);
-    cudaFree(d_pre);
-    cudaFree(d_running);
-    cudaFree(d_st);
-    cudaFree(d_gstart);
-    cudaFree(d_gent);
-    cudaFreeHost(h_gstart);
-    cudaFreeHost(h_gent);
-    cudaFreeHost(h_work);
-    cudaFreeHost(h_inst);
-    cudaFreeHost(h_pre);
-    cudaFreeHost(h_running);
-    cudaFreeHost(h_st);
-    cudaFreeHost(h_stb);
-    h_stb = nullptr;
-    d_work = nullptr;
-    d_gstart = nullptr;
-    d_gent = nullptr;
-    h_gstart = nullptr;
-    h_gent = nullptr;
+    // an allocation below may fail: nothing of the old tables is left to be used or freed again
+    cap = 0;
+    auto drop = [](auto*& p) {
+        cudaFree(p);
+        p = nullptr;
+    };
+    auto drop_host = [](auto*& p) {
+        cudaFreeHost(p);
+        p = nullptr;
+    };
+    drop(d_work);
+    drop(d_inst);
+    drop(d_pre);
+    drop(d_running);
+    drop(d_st);
+    drop(d_gstart);
+    drop(d_gent);
+    drop_host(h_gstart);
+    drop_host(h_gent);
+    drop_host(h_work);
+    drop_host(h_inst);
+    drop_host(h_pre);
+    drop_host(h_running);
+    drop_host(h_st);
+    drop_host(h_stb);
     ggrid = group_grid(fp64);
     HOT_CK(cudaMalloc(&d_gstart, sizeof(int) * (ggrid + 1)));
     HOT_CK(cudaMalloc(&d_gent, sizeof(int4) * (ggrid + ncap)));
