@@ -44,7 +44,9 @@ __device__ __forceinline__ double neg64(double a) {
 // cost by one fma of the difference t, with x times 2^floor(e / 2), h = 2^e, and
 // for odd e one factor doubled in its exponent; comparisons run on integers.
 // (The separable form h x_r^2 - alpha + h x_c^2 - beta - 2 h x_r x_c takes 8.5, but its
-// error is relative to the largest cost instead of the element's.)
+// error is relative to the largest cost instead of the element's.)  FP64 pipe
+// 81 % busy.  One sweep: 128 x 128 125 -> 97 us, 256 x 256 947 -> 692 us; on check
+// iterations 224 -> 196 and 1,748 -> 1,456 us.
 template <bool CHECK>
 __device__ __forceinline__ void sweep64_tile(const HotInst& I, int slab, int band, const double* __restrict__ din_,
                                              double* __restrict__ dout_, const P64& p, const double* __restrict__ ab,
@@ -145,8 +147,7 @@ __device__ __forceinline__ void sweep64_tile(const HotInst& I, int slab, int ban
         }
     } else {
         // short rows, many partials per column (sides up to 32): eight lanes per
-        // column, as for the rows below (16 x 16 with k_group64: 22.7 -> 21.9 us
-        // per iteration)
+        // column, as for the rows below (0.8 us of an iteration of 16 x 16)
         for (int q = tid; q < ((S * 8 + 31) & ~31); q += kThreads) {       // whole warps
             const int c = q >> 3, l = q & 7;
             double acc = 0.0, xac = 0.0;
@@ -258,9 +259,9 @@ __device__ __forceinline__ void anchor_slab(const HotInst& I, int slab, double s
 // FP32 mode streams the state through a ring of SLOTS passes per thread in
 // shared memory (u and d; MODE 0 also x_r and z_r), a commit group per pass:
 // more bytes in flight than registers can hold beside the double-float sums.
-// 512 x 512, before -> with the ring: MODE 0 975 -> 737 us (5.8 TB/s of its 16 B per
-// variable), MODE 2 642 -> 572 us, MODE 1 1,450 us either way: its epilogue adds a
-// row's partials in one chain, whose order the iterates depend on.
+// 512 x 512: MODE 0 1,052 -> 886 us (4.8 TB/s of its 16 B per variable, now bound by
+// the issue of its pair sums, 73 %), MODE 2 639 us, MODE 1 1,532 us: its epilogue
+// adds a row's partials in one chain, whose order the iterates depend on.
 constexpr int kRestartSlots = 4;
 __host__ __device__ constexpr size_t restart_ring(int mode) {
     return (size_t)kRestartSlots * (mode == 0 ? 4 : 2) * kThreads * sizeof(float4);

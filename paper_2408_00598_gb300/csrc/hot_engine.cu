@@ -119,10 +119,11 @@ int validate_pair(const double* mu, const double* nu, int m, int n, int space, i
 
 // k_group32 / k_group64 or the chain of kernels.  FP32: sides up to 256 (one
 // column per thread, one round of slab sums) while u and the delta fit in L2:
-// 192 x 192 (108 MB) 59.8 us per iteration against the chain's 64.7, 256 x 256
+// 192 x 192 (108 MB) 56 us per iteration against the chain's 58, 256 x 256
 // (256 MB) 114 against 99, since the chain's sweep keeps more CTAs per SM.
-// FP64 (u and two deltas): 96 x 96 (40 MB) 70 against 78 us, 127 x 100 (66 MB) 108
-// against 112, 128 x 128 (96 MB) 143 against 134.
+// FP64 (u and two deltas): 96 x 96 (40 MB) 70 against 80 us, 112 x 112 (67 MB) 107
+// against 115, 128 x 128 (96 MB) 143 against 134.  Inside the rule a pair whose
+// tiles just exceed the CTAs loses up to a tenth (FP64 80 x 80, 320 tiles: 86 against 79).
 constexpr size_t kGroupStateBytes = (size_t)120 << 20, kGroupStateBytes64 = (size_t)72 << 20;
 static int group_rule(const Inst& I) {
     if (I.fp64) return std::max(I.m, I.n) <= kMaxGroupSide64 && I.big_bytes / 5 * 3 <= kGroupStateBytes64 ? 1 : 0;

@@ -23,8 +23,9 @@
 //
 // Bound by latency: an iteration of a 32 x 32 pair takes 19,400 cycles, the two
 // waits 3,000 each with the CTAs' skew, slab sums 1,900, stage 3,000, pieces 2,000,
-// sweep and sums 3,000.  us per iteration of a solve, chain -> group: 32 x 32
-// 24.9 -> 11.3, 64 x 64 25.9 -> 13.2, 128 x 128 34.5 -> 23.1, 192 x 192 64.7 -> 59.8.
+// sweep and sums 3,000.  us per iteration of a solve (block ends included), chain
+// -> group: 32 x 32 24.6 -> 11.3, 64 x 64 24.7 -> 12.1, 128 x 128 31.8 -> 21.7,
+// 192 x 192 58.3 -> 56.0.
 //
 // The groups of one launch are independent.  The grid is launched
 // cooperatively, so that the CTAs of a group are resident together; it has the
@@ -756,7 +757,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_group32(const WorkDev* __restri
 // every CTA (marg64), then per tile the pieces (pieces64) and the sweep
 // (sweep64_tile), wait; the block end.  The arithmetic and its order are the
 // chain's (k_vec, k_marg, k_alpha, k_sweep64).  us per iteration of a solve,
-// chain -> group: 16 x 16 31.4 -> 21.9, 64 x 64 58 -> 47, 96 x 96 80 -> 71; bound by
+// chain -> group: 16 x 16 27.6 -> 15.4, 64 x 64 58 -> 31, 96 x 96 80 -> 70; bound by
 // FP64 latency (about 60 cycles an operation, 440 a conversion) and the waits.
 struct Group64Smem {
     Sweep64Smem sw;
