@@ -204,7 +204,7 @@ int inst_create(const PairHost& p, int fp64, const hot_config& cfg, double tol, 
     const size_t o_stg2 = take(4 * (size_t)L * F2);
     const size_t o_rsb = fp64 ? take(2 * MN * 8) : 0;
     const size_t o_csb = fp64 ? take(CP * 8) : 0;
-    const size_t o_rs2b = take(2 * MN * F2);
+    const size_t o_rs2b = fp64 ? 0 : take(2 * MN * F2);
     const size_t o_cs32b = fp64 ? 0 : take(CP * 4);
     const size_t o_tp = fp64 ? 0 : take((size_t)NS * sizeof(float4));
     const size_t o_gcount = take(2 * sizeof(unsigned int));

@@ -57,17 +57,19 @@ static int serve_tile_rows(Ctx* ctx, int m, int n, int fp64) {
     return t ? t : tile_rows(m, n, fp64, sweep_grid(fp64));
 }
 
-// Device bytes of one instance (an upper bound of inst_create's layout).
+// Device bytes of one instance (an upper bound of inst_create's layout), for admission;
+// an admitted request is then accounted with what was allocated.
 static size_t inst_bytes_estimate(Ctx* ctx, int m, int n, int fp64) {
-    const size_t MN = (size_t)m * n;
-    const size_t V = MN * (size_t)(m + n);
+    const size_t MN = (size_t)m * n, L = std::max(m, n);
+    const size_t V = MN * (size_t)(((m + 3) & ~3) + ((n + 3) & ~3));       // rows at their pitch
     const size_t big = 5 * (V * (fp64 ? 8 : 4) + 256);
     const int tr = serve_tile_rows(ctx, m, n, fp64);
-    const size_t CP = (size_t)n * ((m + tr - 1) / tr) * m + (size_t)m * ((n + tr - 1) / tr) * n;
-    // pieces 3 x 32 MN, slab-row sums 5 x 16 MN, marginals 16 MN, column partials 28 CP
-    size_t small = MN * (96 + 80 + 16) + CP * 28 + 1024 * 64;
-    if (fp64) small += MN * 16 + CP * 8;                                              // group buffers
-    if (!fp64) small += MN * 208 + CP * 4 + (size_t)(m + n) * 16;   // double-float arrays and group buffers of FP32 mode
+    const size_t nb1 = (m + tr - 1) / tr, nb2 = (n + tr - 1) / tr;
+    const size_t CP = n * nb1 * m + m * nb2 * n, tiles = n * nb1 + m * nb2;
+    // pieces 96 (FP32 mode 96 more), slab-row sums 80, pairs 80, marginals 32, the group kernels' second
+    // row sums 16; column partials 36; tile sums 64; the vectors of Prop. 3 and their partials
+    const size_t small = MN * (fp64 ? 304 : 400) + CP * 36 + tiles * 65 + L * 8 * (17 + (m + n) / 64) + 4 * (m + n) * 16 +
+                         MN / 8 + 64 * 1024;
     return big + small;
 }
 
@@ -155,6 +157,9 @@ static void serve_loop(Ctx* ctx) {
                 finish_req(ctx, s, r, rc);
                 continue;
             }
+            s->in_use -= std::min(s->in_use, r->bytes);
+            r->bytes = I->big_bytes + I->small_bytes;
+            s->in_use += r->bytes;
             r->inst = I;
             r->state = 1;
             s->active.push_back(r);

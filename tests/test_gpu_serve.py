@@ -98,3 +98,26 @@ def test_invalid_request(lib):
             srv.submit(a * 2, b)
         with pytest.raises(lib.HotError):
             srv.submit(a, b, max_iter=0)
+
+
+@pytest.mark.parametrize("precision,m,n", [("fp32", 65, 65), ("fp64", 65, 65), ("fp64", 8, 8), ("fp32", 3, 2)])
+def test_bytes_in_use_count_the_padded_state_and_every_array(lib, precision, m, n):
+    """device_bytes_in_use of a running request: five state arrays, each row at its pitch, and the arrays of 304 (FP64)
+    or 400 (FP32) bytes per bin pair (i, j)."""
+    mu, nu = syn.make_pair("white", m, 1, n)
+    es, per = (8, 304) if precision == "fp64" else (4, 400)
+    least = 5 * es * m * n * (((m + 3) & ~3) + ((n + 3) & ~3)) + per * m * n
+    with lib.Context(precision=precision) as ctx:
+        t = ctx.submit(mu, nu, tol=0.0, max_iter=10 ** 9)
+        seen = 0
+        for _ in range(2000):
+            s = ctx.serve_stats()
+            if s["running"] == 1:
+                seen = s["device_bytes_in_use"]
+                break
+            time.sleep(0.001)
+        ctx.cancel(t)
+        assert ctx.wait(t, timeout_ms=60000)[0] == lib.HOT_ECANCELLED
+        left = ctx.serve_stats()["device_bytes_in_use"]
+    assert least <= seen <= 2 * least + 10 ** 5
+    assert left == 0
